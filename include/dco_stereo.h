@@ -41,12 +41,9 @@
  *     handle stays usable, and its next calls allocate what they need.
  *   - Device-side failures do not trap: they set the handle's status word,
  *     read with dco_stereo_sync_status() or dco_stereo_stream_status().  The
- *     vertical pass sets bit 0 when a TMA tile copy does not complete within
- *     its bounded mbarrier wait (reported as DCO_ETIMEOUT; the block stops
- *     issuing copies and returns), and so does the cost pass when its
- *     staging bulk copies do not; bit 1 when the vertical pass's shared
- *     memory is not 128-byte aligned for the copies (DCO_EDEVICE); the
- *     pass's outputs are then not valid.
+ *     cost pass sets bit 0 when its staging bulk copies do not complete
+ *     within their bounded mbarrier wait (reported as DCO_ETIMEOUT; the block
+ *     returns); the pass's outputs are then not valid.
  */
 #ifndef DCO_STEREO_H
 #define DCO_STEREO_H
@@ -141,8 +138,8 @@ void dco_stereo_destroy(dco_stereo *h);
 /*
  * Device bytes of workspace one match of a W x H pair with D disparities
  * needs under params p (0 if the arguments are invalid).  Per pixel: two
- * 16-byte census/colour records, two arm words, the running best cost and
- * disparity of both views; per pixel and per disparity of one pass: the
+ * 16-byte census/colour records, two arm words, the best cost and
+ * disparity of both views so far; per pixel and per disparity of one pass: the
  * two horizontal-aggregate slices (4 bytes each).  Never the full
  * W x H x D cost volume.
  */
@@ -165,10 +162,9 @@ dco_status dco_stereo_reserve(dco_stereo *h, int W, int H, int D, const dco_para
  * pass (rows for agg_order 0, columns for 1) splits each line into blocks
  * of p->h_chunk outputs (0: whole lines up to 1024 positions, else 512;
  * otherwise 32 <= h_chunk, capped at 1024 - 2 arm_l1 below the line); the second
- * pass splits each line into balanced blocks of at most p->v_chunk outputs
- * (0: whole lines up to 512 positions, else blocks of at most 432; otherwise
- * 32 <= v_chunk, capped at 512 - 2 arm_l1).  Each block reads arm_l1
- * positions of halo on both sides.
+ * pass walks each line in balanced runs of at most p->v_chunk outputs
+ * (0: dealt out evenly to the device; otherwise 32 <= v_chunk).  Each block
+ * reads arm_l1 positions of halo on both sides.
  * p = NULL uses the defaults.
  */
 dco_status dco_stereo_match(dco_stereo *h, const uint8_t *left, const uint8_t *right,
@@ -359,8 +355,8 @@ size_t dco_stereo_workspace_allocated(dco_stereo *h);
 
 /*
  * Waits for all work of the handle's device, then reads and clears the
- * device status word.  DCO_OK; DCO_ETIMEOUT if a copy of the cost or the
- * vertical pass did not complete within its bounded wait; DCO_EDEVICE if a kernel
+ * device status word.  DCO_OK; DCO_ETIMEOUT if a copy of the cost pass did
+ * not complete within its bounded wait; DCO_EDEVICE if a kernel
  * reported another failed internal check since the last read.
  */
 dco_status dco_stereo_sync_status(dco_stereo *h);
@@ -375,10 +371,10 @@ dco_status dco_stereo_stream_status(dco_stereo *h, dco_stream stream);
 
 /*
  * Failure tests (not for normal use).  DCO_TEST_LOSE_TILE_COPIES: the
- * cost pass's staging and the vertical pass's tiles arm their mbarriers but
- * issue no copy, and wait only a few polls, so every wait runs out with
- * nothing in flight; the kernels set bit 0 of the status word and return,
- * and the stream status reads DCO_ETIMEOUT.  DCO_TEST_LOSE_GRID_ARRIVAL: in the one-launch
+ * cost pass's blocks arm their staging mbarriers but issue no copy, and wait
+ * only a few polls, so every wait runs out with nothing in flight; the kernel
+ * sets bit 0 of the status word and returns, and the stream status reads
+ * DCO_ETIMEOUT.  DCO_TEST_LOSE_GRID_ARRIVAL: in the one-launch
  * densification solve, block 0 never arrives at the first grid barrier and
  * every barrier waits only a few polls, so all blocks give up and return;
  * dco_stereo_densify returns DCO_ETIMEOUT.  0 restores normal operation.

@@ -13,10 +13,10 @@
 //     k_hagg  Eq. 1 cost in fixed point for every (column, disparity) of a
 //             row, prefixes over 16-column segments in shared memory, and
 //             the horizontal segment sum of every pixel -> sh slice
-//     k_vagg  column prefix of the sh slice (TMA tiles), the vertical sum
-//             over the up/down arms (Eq. 2) and the running minimum over
-//             the disparities (Eq. 3), merged with the previous passes
-//   k_lr     left-right consistency -> disparity map
+//     k_vagg  column prefix of the sh slice, the vertical sum over the
+//             up/down arms (Eq. 2) and the minimum over the disparities
+//             (Eq. 3), merged into one key per pixel
+//   k_end    keys -> disparities; left-right consistency -> disparity map
 // Every kernel is launched with programmatic stream serialization and waits
 // for its predecessors before its first global access.
 // Lanes of a warp hold consecutive disparities of one pixel (pairs of them
@@ -36,6 +36,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 namespace dco {
@@ -498,8 +499,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 constexpr int kWaitLimit = 1 << 22;   // mbarrier polls before a copy is declared lost
 constexpr int kTestWaitLimit = 64;    // the same, under the lost-copy failure test
-constexpr int kStatusCopyTimeout = 1; // status word: a copy (k_hagg staging, k_vagg tiles) did not complete
-constexpr int kStatusAlign = 2;       // status word: shared memory not aligned for the tile copies
+constexpr int kStatusCopyTimeout = 1; // status word: k_hagg's staging copies did not complete
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
@@ -768,6 +768,9 @@ __device__ __forceinline__ void hagg_body(const HArgs &a, int bx, int by, int bz
     const uint2 *cenE = scen + hoff_s[0], *cenO = scen + L.hhc + hoff_s[1];
     const uint32_t *colE = scol + hoff_s[2], *colO = scol + L.hhk + hoff_s[3];
     const uchar4 *sarm0 = sarm + (ga - gas);   // arm of output column xs
+    unsigned long long *init = view ? a.init[1] : a.init[0];
+    if (init && g == 0)   // the keys the V pass minimises into
+        for (int i = threadIdx.x; i < xe - xs; i += blockDim.x) init[ga + i] = ~0ull;
 
     // ---- A: costs and local prefixes of this half-warp's segment
     const int half = lane >> 4, hl = lane & 15;
@@ -844,6 +847,9 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
     const uint4 *rref = view ? a.rec[1] : a.rec[0];   // padded rows, pitch rpitch
     const uint4 *roth = view ? a.rec[0] : a.rec[1];
     const uchar4 *aref = view ? a.arms[1] : a.arms[0];
+    unsigned long long *init = view ? a.init[1] : a.init[0];
+    if (init && g == 0)   // the keys the second pass minimises into
+        for (int i = threadIdx.x; i < ye - ys; i += blockDim.x) init[(size_t)(ys + i) * W + x] = ~0ull;
 
     for (int i = threadIdx.x; i < kTabBytes / 16; i += blockDim.x)
         cp_async16(smem_raw + 16 * i, reinterpret_cast<const uint8_t *>(a.tables) + 16 * i);
@@ -980,7 +986,17 @@ __device__ __forceinline__ void hvote_body(const HVArgs &a, int bx, int by, int 
     if (threadIdx.x < 32) P[(int)threadIdx.x - 32] = 0;
     const int16_t *drow = a.disp + (size_t)y * W;
     const uchar4 *aref = a.arms + (size_t)y * W;
-    for (int i = threadIdx.x; i < len; i += blockDim.x) sd[i] = drow[xa + i];
+    if (a.keys) {   // a later round: the previous round's winners where the first map was valid
+        const unsigned long long *krow = a.keys + (size_t)y * W;
+        for (int i = threadIdx.x; i < len; i += blockDim.x) {
+            const int v = drow[xa + i];
+            sd[i] = v >= a.dmin && v < a.D ? (int16_t)(krow[xa + i] & 0xffffu) : (int16_t)-1;
+        }
+    } else {
+        for (int i = threadIdx.x; i < len; i += blockDim.x) sd[i] = drow[xa + i];
+    }
+    if (a.init && g == 0)   // the keys the V pass minimises into
+        for (int i = threadIdx.x; i < xe - xs; i += blockDim.x) a.init[(size_t)y * W + xs + i] = ~0ull;
     for (int i = threadIdx.x; i < xe - xs; i += blockDim.x) sarm[i] = aref[xs + i];
     __syncthreads();
 
@@ -1007,233 +1023,293 @@ __device__ __forceinline__ void hvote_body(const HVArgs &a, int bx, int by, int 
 }
 
 // ------------------------------------------------------------------ k_vagg
-// Block = one column x of one reference view, a chunk of output rows.  The
-// prefix range [ya, yb) is split into warp segments of 32 rows.  For each
-// group of 32 disparities of the pass:
-//   0. every warp moves its 32 slice rows (128 bytes each: the group's
-//      disparities of one pixel) into Q[y - ya] with one TMA tile copy
-//      (completing on the warp's mbarrier);
-//   A. lane = disparity: the warp's 32 tile rows into registers, the
-//      segment sum exchanged with the other warps, then the column prefix
-//      (with its segment offset) written back in place (the rows of a
-//      partial tile past the range are summed after the range's last row,
-//      and the last warp's total is read by no other warp);
-//   C. lane = output row: V(d) = Q(y + dn, d) - Q(y - up - 1, d) for the 32
-//      disparities (Eq. 2: the sum over the vertical arm of the horizontal
-//      sums; N does not depend on d, so the WTA compares V), running minimum
-//      with the smallest d on ties (Eq. 3) in registers across groups; four
-//      disparities per 16-byte shared load.
-// Finally the running best is merged with earlier passes and written.
-// Q rows are 36 words (144 bytes: the tile box is 32 disparities plus 4
-// zero-filled words, a multiple of 16 bytes); in phase C the 16-byte loads
-// of 32 rows spread over the 8 bank quads.
-constexpr int kQS = 36;   // Q row stride in words
-constexpr int kVSeg = 32; // rows per warp
-constexpr int kQ0 = 64;   // Q[0] at word 64 (256 bytes): every warp's tile starts on a 128-byte boundary
-constexpr uint32_t kVTileBytes = kVSeg * kQS * 4;
-
-// words before the mbarriers: Q[-1] (zeros, at kQ0 - kQS) and Q [nw*32 rows:
-// every warp's tile is 32 rows], T [nw][32], NQ [len], NT [nw]
-__host__ __device__ inline size_t vagg_bar_word(int len, int nw)
-{
-    return ((size_t)kQ0 + (size_t)nw * kVSeg * kQS + nw * 32 + len + nw + 1) / 2 * 2;
-}
-__host__ __device__ inline size_t vagg_smem_words(int len, int nw) { return vagg_bar_word(len, nw) + 2 * nw; }
-
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *tm, int c0, int c1, int c2, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-                 " [%0], [%1, {%2, %3, %4}], [%5];\n" ::"r"(dst),
-                 "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
-                 : "memory");
-}
-// TMA tile copy of the box at coordinates (c0, c1, c2, c3) of map `tm` to
-// shared address `dst` (128-byte aligned), completing on mbarrier `bar`
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *tm, int c0, int c1, int c2, int c3,
-                                            uint32_t bar)
-{
-    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-                 " [%0], [%1, {%2, %3, %4, %5}], [%6];\n" ::"r"(dst),
-                 "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-                 : "memory");
-}
-
-// kMax: the WTA takes the largest V (the vote counts of Eq. 4) instead of the
-// smallest: V is complemented, so the strict < keeps the smallest d on ties
-// and the key merge across passes is unchanged
+// Second 1-D sum (Eq. 2) and winner-take-all (Eq. 3).  A block of four warps
+// walks down strips of four neighbouring columns for one group of 32
+// disparities of one view, 32 slice rows per step, eight per warp; lane =
+// (column, four consecutive disparities), so a row of the strip is one
+// 16-byte load per lane (four 128-byte slice lines), issued a step ahead.
+// A step:
+//   - the totals of the warps' rows and the prefix before the step give each
+//     warp its start; it writes the column prefix Q of its rows to a ring in
+//     shared memory that holds the last 2 L1 + 1 rows besides the step's;
+//   - V(d) = Q(y + down, d) - Q(y - up - 1, d) of the output rows that the
+//     entered rows complete: two 16-byte reads per lane, on the same eight
+//     bank quads whatever the arms are;
+//   - the minimum over a lane's four disparities goes through a small tile to
+//     the lane that owns the row, which finds the minimum over the group
+//     (smallest d on ties) and minimises (V << 32 | d) into the pixel's key.
+// A run of rows starts up to 2 L1 + 1 rows before its first output, so strips
+// are split only where whole ones do not fill the SMs evenly (vagg_geom).
+// Bound by the shared-memory and L1 data path (70 % of its cycles, DRAM at
+// 45 %): per 32 evaluations one wavefront each for the load and the prefix's
+// store and two for the window.  Four blocks (62 KB, L1 = 34) per SM.
+// Against one block per column that held its whole column's prefix, lane =
+// disparity: 1920x1080, D = 256, eight passes 2117 -> 998 us, one pass 1073
+// -> 882 us; 640x480, D = 64, two passes 66.3 -> 50.5 us; the smallest images
+// pay for the longer chain (320x240, D = 32: 12.4 -> 14.2 us).  Walks of one
+// warp per strip with no block barrier (six or four warps per SM, by loads or
+// TMA boxes) were latency bound: 55-65 us and 1090-1390 us.
 //
-// kRow: the other aggregation order (the region is the union over q on p's
-// horizontal arm of q's vertical segment): the block is one row y, the scan
-// runs along x over the vertical segment sums, the window is p's horizontal
-// arm and the region size adds u + d + 1 of every column.  Below, "rows" are
-// the scan positions.
-template <bool kMax, bool kRow>
-__device__ __forceinline__ void vagg_body(const VArgs &a, int bx, int by, int bz)
+// kMax: the WTA takes the largest V (the vote counts of Eq. 4, at most
+// (2 L1 + 1)^2): it minimises 0x7fffffff - V.
+// kRow: the other aggregation order: the walk runs along x over the vertical
+// segment sums of four neighbouring rows, with p's horizontal arms.  Below,
+// "rows" are the positions of the walk and "columns" the lines across it.
+constexpr int kVCols = 4;        // columns per strip
+constexpr int kVWarps = 4;
+constexpr int kVThreads = 32 * kVWarps;
+constexpr int kVSub = 8;         // rows per warp and step
+constexpr int kVStep = kVWarps * kVSub;
+constexpr int kVRow = 512;       // ring bytes per row: 32 lanes x 16
+constexpr int kVTile = 128;      // reduction tile: bytes per output row (4 columns x 8 words)
+constexpr int kVHalf = 2;        // output rows whose window ends are loaded together (4 and 8: 1-2 % slower)
+// the output rows of a step read back to 2 L1 + 1 rows above it
+__host__ __device__ inline uint32_t vagg_ring_bytes(int L1)
 {
-    extern __shared__ __align__(16) uint32_t vsmem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int W = a.W, H = a.H, L1 = a.L1;
-    const int fix = bx, view = by;              // the column x (kRow: the row y)
-    const int E = kRow ? W : H;                 // extent of the scan
-    const int ys = bz * a.chunk, ye = min(E, ys + a.chunk);
-    const int ya = max(0, ys - L1), yb = min(E, ye + L1);
-    const int len = yb - ya;
-    auto pix = [&](int sp) -> size_t { return kRow ? (size_t)fix * W + sp : (size_t)sp * W + fix; };
-    uint32_t *Q = vsmem + kQ0;                // [nw * 32][kQS], Q[-1] = 0
-    uint32_t *T = Q + nw * kVSeg * kQS;       // [nw][32] segment sums
-    uint32_t *NQ = T + nw * 32;               // [len] prefix of l + r + 1
-    uint32_t *NT = NQ + len;                  // [nw]
-    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(vsmem) + 4u * (uint32_t)vagg_bar_word(len, nw) + 8u * warp;
-    if (((uint32_t)__cvta_generic_to_shared(Q) & 127u) != 0) {   // the tile copies need 128-byte alignment
-        if (threadIdx.x == 0 && a.status) atomicOr(a.status, kStatusAlign);
-        return;
-    }
+    return (uint32_t)((2 * L1 + 1 + kVSub - 1) / kVSub * kVSub + kVStep) * kVRow;
+}
+__host__ __device__ inline size_t vagg_smem_bytes(int L1)
+{
+    return vagg_ring_bytes(L1) + (kVWarps + 2) * 512 + kVWarps * (kVSub * kVTile + 128);
+}
+static_assert(((2 * kMaxL1 + kVSub) / kVSub * kVSub + kVStep) * kVRow <= 1 << 16, "k_vagg: ring offsets in 16 bits");
 
-    const CUtensorMap *tm = view ? &a.tm[1] : &a.tm[0];
-    const uint32_t *arms = reinterpret_cast<const uint32_t *>(view ? a.arms[1] : a.arms[0]) + pix(0);
-    const size_t astride = kRow ? 1 : (size_t)W;
-    const int sa = warp * kVSeg, sb = min(len, sa + kVSeg);   // relative to ya
-    const int nrow = max(0, sb - sa);
-    const int ng = (a.dc + 31) / 32;
-    const bool want_vol = a.vol != nullptr && view == a.vol_view;
-
-    if (lane == 0) mbar_init(bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    __syncwarp();
-    // group g's 32 rows of this warp's segment -> Q[sa .. sa + 31] (rows
-    // past the image are zero-filled, rows past yb are read and unused; the
-    // generic accesses of the previous group are ordered before the copy by
-    // the block barrier and the proxy fence)
-    auto issue = [&](int g) {
-        if (nrow == 0 || lane != 0) return;
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        mbar_expect_tx(bar, kVTileBytes);
-        if (a.skip_copy) return;   // failure test: the barrier's phase never completes
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(Q + sa * kQS);
-        if (a.tm_rank == 4)
-            tma_load_4d(dst, tm, 0, g, kRow ? ya + sa : fix, kRow ? fix : ya + sa, bar);
-        else
-            tma_load_3d(dst, tm, 32 * g, kRow ? ya + sa : fix, kRow ? fix : ya + sa, bar);
-    };
-    issue(0);   // the first group's rows are in flight during the arm-word work
-
-    // arm word of this lane's row and the region-size prefix (d independent)
-    const int r = sa + lane;
-    const bool rin = r < sb;
-    const uint32_t aw = rin ? __ldg(arms + (size_t)(ya + r) * astride) : 0u;
-    // window arms along the scan (computed where used: short live ranges),
-    // and the segment length across it
-    auto back = [&]() { return kRow ? (int)(aw & 0xffu) : (int)((aw >> 16) & 0xffu); };
-    auto fwd = [&]() { return kRow ? (int)((aw >> 8) & 0xffu) : (int)(aw >> 24); };
-    {
-        uint32_t nv = !rin ? 0u : kRow ? ((aw >> 16) & 0xffu) + (aw >> 24) + 1u : (aw & 0xffu) + ((aw >> 8) & 0xffu) + 1u;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {   // inclusive scan across the segment's rows
-            const uint32_t t = __shfl_up_sync(0xffffffffu, nv, o);
-            if (lane >= o) nv += t;
+// N(p) of Eq. 2: the segment lengths along p's second arm
+__device__ __forceinline__ uint32_t region_size(const uchar4 *arms, int W, size_t i, bool row_order)
+{
+    const uchar4 p = arms[i];
+    uint32_t n = 0;
+    if (!row_order)
+        for (int k = -(int)p.z; k <= (int)p.w; k++) {
+            const uchar4 q = arms[(ptrdiff_t)i + (ptrdiff_t)k * W];
+            n += q.x + q.y + 1u;
         }
-        if (rin) NQ[r] = nv;
-        if (lane == 31) NT[warp] = nv;
-    }
-    const bool out_row = rin && ya + r >= ys && ya + r < ye;
-    uint32_t bv = 0xffffffffu, bd = 0;
-    if (warp == 0) Q[-kQS + lane] = 0u;   // Q[-1]: read by rows whose up arm reaches the top
-    for (int g = 0; g < ng; g++) {
-        // ---- A: this warp's rows of the slice column, lane = disparity
-        const bool lost = nrow > 0 && !mbar_wait(bar, (uint32_t)(g & 1), a.wait_limit);
-        if (__syncthreads_or(lost)) {
-            // a copy did not complete: report it, issue no further copies,
-            // and give this warp's copy a last bounded wait before the
-            // block's shared memory is released
-            if (lost) {
-                if (lane == 0 && a.status) atomicOr(a.status, kStatusCopyTimeout);
-                mbar_wait(bar, (uint32_t)(g & 1), a.wait_limit);
+    else
+        for (int k = -(int)p.x; k <= (int)p.y; k++) {
+            const uchar4 q = arms[(ptrdiff_t)i + k];
+            n += q.z + q.w + 1u;
+        }
+    return n;
+}
+
+template <bool kMax, bool kRow, bool kVol>
+__device__ __forceinline__ void vagg_body(const VArgs &a, int blk)
+{
+    extern __shared__ __align__(128) uint8_t vring[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = lane >> 3, dq = lane & 7;
+    const int E = kRow ? a.W : a.H, F = kRow ? a.H : a.W;     // extents along and across the walk
+    const int pstep = kRow ? 1 : a.W, pcol = kRow ? a.W : 1;   // the same as pixel steps
+    const int L1 = a.L1;
+    const uint32_t rb = vagg_ring_bytes(L1);
+    uint4 *sums = reinterpret_cast<uint4 *>(vring + rb);                 // [kVWarps][32]: totals of the warps' rows
+    uint4 *carry = sums + kVWarps * 32;                                  // [2][32]: prefix before the step
+    uint8_t *tile = reinterpret_cast<uint8_t *>(carry + 2 * 32) + warp * (kVSub * kVTile + 128);   // [8 rows][32 lanes]
+    uint8_t *offs = tile + kVSub * kVTile;                               // ring offsets: [4 columns][8 rows]
+    uint8_t *own = vring + 16 * lane;                                    // the lane's words of ring row 0
+    const uint32_t step = (uint32_t)pstep * (uint32_t)a.dstride * 4u;    // slice bytes per row
+
+    // the block's runs of output rows: whole strips first, then its share of
+    // the strips that are left over
+    for (int k = 0;; k++) {
+        int strip, ys, ye;
+        if (k < a.rounds) {
+            strip = k * a.nblk + blk;
+            ys = 0;
+            ye = E;
+        } else {
+            int first, f, f1;   // strip and rows among those that are left
+            if (a.bands) {
+                first = blk / a.bands;
+                if (k > a.rounds || first >= a.rest) return;
+                f = (blk - first * a.bands) * a.share;
+                f1 = min(E, f + a.share);
+            } else {
+                const int f0 = blk * a.share;
+                f1 = min(f0 + a.share, a.rest * E);
+                first = f0 / E + k - a.rounds;
+                f = k == a.rounds ? f0 : first * E;
+                if (f >= f1) return;
+                f -= first * E;
+                f1 = min(E, f1 - first * E);
             }
-            return;
+            strip = a.rounds * a.nblk + first;
+            ys = f;
+            ye = f1;
         }
-        uint32_t *q = Q + sa * kQS + lane;
-        uint32_t tot = 0;
-        uint32_t v[kVSeg];
+        const int layer = strip / a.strips, view = layer / a.ng, g = layer - view * a.ng;
+        const int line = kVCols * (strip - layer * a.strips) + col;
+        const size_t pix0 = (size_t)min(line, F - 1) * pcol;   // lanes past the last column repeat it
+        const int dbase = a.d0 + 32 * g, nlive = min(32, min(a.dc - 32 * g, a.D - dbase));
+        const uint32_t *arms = reinterpret_cast<const uint32_t *>(view ? a.arms[1] : a.arms[0]) + pix0;
+        unsigned long long *best = (view ? a.best[1] : a.best[0]) + pix0;
+        // Rows enter the ring kVStep at a time, eight per warp; row ys + L1 is
+        // the first, at ring row 0.  The nfill rows before it end at the last
+        // ring row, and the row before them counts as zeros.
+        const int ya = max(0, ys - L1), yb = min(E, ye + L1);
+        int y = ys + kVSub * warp;   // the output row that the warp's first entering row completes
+        const uint8_t *src = reinterpret_cast<const uint8_t *>((view ? a.sh[1] : a.sh[0]) + pix0 * a.dstride + 32 * g) + 16 * dq;
+        uint4 v[kVSub];
+        auto load = [&](int row) {   // the warp's eight rows from `row` on
+            const uint8_t *p = src + (ptrdiff_t)row * (ptrdiff_t)step;
+            if (row + kVSub <= yb) {
 #pragma unroll
-        for (int u = 0; u < kVSeg; u++) { v[u] = q[u * kQS]; tot += v[u]; }
-        T[warp * 32 + lane] = tot;
+                for (int r = 0; r < kVSub; r++) v[r] = __ldg(reinterpret_cast<const uint4 *>(p + (size_t)r * step));
+            } else {   // (rows past the image are never read)
+#pragma unroll
+                for (int r = 0; r < kVSub; r++)
+                    v[r] = row + r < yb ? __ldg(reinterpret_cast<const uint4 *>(p + (size_t)r * step))
+                                        : make_uint4(0u, 0u, 0u, 0u);
+            }
+        };
+        auto arm_word = [&](int row) { return row < ye ? __ldg(arms + (size_t)row * pstep) : 0u; };
+        // the fill: a quarter of its rows per warp, all in flight at once
+        const int nfill = ys + L1 - ya, quarter = (nfill + kVWarps - 1) / kVWarps;
+        const int i0 = min(quarter * warp, nfill), i1 = min(i0 + quarter, nfill);
+        uint8_t *fill = own + rb - (uint32_t)nfill * kVRow;   // ring row of row ya
+        {
+            const uint8_t *p = src + (size_t)(ya + i0) * step;
+#pragma unroll 4
+            for (int i = i0; i < i1; i++, p += step)
+                if (ya + i < yb) cp_async16(fill + i * kVRow, p);
+        }
+        load(y + L1);
+        uint32_t aw = arm_word(y + dq);   // the lane's own row of the warp's eight
+        cp_async_wait_all();   // (a lane reads only what it copied itself)
+        uint4 t = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 4
+        for (int i = i0; i < i1; i++) {
+            const uint4 w = *reinterpret_cast<const uint4 *>(fill + i * kVRow);
+            t = make_uint4(t.x + w.x, t.y + w.y, t.z + w.z, t.w + w.w);
+        }
+        sums[32 * warp + lane] = t;
         __syncthreads();
-        uint32_t run = 0;
-        for (int w = 0; w < warp; w++) run += T[w * 32 + lane];
-        if (g == 0) {
-            // region-size offsets (once)
-            uint32_t noff = 0;
-            for (int w = 0; w < warp; w++) noff += NT[w];
-            if (rin) NQ[r] += noff;
+        uint4 run = make_uint4(0u, 0u, 0u, 0u);
+        if (warp == 0) *reinterpret_cast<uint4 *>(fill - kVRow) = run;
+        for (int w = 0; w < warp; w++) {
+            const uint4 s = sums[32 * w + lane];
+            run = make_uint4(run.x + s.x, run.y + s.y, run.z + s.z, run.w + s.w);
         }
-#pragma unroll
-        for (int u = 0; u < kVSeg; u++) {
-            run += v[u];
-            q[u * kQS] = run;
+#pragma unroll 4
+        for (int i = i0; i < i1; i++) {
+            uint4 *p = reinterpret_cast<uint4 *>(fill + i * kVRow);
+            const uint4 w = *p;
+            run = make_uint4(run.x + w.x, run.y + w.y, run.z + w.z, run.w + w.w);
+            *p = run;
         }
-        __syncthreads();
-        // ---- C: lane = output row, loop over the group's disparities
-        const int dbase = a.d0 + g * 32;
-        const int nlive = max(0, min(32, min(a.dc - g * 32, a.D - dbase)));
-        if (out_row) {
-            const uint32_t *qh = Q + (r + fwd()) * kQS;
-            const int lo = r - back() - 1;           // >= -1
-            const uint32_t *ql = Q + lo * kQS;
-            // running minimum; strict < keeps the smallest d on ties
-            uint32_t bj = 0xffffffffu, bmin = bv;
-            if (nlive == 32) {
-                const uint4 *qh4 = reinterpret_cast<const uint4 *>(qh), *ql4 = reinterpret_cast<const uint4 *>(ql);
-#pragma unroll 2
-                for (int j4 = 0; j4 < 8; j4++) {
-                    const uint4 h4 = qh4[j4], l4 = ql4[j4];
-                    const uint32_t hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+        if (warp == kVWarps - 1) carry[lane] = run;
+        __syncthreads();   // (the totals have been read)
+        uint32_t in = kVSub * kVRow * warp;   // ring offset of the warp's first entering row
+        int buf = 0;
+        for (int yb0 = ys; yb0 < ye; yb0 += kVStep) {
+            // ---- the column prefix over the block's kVStep rows
+            t = v[0];
 #pragma unroll
-                    for (int k = 0; k < 4; k++) {
-                        const uint32_t vv = kMax ? ~(hv[k] - lv[k]) : hv[k] - lv[k];
-                        bj = vv < bmin ? (uint32_t)(4 * j4 + k) : bj;
-                        bmin = min(bmin, vv);
+            for (int r = 1; r < kVSub; r++) t = make_uint4(t.x + v[r].x, t.y + v[r].y, t.z + v[r].z, t.w + v[r].w);
+            sums[32 * warp + lane] = t;
+            __syncthreads();   // (also: the window reads of the last step are done)
+            run = carry[32 * buf + lane];
+            for (int w = 0; w < warp; w++) {
+                const uint4 s = sums[32 * w + lane];
+                run = make_uint4(run.x + s.x, run.y + s.y, run.z + s.z, run.w + s.w);
+            }
+            {
+                uint8_t *p = own + in;
+#pragma unroll
+                for (int r = 0; r < kVSub; r++) {
+                    run = make_uint4(run.x + v[r].x, run.y + v[r].y, run.z + v[r].z, run.w + v[r].w);
+                    *reinterpret_cast<uint4 *>(p + r * kVRow) = run;
+                }
+            }
+            buf ^= 1;
+            if (warp == kVWarps - 1) carry[32 * buf + lane] = run;
+            load(y + kVStep + L1);   // the next step's rows are in flight during this one's output
+            // and the lines of the step after it, one per lane, on their way to
+            // L2 (a second step in registers made every wait on the first one
+            // wait for both: 860 against 1190 us at 1920x1080, D = 256)
+            if (const int row = y + 2 * kVStep + L1 + dq; row < yb)
+                asm volatile("prefetch.global.L2 [%0];\n" ::"l"(src - 16 * dq + (ptrdiff_t)row * (ptrdiff_t)step));
+            const uint32_t aw_next = arm_word(y + kVStep + dq);
+            // ring offsets of the windows, each lane its own row's, passed to
+            // the lanes of its column packed in one word
+            const uint32_t back = kRow ? aw & 0xffu : (aw >> 16) & 0xffu, fwd = kRow ? (aw >> 8) & 0xffu : aw >> 24;
+            uint32_t h = in + (dq + fwd) * kVRow + rb - L1 * kVRow, l = in + dq * kVRow + rb - (L1 + 1 + back) * kVRow;
+            h = min(h, h - rb);   // modulo the ring (h below 3 rb, l below 2 rb)
+            h = min(h, h - rb);
+            l = min(l, l - rb);
+            *reinterpret_cast<uint32_t *>(offs + 4 * lane) = h | l << 16;
+            __syncthreads();
+            // ---- the warp's output rows y .. y + 7
+            if (y < ye) {
+                const uint4 o0 = *reinterpret_cast<const uint4 *>(offs + 32 * col);
+                const uint4 o1 = *reinterpret_cast<const uint4 *>(offs + 32 * col + 16);
+                const uint32_t ov[kVSub] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
+                uint32_t who = 0;   // per row, which of the lane's four disparities wins
+#pragma unroll
+                for (int r0 = 0; r0 < kVSub; r0 += kVHalf) {
+                    uint4 hi[kVHalf], lo[kVHalf];
+#pragma unroll
+                    for (int r = 0; r < kVHalf; r++) {
+                        hi[r] = *reinterpret_cast<const uint4 *>(vring + ((ov[r0 + r] & 0xffffu) | 16 * lane));
+                        lo[r] = *reinterpret_cast<const uint4 *>(vring + (ov[r0 + r] >> 16) + 16 * lane);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kVHalf; u++) {
+                        const int r = r0 + u;
+                        uint32_t c[4] = {hi[u].x - lo[u].x, hi[u].y - lo[u].y, hi[u].z - lo[u].z, hi[u].w - lo[u].w};
+                        if (kVol && view == a.vol_view && line < F && y + r < ye) {
+                            const size_t p = pix0 + (size_t)(y + r) * pstep;
+                            const uint32_t n =
+                                region_size(reinterpret_cast<const uchar4 *>(view ? a.arms[1] : a.arms[0]), a.W, p, kRow);
+#pragma unroll
+                            for (int j = 0; j < 4; j++)
+                                if (4 * dq + j < nlive)
+                                    a.vol[(size_t)(dbase + 4 * dq + j - a.dmin) * a.H * a.W + p] =
+                                        float(c[j]) / (float(n) * a.S);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; j++)
+                            if (kMax) c[j] = 0x7fffffffu - c[j];
+                        if (nlive < 32) {
+#pragma unroll
+                            for (int j = 0; j < 4; j++) c[j] = 4 * dq + j < nlive ? c[j] : 0xffffffffu;
+                        }
+                        bool p01, p23, p;
+                        const uint32_t m01 = __vibmin_u32(c[0], c[1], &p01), m23 = __vibmin_u32(c[2], c[3], &p23);
+                        const uint32_t m = __vibmin_u32(m01, m23, &p);   // p: m01 <= m23
+                        who = 4u * who + (p ? (p01 ? 0u : 1u) : (p23 ? 2u : 3u));
+                        // 16-byte chunks of row r permuted by r: the reads below hit distinct banks
+                        *reinterpret_cast<uint32_t *>(tile + r * kVTile + ((4 * lane) ^ (16 * r))) = m;
                     }
                 }
-            } else {
-                for (int j = 0; j < nlive; j++) {
-                    const uint32_t vv = kMax ? ~(qh[j] - ql[j]) : qh[j] - ql[j];
-                    bj = vv < bmin ? (uint32_t)j : bj;
-                    bmin = min(bmin, vv);
+                __syncwarp();
+                // the lane's row y + dq: the minimum over the eight lanes of its
+                // column, and which of that lane's four disparities has it
+                const uint8_t *row = tile + dq * kVTile;
+                const uint4 t0 = *reinterpret_cast<const uint4 *>(row + ((32 * col) ^ (16 * dq)));
+                const uint4 t1 = *reinterpret_cast<const uint4 *>(row + ((32 * col + 16) ^ (16 * dq)));
+                const uint32_t tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+                uint32_t m = tv[0];
+                int q = 0;
+#pragma unroll
+                for (int i = 1; i < 8; i++) {
+                    q = tv[i] < m ? i : q;   // strict: the smallest d on ties
+                    m = min(m, tv[i]);
+                }
+                const uint32_t w = __shfl_sync(0xffffffffu, who, (lane & 24) | q);
+                const uint32_t j = (w >> (2 * (kVSub - 1 - dq))) & 3u;
+                if (line < F && y + dq < ye) {
+                    const unsigned long long key = ((unsigned long long)m << 32) | (uint32_t)(dbase + 4 * q + j);
+                    unsigned long long *b = best + (size_t)(y + dq) * pstep;
+                    if (a.single) *b = key;
+                    else atomicMin(b, key);
                 }
             }
-            if (bj != 0xffffffffu) { bv = bmin; bd = (uint32_t)dbase + bj; }
-            if (want_vol) {
-                const uint32_t n = NQ[r + fwd()] - (lo >= 0 ? NQ[lo] : 0u);
-                for (int j = 0; j < nlive; j++) {
-                    const uint32_t vv = qh[j] - ql[j];
-                    a.vol[(size_t)(dbase - a.dmin + j) * H * W + pix(ya + r)] = float(vv) / (float(n) * a.S);
-                }
-            }
+            aw = aw_next;
+            y += kVStep;
+            in += kVStep * kVRow;
+            in = min(in, in - rb);
         }
-        __syncthreads();   // Q and T are reused by the next group
-        if (g + 1 < ng) issue(g + 1);
-    }
-    // ---- merge with earlier passes, write the disparity (last pass) or state
-    if (!out_row) return;
-    unsigned long long *best = view ? a.best[1] : a.best[0];
-    int16_t *disp = view ? a.disp[1] : a.disp[0];
-    float *cost = view ? a.cost[1] : a.cost[0];
-    const size_t i = pix(ya + r);
-    unsigned long long key = ((unsigned long long)bv << 32) | bd;
-    if (!a.first) {
-        const unsigned long long prev = best[i];
-        key = prev <= key ? prev : key;   // earlier passes hold smaller d
-    }
-    if (a.last) {
-        const bool invalid = kMax && (a.mask[i] < a.dmin || a.mask[i] >= a.D);   // Eq. 4: no vote, stays invalid
-        disp[i] = invalid ? (int16_t)-1 : (int16_t)(key & 0xffffffffu);
-        if (cost) {
-            const int lo = r - back() - 1;
-            const uint32_t n = NQ[r + fwd()] - (lo >= 0 ? NQ[lo] : 0u);
-            cost[i] = float(uint32_t(key >> 32)) / (float(n) * a.S);
-        }
-    } else {
-        best[i] = key;
+        __syncthreads();   // the ring is the next run's
     }
 }
 
@@ -1250,6 +1326,33 @@ __device__ __forceinline__ void lr_body(const LrArgs &a, size_t i)
         if (d2 >= 0 && abs(d - d2) <= a.tol) r = (int16_t)d;
     }
     a.out[i] = r;
+}
+
+// -------------------------------------------------------------------- k_end
+// The per-pixel end of a match: the winners' keys become the two views'
+// disparities and minimum costs (where asked for) and the consistency map.
+// The region size N(p) of a cost is summed on the spot: only callers that
+// ask for costs pay for it.
+__device__ __forceinline__ void end_body(const EndArgs &a, size_t i)
+{
+    if (i >= (size_t)a.W * a.H) return;
+    const int x = int(i % a.W);
+    const unsigned long long kl = a.best[0][i];
+    const int d = (int)(kl & 0xffffu);
+    if (a.out) {
+        int16_t r = -1;
+        if (a.tol < 0) r = (int16_t)d;
+        else if (x - d >= 0 && abs(d - (int)(a.best[1][i - d] & 0xffffu)) <= a.tol) r = (int16_t)d;
+        a.out[i] = r;
+    }
+#pragma unroll
+    for (int v = 0; v < 2; v++) {
+        if (!a.disp[v] && !a.cost[v]) continue;
+        const unsigned long long k = v ? a.best[1][i] : kl;
+        if (a.disp[v]) a.disp[v][i] = (int16_t)(k & 0xffffu);
+        if (a.cost[v])
+            a.cost[v][i] = float(uint32_t(k >> 32)) / (float(region_size(a.arms[v], a.W, i, a.order == 1)) * a.S);
+    }
 }
 
 // ------------------------------------------------------ quarter size, depth
@@ -1378,13 +1481,13 @@ __global__ void __launch_bounds__(kWide ? 1024 : kHNarrow * 32) k_hagg(const __g
     hagg_body(b.p[i], bx, by, bz);
 }
 
-template <int N, bool kMax, bool kRow = false>
-__global__ void __launch_bounds__(16 * 32, 2) k_vagg(const __grid_constant__ Batch<VArgs, N> b)
+template <int N, bool kMax, bool kRow, bool kVol>
+__global__ void __launch_bounds__(kVThreads, 4) k_vagg(const __grid_constant__ Batch<VArgs, N> b)
 {
     pdl_enter();
     int bx, by, bz;
     const int i = batch_pair(b, blockIdx.x, bx, by, bz);
-    vagg_body<kMax, kRow>(b.p[i], bx, by, bz);
+    vagg_body<kMax, kRow, kVol>(b.p[i], bx);
 }
 
 template <int N>
@@ -1412,6 +1515,28 @@ __global__ void __launch_bounds__(256) k_lr(const __grid_constant__ Batch<LrArgs
     int bx, by, bz;
     const int i = batch_pair(b, blockIdx.x, bx, by, bz);
     lr_body(b.p[i], (size_t)bx * 256 + threadIdx.x);
+}
+
+template <int N>
+__global__ void __launch_bounds__(256) k_end(const __grid_constant__ Batch<EndArgs, N> b)
+{
+    pdl_enter();
+    int bx, by, bz;
+    const int i = batch_pair(b, blockIdx.x, bx, by, bz);
+    end_body(b.p[i], (size_t)bx * 256 + threadIdx.x);
+}
+
+template <int N>
+__global__ void __launch_bounds__(256) k_vote_end(const __grid_constant__ Batch<VoteEndArgs, N> b)
+{
+    pdl_enter();
+    int bx, by, bz;
+    const int i = batch_pair(b, blockIdx.x, bx, by, bz);
+    const VoteEndArgs &a = b.p[i];
+    const int k = bx * 256 + threadIdx.x;
+    if (k >= a.npx) return;
+    const int v = a.mask[k];
+    a.out[k] = v >= a.dmin && v < a.D ? (int16_t)(a.best[k] & 0xffffu) : (int16_t)-1;
 }
 
 __global__ void k_extract_census(const uint4 *__restrict__ rec, int W, int H, int rpitch,
@@ -1451,11 +1576,12 @@ struct Derived {
 };
 
 struct Layout {
-    size_t rgbx[2], grey[2], rec[2], cen[2], col[2], arms[2], atmp[2], best[2], disp[2], sh[2], vtmp, total;
+    size_t rgbx[2], grey[2], rec[2], cen[2], col[2], arms[2], atmp[2], best[2], sh[2], total;
     int dc, dstride, npass, rpitch, phw;
 };
 
 constexpr size_t kAlign = 256;
+constexpr size_t kSmShared = 228 << 10, kBlockShared = 1 << 10;   // shared memory of an SM; kept back per block
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 bool derive(const dco_params &p, Derived &d)
@@ -1531,11 +1657,8 @@ Layout make_layout(int W, int H, int D, const dco_params &p, int dc_override = 0
     // arms: 16 bytes of slack, read by the cost pass's bulk copies past the last pixel
     for (int v = 0; v < 2; v++) { L.arms[v] = off; off = align_up(off + 4 * npx + 16); }
     for (int v = 0; v < 2; v++) { L.atmp[v] = off; off = align_up(off + (p.smooth_arms ? 4 * npx : 0)); }
-    for (int v = 0; v < 2; v++) { L.best[v] = off; off = align_up(off + (L.npass > 1 ? 8 * npx : 0)); }
-    for (int v = 0; v < 2; v++) { L.disp[v] = off; off = align_up(off + 2 * npx); }
+    for (int v = 0; v < 2; v++) { L.best[v] = off; off = align_up(off + 8 * npx); }
     for (int v = 0; v < 2; v++) { L.sh[v] = off; off = align_up(off + 4 * npx * (size_t)L.dstride); }
-    L.vtmp = off;   // second map of the Eq. 4 rounds
-    off = align_up(off + (p.vote_iters > 0 ? 2 * npx : 0));
     L.total = off;
     return L;
 }
@@ -1585,61 +1708,52 @@ HGeom hagg_geom(int W, int H, int dc, int L1, int want)
     return g;
 }
 
-// V geometry: one block per (column, view, chunk of output rows)
+// V geometry: the walk is dealt out to as many blocks as the SMs hold at once:
+// whole strips (kVCols columns of one group and view) round by round,
+// neighbouring blocks on neighbouring strips; the strips that are left are
+// cut into bands, or, where there are too many for two bands each, into equal
+// shares that run on from strip to strip.  A run costs its fill of up to 2 L1
+// rows again, so strips of at most kVRunOn rows are not shared (160x120,
+// D = 16: 8.4 us in bands, 11.5 us in shares that run on).
 struct VGeom {
-    int chunk, nw, seglog;
-    size_t smem;
-    dim3 grid;
+    int strips;   // per layer (group and view)
+    int rounds, rest, share, bands, nblk;   // bands: per strip that is left (0: shares run on)
 };
+constexpr int kVRunOn = 256;
 
-VGeom vagg_geom(int W, int H, int L1, int want)
+size_t vagg_units(int F, int layers) { return (size_t)((F + kVCols - 1) / kVCols) * layers; }
+
+// `blocks`: this pair's part of the resident blocks; want > 0: rows per band
+VGeom vagg_geom(int E, int F, int layers, int want, int blocks)
 {
     VGeom g{};
-    // at most 16 warps of 32 rows: the prefix range (chunk + 2*L1) <= 512;
-    // balanced chunks of at most `want` rows (automatic: whole columns up
-    // to 512 rows, else at most 512 - 2 kMaxL1)
-    int nchunks;
-    if (want <= 0) {
-        nchunks = H <= 512 ? 1 : (H + (512 - 2 * kMaxL1) - 1) / (512 - 2 * kMaxL1);
+    g.strips = (F + kVCols - 1) / kVCols;
+    const int units = g.strips * layers;
+    if (want > 0) {
+        g.bands = (E + want - 1) / want;
+        g.rest = units;
     } else {
-        int c = std::min(want, H);
-        if (c < H || H > 512) c = std::min(c, 512 - 2 * L1);
-        nchunks = (H + c - 1) / c;
+        g.rounds = units / blocks;
+        g.rest = units - g.rounds * blocks;
+        const int nb = g.rest > 0 ? blocks / g.rest : 1;
+        if (nb > 1) g.bands = std::min(nb, (E + kVStep - 1) / kVStep);
+        else if (E <= kVRunOn) g.bands = 1;
     }
-    g.chunk = (H + nchunks - 1) / nchunks;
-    const int len = std::min(H, g.chunk + 2 * L1);
-    g.seglog = 5;   // 32 rows per warp, one output row per lane
-    g.nw = (len + kVSeg - 1) / kVSeg;
-    g.smem = vagg_smem_words(len, g.nw) * 4;
-    g.grid = dim3(W, 2, nchunks);
+    const long long rows = g.bands ? E : (long long)g.rest * E;
+    const int parts = g.bands ? g.bands : blocks;
+    g.share = (int)((rows + parts - 1) / parts);
+    if (want <= 0) g.share = std::max(1, (g.share + kVStep - 1) / kVStep) * kVStep;   // whole steps
+    if (g.bands) g.bands = (E + g.share - 1) / g.share;
+    const int tail = g.bands ? g.rest * g.bands : (int)((rows + g.share - 1) / g.share);
+    g.nblk = g.rounds > 0 ? blocks : tail;
     return g;
 }
-
-// ---- TMA tile maps of the slices (k_vagg)
-using TmapEncode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-TmapEncode tmap_encoder()
-{
-    static TmapEncode fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q{};
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<TmapEncode>(f);
-    });
-    return fn;
-}
-
 
 } // namespace
 
 struct dco_stereo {
     int device = 0;
+    int nsm = 152;                           // multiprocessors of the device
     size_t budget = 0;
     char *ws = nullptr;
     size_t ws_cap = 0;
@@ -1821,12 +1935,8 @@ T *ws_ptr(dco_stereo *h, size_t off) { return reinterpret_cast<T *>(h->ws + off)
 // image 0 go to arms0 (the caller's buffer for the arms entry point)
 // ----------------------------------------------------------- batched launches
 constexpr int kBatchMax = 64;   // pairs per launch (kernel parameter space)
-// pairs per launch of a kind of argument block: the V blocks carry two
-// tensor maps, so half as many fit the 32764 bytes of kernel parameters
-template <class A> constexpr int batch_max() { return sizeof(A) > 256 ? kBatchMax / 2 : kBatchMax; }
-static_assert(sizeof(Batch<VArgs, batch_max<VArgs>()>) <= 32764, "kernel parameters of a full V batch");
-static_assert(sizeof(Batch<HArgs, batch_max<HArgs>()>) <= 32764, "kernel parameters of a full H batch");
-constexpr int kVBatch = batch_max<VArgs>();
+static_assert(sizeof(Batch<VArgs, kBatchMax>) <= 32764, "kernel parameters of a full V batch");
+static_assert(sizeof(Batch<HArgs, kBatchMax>) <= 32764, "kernel parameters of a full H batch");
 
 // The dynamic shared-memory limit is an attribute of the kernel on a device,
 // shared by every handle and thread of the process: it is raised under a lock
@@ -1883,12 +1993,12 @@ dco_status launch_group(dco_stereo *h, cudaStream_t s, const char *name, K kerne
 }
 
 // one launch for a single pair (small parameter block), else groups of
-// batch_max<A>() (kn is the kernel instance for that many)
+// kBatchMax (kn is the kernel instance for that many)
 template <class A, class K1, class KN>
 dco_status launch_items(dco_stereo *h, cudaStream_t s, const char *name, K1 k1, KN kn,
                         const std::vector<Item<A>> &items, int block, size_t smem)
 {
-    constexpr int nmax = batch_max<A>();
+    constexpr int nmax = kBatchMax;
     if (items.empty()) return DCO_OK;
     if (items.size() == 1) return launch_group<A, 1>(h, s, name, k1, items.data(), 1, block, smem);
     for (size_t i = 0; i < items.size(); i += nmax) {
@@ -1910,8 +2020,8 @@ struct Job {
     int dchunk = 0;                  // this pair's pass width (0: the call's parameters)
     int hchunk = 0, vchunk = 0;      // this pair's tile shapes (0: the call's parameters)
     int host_in = -1;                // images in host memory: 1, in device memory: 0, -1: ask the driver
-    const int16_t *vsrc = nullptr;   // Eq. 4 round: map voted on (null: no vote)
-    int16_t *vdst = nullptr;         //   and the map written
+    const unsigned long long *vkeys = nullptr;   // Eq. 4 round: the previous round's keys (null: first round)
+    unsigned long long *vbest = nullptr;         //   and the keys it minimises into
     Layout L{};
     size_t base = 0;           // workspace offset of this pair
 };
@@ -2042,78 +2152,40 @@ dco_status launch_prep(dco_stereo *h, const dco_params &p, const Derived &dv, co
 // pass `pass` (disparities [pass*dc, pass*dc + dc)) of every job that has it.
 // Pairs are bucketed by block size (warps per block) so no block carries
 // idle warps for a larger pair; one launch per bucket and stage.
-// The slice of one view (dstride words per pixel, pixel index y * W + x) for
-// the tile copies of k_vagg: a box of 36 words (the group's 32 disparities
-// and 4 words of padding) by 32 consecutive rows (row_scan: columns).  Rank
-// 4: dims (disparity within the group, group, x, y), the padding beyond the
-// 32-long dimension 0 is zero-filled without a read.  Rank 3 (used if the
-// encoder refuses a box wider than dimension 0): dims (disparity, x, y), the
-// padding reads the next group's first words (zeros past the last group).
-dco_status slice_map(dco_stereo *h, VArgs &a, int v, const uint32_t *slice, int W, int H, int dstride, bool row_scan)
+// Deals the resident V blocks of a launch out to its pairs by their work
+// (strips x rows; a pair's own v_chunk in it[].gy, the layers in it[].gz).
+void deal_v_blocks(const dco_stereo *h, std::vector<Item<VArgs>> &it, int L1, bool row_scan)
 {
-    // the encoder's answer for rank 4, kept for the process (serving lanes
-    // encode maps from several threads)
-    static std::atomic<int> rank_seen{4};
-    int rank = rank_seen.load(std::memory_order_relaxed);
-    TmapEncode enc = tmap_encoder();
-    if (!enc) {
-        h->last_error = "cuTensorMapEncodeTiled is not available";
-        return DCO_ECUDA;
+    const int slots = h->nsm * std::max(1, (int)(kSmShared / (vagg_smem_bytes(L1) + kBlockShared)));
+    double all = 0.0;
+    for (auto &b : it)
+        all += double(vagg_units(row_scan ? b.a.H : b.a.W, b.gz)) * (row_scan ? b.a.W : b.a.H);
+    for (auto &b : it) {
+        const int E = row_scan ? b.a.W : b.a.H, F = row_scan ? b.a.H : b.a.W;
+        const int mine = std::max(1, (int)(slots * (double(vagg_units(F, b.gz)) * E / all)));
+        const VGeom g = vagg_geom(E, F, b.gz, b.gy, mine);
+        b.a.strips = g.strips;
+        b.a.nblk = g.nblk; b.a.rounds = g.rounds; b.a.rest = g.rest; b.a.share = g.share; b.a.bands = g.bands;
+        b.gx = g.nblk;
+        b.gy = b.gz = 1;
     }
-    const cuuint32_t rows = row_scan ? 1u : (cuuint32_t)kVSeg, cols = row_scan ? (cuuint32_t)kVSeg : 1u;
-    const cuuint32_t es[4] = {1, 1, 1, 1};
-    CUresult r = CUDA_ERROR_INVALID_VALUE;
-    if (rank == 4) {
-        const cuuint64_t dims[4] = {32, (cuuint64_t)(dstride / 32), (cuuint64_t)W, (cuuint64_t)H};
-        const cuuint64_t strides[3] = {128, (cuuint64_t)dstride * 4, (cuuint64_t)W * dstride * 4};
-        const cuuint32_t box[4] = {(cuuint32_t)kQS, 1, cols, rows};
-        r = enc(&a.tm[v], CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, const_cast<uint32_t *>(slice), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) {
-            rank = 3;
-            rank_seen.store(3, std::memory_order_relaxed);
-        }
-    }
-    if (rank == 3) {
-        const cuuint64_t dims[3] = {(cuuint64_t)dstride, (cuuint64_t)W, (cuuint64_t)H};
-        const cuuint64_t strides[2] = {(cuuint64_t)dstride * 4, (cuuint64_t)W * dstride * 4};
-        const cuuint32_t box[3] = {(cuuint32_t)kQS, cols, rows};
-        r = enc(&a.tm[v], CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint32_t *>(slice), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    }
-    if (r != CUDA_SUCCESS) {
-        h->last_error = "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
-        return DCO_ECUDA;
-    }
-    a.tm_rank = rank;
-    return DCO_OK;
-}
-
-// bounded tile waits of the V pass; the lost-copy failure test arms the
-// barriers without copies and gives up after a few polls
-void set_wait(const dco_stereo *h, VArgs &a)
-{
-    const bool lose = (h->test_flags & DCO_TEST_LOSE_TILE_COPIES) != 0;
-    a.wait_limit = lose ? kTestWaitLimit : kWaitLimit;
-    a.skip_copy = lose ? 1 : 0;
 }
 
 dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> &jobs, int pass, cudaStream_t s)
 {
     std::map<int, std::vector<Item<HArgs>>> hb;
-    std::map<int, std::vector<Item<VArgs>>> vb;
-    std::map<int, size_t> hsm, vsm;
+    std::vector<Item<VArgs>> vb, vvol;
+    std::map<int, size_t> hsm;
+    const size_t vsm = vagg_smem_bytes(dv.L1);
     const bool vh = dv.order == 1;   // vertical segment sums first (k_vcost), then rows (k_vagg<.., kRow>)
     for (const Job &j : jobs) {
         if (pass >= j.L.npass) continue;
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
+        const int ng = (dc + 31) / 32;
         const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk, vw = j.vchunk > 0 ? j.vchunk : dv.vchunk;
         const HGeom hg = vh ? vcost_geom(j.W, j.H, dc, dv.L1, hw) : hagg_geom(j.W, j.H, dc, dv.L1, hw);
-        const VGeom vg = vh ? vagg_geom(j.H, j.W, dv.L1, vw) : vagg_geom(j.W, j.H, dv.L1, vw);
+        const bool single = j.L.npass == 1 && ng == 1;
         hsm[hg.nw] = std::max(hsm[hg.nw], hg.smem);
-        vsm[vg.nw] = std::max(vsm[vg.nw], vg.smem);
         Item<HArgs> a{};
         for (int v = 0; v < 2; v++) {
             a.a.rec[v] = jptr<uint4>(h, j, j.L.rec[v]) + kRPad;
@@ -2121,6 +2193,7 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
             a.a.col[v] = jptr<uint32_t>(h, j, j.L.col[v]);
             a.a.arms[v] = jptr<uchar4>(h, j, j.L.arms[v]);
             a.a.sh[v] = jptr<uint32_t>(h, j, j.L.sh[v]);
+            a.a.init[v] = pass == 0 && !single ? jptr<unsigned long long>(h, j, j.L.best[v]) : nullptr;
         }
         a.a.phw = j.L.phw;
         a.a.status = h->d_status;
@@ -2132,7 +2205,7 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
         a.a.tables = h->d_tables;
         a.a.W = j.W; a.a.H = j.H; a.a.D = dv.dmin + j.D; a.a.rpitch = j.L.rpitch;
         a.a.d0 = d0; a.a.dc = dc; a.a.dstride = j.L.dstride;
-        a.a.ngroups = (dc + 31) / 32;
+        a.a.ngroups = ng;
         a.a.L1 = dv.L1; a.a.chunk = hg.chunk; a.a.S = dv.S; a.a.Sint = dv.Sint;
         a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = hg.grid.z;
         hb[hg.nw].push_back(a);
@@ -2142,21 +2215,17 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
             b.a.arms[v] = a.a.arms[v];
             b.a.best[v] = jptr<unsigned long long>(h, j, j.L.best[v]);
         }
-        b.a.disp[0] = j.disp_l; b.a.disp[1] = j.disp_r;
-        b.a.cost[0] = j.cost_l; b.a.cost[1] = j.cost_r;
         b.a.vol = j.vol; b.a.vol_view = j.vol_view;
         b.a.W = j.W; b.a.H = j.H; b.a.D = dv.dmin + j.D; b.a.dmin = dv.dmin;
         b.a.d0 = d0; b.a.dc = dc; b.a.dstride = j.L.dstride;
-        b.a.first = pass == 0; b.a.last = pass == j.L.npass - 1;
-        b.a.status = h->d_status; b.a.L1 = dv.L1; b.a.chunk = vg.chunk; b.a.seglog = vg.seglog; b.a.S = dv.S;
-        set_wait(h, b.a);
-        for (int v = 0; v < 2; v++) {
-            dco_status st = slice_map(h, b.a, v, b.a.sh[v], j.W, j.H, j.L.dstride, vh);
-            if (st != DCO_OK) return st;
-        }
-        b.gx = vg.grid.x; b.gy = vg.grid.y; b.gz = vg.grid.z;
-        vb[vg.nw].push_back(b);
+        b.a.ng = ng; b.a.single = single;
+        b.a.L1 = dv.L1; b.a.S = dv.S;
+        b.gy = vw;
+        b.gz = 2 * ng;
+        (j.vol ? vvol : vb).push_back(b);
     }
+    deal_v_blocks(h, vb, dv.L1, vh);
+    deal_v_blocks(h, vvol, dv.L1, vh);
     for (auto &kv : hb) {
         if (vh) {
             dco_status st = launch_items(h, s, "k_vcost", k_vcost<1>, k_vcost<kBatchMax>, kv.second, kv.first * 32,
@@ -2171,11 +2240,15 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
                                            kv.first * 32, hsm[kv.first]);
         if (st != DCO_OK) return st;
     }
-    for (auto &kv : vb) {
-        dco_status st = vh ? launch_items(h, s, "k_hwta", k_vagg<1, false, true>, k_vagg<kVBatch, false, true>,
-                                          kv.second, kv.first * 32, vsm[kv.first])
-                           : launch_items(h, s, "k_vagg", k_vagg<1, false>, k_vagg<kVBatch, false>, kv.second,
-                                          kv.first * 32, vsm[kv.first]);
+    dco_status st = vh ? launch_items(h, s, "k_hwta", k_vagg<1, false, true, false>,
+                                      k_vagg<kBatchMax, false, true, false>, vb, kVThreads, vsm)
+                       : launch_items(h, s, "k_vagg", k_vagg<1, false, false, false>,
+                                      k_vagg<kBatchMax, false, false, false>, vb, kVThreads, vsm);
+    if (st != DCO_OK) return st;
+    // (a cost volume is asked for one pair at a time)
+    for (const auto &it : vvol) {
+        st = vh ? launch_group<VArgs, 1>(h, s, "k_hwta", k_vagg<1, false, true, true>, &it, 1, kVThreads, vsm)
+                : launch_group<VArgs, 1>(h, s, "k_vagg", k_vagg<1, false, false, true>, &it, 1, kVThreads, vsm);
         if (st != DCO_OK) return st;
     }
     return DCO_OK;
@@ -2193,81 +2266,82 @@ dco_status launch_vote_pass(dco_stereo *h, const Derived &dv, const std::vector<
                             cudaStream_t s)
 {
     std::map<int, std::vector<Item<HVArgs>>> hb;
-    std::map<int, std::vector<Item<VArgs>>> vb;
-    std::map<int, size_t> hsm, vsm;
+    std::vector<Item<VArgs>> vb;
+    std::map<int, size_t> hsm;
+    const size_t vsm = vagg_smem_bytes(dv.L1);
     for (const Job &j : jobs) {
-        if (!j.vsrc || pass >= j.L.npass) continue;
+        if (!j.vbest || pass >= j.L.npass) continue;
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
+        const int ng = (dc + 31) / 32;
         const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk, vw = j.vchunk > 0 ? j.vchunk : dv.vchunk;
         const HGeom hg = hagg_geom(j.W, j.H, dc, dv.L1, hw);
-        const VGeom vg = vagg_geom(j.W, j.H, dv.L1, vw);
-        const int hlen = std::min(j.W, hg.chunk + 2 * dv.L1), vlen = std::min(j.H, vg.chunk + 2 * dv.L1);
+        const bool single = j.L.npass == 1 && ng == 1;
+        const int hlen = std::min(j.W, hg.chunk + 2 * dv.L1);
         const int hnw = (hlen + kHSeg - 1) / kHSeg;   // the vote pass walks 64-column segments
         hsm[hnw] = std::max(hsm[hnw], (size_t)HVSmem(hlen, hg.chunk, hnw).total);
-        vsm[vg.nw] = std::max(vsm[vg.nw], vagg_smem_words(vlen, vg.nw) * 4);
         Item<HVArgs> a{};
-        a.a.disp = j.vsrc;
+        a.a.disp = j.out;
+        a.a.keys = j.vkeys;
+        a.a.init = pass == 0 && !single ? j.vbest : nullptr;
+        a.a.dmin = dv.dmin; a.a.D = dv.dmin + j.D;
         a.a.arms = jptr<uchar4>(h, j, j.L.arms[0]);
         a.a.sh = jptr<uint32_t>(h, j, j.L.sh[0]);
         a.a.W = j.W; a.a.H = j.H; a.a.d0 = d0; a.a.dstride = j.L.dstride;
         a.a.L1 = dv.L1; a.a.chunk = hg.chunk;
-        a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = (dc + 31) / 32;
+        a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = ng;
         hb[hnw].push_back(a);
         Item<VArgs> b{};
-        for (int v = 0; v < 2; v++) {
-            b.a.sh[v] = a.a.sh;
-            b.a.arms[v] = a.a.arms;
-            b.a.best[v] = jptr<unsigned long long>(h, j, j.L.best[0]);
-            b.a.disp[v] = j.vdst;
-        }
-        b.a.mask = j.vsrc;
+        b.a.sh[0] = a.a.sh;
+        b.a.arms[0] = a.a.arms;
+        b.a.best[0] = j.vbest;
         b.a.W = j.W; b.a.H = j.H; b.a.D = dv.dmin + j.D; b.a.dmin = dv.dmin;
         b.a.d0 = d0; b.a.dc = dc; b.a.dstride = j.L.dstride;
-        b.a.first = pass == 0; b.a.last = pass == j.L.npass - 1;
-        b.a.status = h->d_status; b.a.L1 = dv.L1; b.a.chunk = vg.chunk; b.a.seglog = vg.seglog; b.a.S = dv.S;
-        set_wait(h, b.a);
-        if (dco_status st = slice_map(h, b.a, 0, b.a.sh[0], j.W, j.H, j.L.dstride, false); st != DCO_OK) return st;
-        b.a.tm[1] = b.a.tm[0];
-        b.gx = vg.grid.x; b.gy = 1; b.gz = vg.grid.z;   // the left view only
-        vb[vg.nw].push_back(b);
+        b.a.ng = ng; b.a.single = single;
+        b.a.L1 = dv.L1; b.a.S = dv.S;
+        b.gy = vw;
+        b.gz = ng;   // the left view only
+        vb.push_back(b);
     }
+    deal_v_blocks(h, vb, dv.L1, false);
     for (auto &kv : hb) {
         dco_status st = launch_items(h, s, "k_hvote", k_hvote<1>, k_hvote<kBatchMax>, kv.second, kv.first * 32,
                                      hsm[kv.first]);
         if (st != DCO_OK) return st;
     }
-    for (auto &kv : vb) {
-        dco_status st = launch_items(h, s, "k_vvote", k_vagg<1, true>, k_vagg<kVBatch, true>, kv.second,
-                                     kv.first * 32, vsm[kv.first]);
-        if (st != DCO_OK) return st;
-    }
-    return DCO_OK;
+    return launch_items(h, s, "k_vvote", k_vagg<1, true, false, false>, k_vagg<kBatchMax, true, false, false>, vb, kVThreads,
+                        vsm);
 }
 
-// p.vote_iters rounds of Eq. 4 on every job's final map (j.out, in place),
-// alternating with the job's second map; arms of the left view in the
-// workspace
+// p.vote_iters rounds of Eq. 4 on every job's final map (j.out, in place).
+// A round's winners stay keys, which the next round reads (alternating
+// between the two views' key arrays, free by then); the last round's become
+// the map.  Arms of the left view in the workspace.
 dco_status run_vote(dco_stereo *h, const dco_params &p, const Derived &dv, std::vector<Job> &jobs, cudaStream_t s)
 {
+    if (p.vote_iters == 0) return DCO_OK;
     int maxpass = 0;
     for (const Job &j : jobs) maxpass = std::max(maxpass, j.L.npass);
     for (int it = 0; it < p.vote_iters; it++) {
         for (Job &j : jobs) {
-            int16_t *tmp = jptr<int16_t>(h, j, j.L.vtmp);
-            j.vsrc = !j.out ? nullptr : (it & 1) ? tmp : j.out;
-            j.vdst = (it & 1) ? j.out : tmp;
+            j.vkeys = it > 0 ? j.vbest : nullptr;
+            j.vbest = j.out ? jptr<unsigned long long>(h, j, j.L.best[it & 1]) : nullptr;
         }
         for (int pass = 0; pass < maxpass; pass++) {
             dco_status st = launch_vote_pass(h, dv, jobs, pass, s);
             if (st != DCO_OK) return st;
         }
     }
-    if (p.vote_iters & 1)
-        for (const Job &j : jobs)
-            if (j.out)
-                DCO_CUDA(h, cudaMemcpyAsync(j.out, jptr<int16_t>(h, j, j.L.vtmp), sizeof(int16_t) * j.W * j.H,
-                                            cudaMemcpyDeviceToDevice, s));
-    return DCO_OK;
+    std::vector<Item<VoteEndArgs>> end;
+    for (const Job &j : jobs) {
+        if (!j.out) continue;
+        Item<VoteEndArgs> it{};
+        it.a.best = j.vbest;
+        it.a.mask = j.out; it.a.out = j.out;
+        it.a.npx = j.W * j.H; it.a.dmin = dv.dmin; it.a.D = dv.dmin + j.D;
+        it.gx = (j.W * j.H + 255) / 256; it.gy = 1; it.gz = 1;
+        end.push_back(it);
+    }
+    return launch_items(h, s, "k_vote_end", k_vote_end<1>, k_vote_end<kBatchMax>, end, 256, 0);
 }
 
 // every stage of the path for planned jobs (workspace and tables ready)
@@ -2275,25 +2349,26 @@ dco_status launch_jobs(dco_stereo *h, const dco_params &p, const Derived &dv, st
                        cudaStream_t s)
 {
     int maxpass = 0;
-    for (Job &j : jobs) {
-        if (!j.disp_l) j.disp_l = jptr<int16_t>(h, j, j.L.disp[0]);
-        if (!j.disp_r) j.disp_r = jptr<int16_t>(h, j, j.L.disp[1]);
-        maxpass = std::max(maxpass, j.L.npass);
-    }
+    for (const Job &j : jobs) maxpass = std::max(maxpass, j.L.npass);
     dco_status st;
     if ((st = launch_prep(h, p, dv, jobs, 2, s)) != DCO_OK) return st;
     for (int pass = 0; pass < maxpass; pass++)
         if ((st = launch_pass(h, dv, jobs, pass, s)) != DCO_OK) return st;
-    std::vector<Item<LrArgs>> lr;
+    std::vector<Item<EndArgs>> end;
     for (const Job &j : jobs) {
-        if (!j.out) continue;
-        Item<LrArgs> it{};
-        it.a.dl = j.disp_l; it.a.dr = j.disp_r; it.a.out = j.out;
-        it.a.W = j.W; it.a.H = j.H; it.a.tol = p.lr_tol;
+        if (!j.out && !j.disp_l && !j.disp_r && !j.cost_l && !j.cost_r) continue;
+        Item<EndArgs> it{};
+        for (int v = 0; v < 2; v++) {
+            it.a.best[v] = jptr<unsigned long long>(h, j, j.L.best[v]);
+            it.a.arms[v] = jptr<uchar4>(h, j, j.L.arms[v]);
+        }
+        it.a.disp[0] = j.disp_l; it.a.disp[1] = j.disp_r; it.a.out = j.out;
+        it.a.cost[0] = j.cost_l; it.a.cost[1] = j.cost_r;
+        it.a.W = j.W; it.a.H = j.H; it.a.tol = p.lr_tol; it.a.order = dv.order; it.a.S = dv.S;
         it.gx = (j.W * j.H + 255) / 256; it.gy = 1; it.gz = 1;
-        lr.push_back(it);
+        end.push_back(it);
     }
-    if ((st = launch_lr(h, lr, s)) != DCO_OK) return st;
+    if ((st = launch_items(h, s, "k_end", k_end<1>, k_end<kBatchMax>, end, 256, 0)) != DCO_OK) return st;
     return p.vote_iters > 0 ? run_vote(h, p, dv, jobs, s) : DCO_OK;
 }
 
@@ -2429,6 +2504,7 @@ dco_status dco_stereo_create(dco_stereo **out, int device, size_t workspace_budg
     h->device = device;
     h->budget = workspace_budget_bytes;
     cudaError_t e = cudaSetDevice(device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaMalloc((void **)&h->d_status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void **)&h->d_tables, sizeof(float) * kTabFloats);

@@ -9,7 +9,8 @@
 //   arms[i]  uchar4 {left, right, up, down}
 //   sh[i*dstride + j]  uint32 horizontal segment sum (fixed point) of
 //                    disparity d0 + j (one pass of the d range)
-//   best[i]  uint64 (aggregate << 32 | d), WTA state carried across passes
+//   best[i]  uint64 (aggregate << 32 | d), the WTA's running minimum over the
+//            disparity groups and passes
 //
 // Costs are carried in unsigned fixed point with scale S (an integer below
 // 2^20, chosen so a full (2*L1+1)^2 region of costs <= 1 stays below 2^32).
@@ -18,7 +19,6 @@
 // rounded per-pixel costs; only the Eq. 1 evaluation (FP32) and the rounding
 // to fixed point differ from the real-valued definition.
 #pragma once
-#include <cuda.h>   // CUtensorMap (the encoder is reached through the runtime)
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -44,12 +44,11 @@ constexpr int kRPad = 256;
 // The cost H pass gives each warp kHSegCost columns of the prefix range (two
 // half-warp segments of 16; one chunk per row up to kHMaxLen columns, else
 // 512-column chunks), k_vcost each warp kHSegCost rows, the vote H pass
-// segments of kHSeg; the V pass rows in segments of 1 << seglog.
+// segments of kHSeg.
 constexpr int kHSegLog = 6, kHSeg = 1 << kHSegLog;
 constexpr int kHSegCost = 32;
 constexpr int kHNarrow = 20;     // warps of the cost H instantiation kept at two blocks per SM
 constexpr int kHMaxLen = 1024;   // prefix columns one H block holds
-constexpr int kVMaxLen = 1024;   // prefix rows one V block holds
 
 struct PackArgs {
     const uint8_t *rgb[2];
@@ -83,6 +82,7 @@ struct HArgs {
     int skip_copy;         // failure test: arm the staging barrier but issue no copy
     const uchar4 *arms[2];
     uint32_t *sh[2];
+    unsigned long long *init[2];   // first pass: keys to set to the maximum (null: none)
     const float *tables;
     int W, H, D, rpitch;
     int d0, dc;            // this pass covers d in [d0, d0 + dc)
@@ -96,7 +96,10 @@ struct HArgs {
 
 // horizontal pass of the parallax optimisation (Eq. 4): per-d vote counts
 struct HVArgs {
-    const int16_t *disp;   // map voted on, W x H, -1 = invalid
+    const int16_t *disp;   // map of the first round, W x H; outside [dmin, D) = invalid
+    const unsigned long long *keys;   // later rounds: the previous round's keys (d in the low word)
+    unsigned long long *init;         // first pass: keys to set to the maximum (null: none)
+    int dmin, D;
     const uchar4 *arms;    // reference-view arms {l, r, u, d}
     uint32_t *sh;          // count slices [y][x][dstride]
     int W, H, d0, dstride, L1, chunk;
@@ -128,30 +131,41 @@ struct SmoothArgs {
 };
 
 struct VArgs {
-    // per view: the slice as a TMA tile map (dims: disparity within the
-    // group, group, x, y; box: the group's 32 disparities plus 4 zero-filled
-    // words, of 32 consecutive scan positions)
-    CUtensorMap tm[2];
-    const uint32_t *sh[2];
+    const uint32_t *sh[2];        // slices, dstride words per pixel
     const uchar4 *arms[2];
-    unsigned long long *best[2];
-    int16_t *disp[2];
-    float *cost[2];
+    unsigned long long *best[2];  // (aggregate << 32 | d) per pixel, minimised over every pass and group
     float *vol;            // optional (D, H, W) normalised costs of view `vol_view`
-    const int16_t *mask;   // optional: pixels where mask < 0 are written as -1 (vote)
-    int *status;           // device status word (a lost tile copy sets a bit)
-    int wait_limit;        // mbarrier polls before a tile copy is declared lost
-    int skip_copy;         // failure test: arm each tile's barrier but issue no copy
-    int tm_rank;           // 4: tm as above; 3: dims (disparity, x, y), box 36 x 1 x 32 at (32 g, x, y)
     int vol_view;
     int W, H, D;           // D: one past the largest disparity of the search (d_min + count)
     int dmin;              // smallest disparity of the search
-    int d0, dc, dstride;
-    int first, last;       // first / last pass of the d range
+    int d0, dc, dstride;   // this pass covers d in [d0, d0 + dc)
+    int ng;                // 32-disparity groups in the pass
+    int single;            // the only pass and group: keys are stored, not minimised
     int L1;
-    int chunk;             // output rows per block
-    int seglog;            // rows per warp segment = 1 << seglog
+    int strips;            // strips of four columns per layer (group and view)
+    int nblk, rounds;      // blocks; whole strips per block
+    int rest, share, bands;   // strips left over, rows of them per block, blocks per strip (0: shares run on)
     float S;
+};
+
+// the per-pixel end of a match: keys -> disparities and costs of both views,
+// left-right consistency -> disparity map (every output optional)
+struct EndArgs {
+    const unsigned long long *best[2];
+    const uchar4 *arms[2];
+    int16_t *disp[2], *out;
+    float *cost[2];
+    int W, H, tol, order;
+    float S;
+};
+
+// the end of the Eq. 4 rounds: keys -> map; pixels of `mask` outside the
+// range cast no vote and stay invalid
+struct VoteEndArgs {
+    const unsigned long long *best;
+    const int16_t *mask;
+    int16_t *out;
+    int npx, dmin, D;
 };
 
 struct LrArgs {
