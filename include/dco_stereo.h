@@ -137,8 +137,8 @@ void dco_stereo_destroy(dco_stereo *h);
 
 /*
  * Device bytes of workspace one match of a W x H pair with D disparities
- * needs under params p (0 if the arguments are invalid).  Per pixel: two
- * 16-byte census/colour records, two arm words, the best cost and
+ * needs under params p (0 if the arguments are invalid).  Per pixel: the
+ * census and colour of both images, two arm words, the best cost and
  * disparity of both views so far; per pixel and per disparity of one pass: the
  * two horizontal-aggregate slices (4 bytes each).  Never the full
  * W x H x D cost volume.
@@ -159,9 +159,10 @@ dco_status dco_stereo_reserve(dco_stereo *h, int W, int H, int D, const dco_para
  * The disparity range is processed in passes of p->d_chunk disparities
  * (automatic when 0) so the workspace holds slices, never the volume.
  * Tile shapes (they change the speed, never the result): the first 1-D
- * pass (rows for agg_order 0, columns for 1) splits each line into blocks
- * of p->h_chunk outputs (0: whole lines up to 1024 positions, else 512;
- * otherwise 32 <= h_chunk, capped at 1024 - 2 arm_l1 below the line); the second
+ * pass (rows for agg_order 0, columns for 1) splits each line into ranges
+ * of p->h_chunk outputs (0: whole rows up to 640 positions, whole columns up to
+ * 1024, else ranges that fill a block; otherwise 32 <= h_chunk, capped at what
+ * a block holds with its arm_l1 positions of halo); the second
  * pass walks each line in balanced runs of at most p->v_chunk outputs
  * (0: dealt out evenly to the device; otherwise 32 <= v_chunk).  Each block
  * reads arm_l1 positions of halo on both sides.

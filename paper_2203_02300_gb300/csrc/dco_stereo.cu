@@ -8,11 +8,11 @@
 //   k_pack   RGB -> packed colour words (with the two edge bits of the arm
 //            rule's predecessor test) and the grey level, both images
 //   k_prep   census (shared-memory grey tile) + the four arms (walks over the
-//            packed colours) -> 16-byte records + arm words
+//            packed colours) -> census and colour planes + arm words
 //   per pass of dc disparities:
 //     k_hagg  Eq. 1 cost in fixed point for every (column, disparity) of a
-//             row, prefixes over 16-column segments in shared memory, and
-//             the horizontal segment sum of every pixel -> sh slice
+//             row, their row prefixes in shared memory, and the horizontal
+//             segment sum of every pixel -> sh slices
 //     k_vagg  column prefix of the sh slice, the vertical sum over the
 //             up/down arms (Eq. 2) and the minimum over the disparities
 //             (Eq. 3), merged into one key per pixel
@@ -28,7 +28,7 @@
 #include "dco_stereo.h"
 
 #include <algorithm>
-#include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -420,11 +420,8 @@ __device__ __forceinline__ void prep_body(const PrepArgs &a, int bx, int by, int
         arm[e] = n;
     }
     const int lmin = min(min(arm[0], arm[1]), min(arm[2], arm[3]));
-    const float alphaS = __ldg(a.tables + kTabAD + kTabCen + lmin);
     const uint32_t colour = unspread10(p) | (uint32_t(lmin) << 24);
-    (img ? a.rec[1] : a.rec[0])[(size_t)y * a.rpitch + x] =
-        make_uint4((uint32_t)bits, (uint32_t)(bits >> 32), colour, __float_as_uint(alphaS));
-    const size_t pe = (size_t)y * 2 * a.phw + (size_t)(x & 1) * a.phw + (x >> 1);
+    const size_t pe = (size_t)y * a.pw + x;
     (img ? a.cen[1] : a.cen[0])[pe] = make_uint2((uint32_t)bits, (uint32_t)(bits >> 32));
     (img ? a.col[1] : a.col[0])[pe] = colour;
     (img ? a.arms[1] : a.arms[0])[i] = make_uchar4((uint8_t)arm[0], (uint8_t)arm[1], (uint8_t)arm[2], (uint8_t)arm[3]);
@@ -435,7 +432,7 @@ __device__ __forceinline__ void prep_body(const PrepArgs &a, int bx, int by, int
 // opening of each arm map is a 3x3 minimum (kMax = false) followed by a 3x3
 // maximum (kMax = true), windows cut to the image.  An opening never
 // lengthens an arm, so arms stay inside the image and <= L1.  The maximum
-// pass also rewrites the record's L_min and alpha(L_min)*S (Eq. 1).
+// pass also rewrites the colour word's L_min (Eq. 1's weight).
 template <bool kMax>
 __device__ __forceinline__ void smooth_body(const SmoothArgs &a, int i, int img)
 {
@@ -451,35 +448,14 @@ __device__ __forceinline__ void smooth_body(const SmoothArgs &a, int i, int img)
             for (int k = 0; k < 4; k++) v[k] = kMax ? max(v[k], c[k]) : min(v[k], c[k]);
         }
     (img ? a.dst[1] : a.dst[0])[i] = make_uchar4((uint8_t)v[0], (uint8_t)v[1], (uint8_t)v[2], (uint8_t)v[3]);
-    uint4 *rec = img ? a.rec[1] : a.rec[0];
-    if (kMax && rec) {
+    if (kMax) {
         const int lmin = min(min(v[0], v[1]), min(v[2], v[3]));
-        uint4 *r = rec + (size_t)y * a.rpitch + x;
-        r->z = (r->z & 0x00ffffffu) | (uint32_t(lmin) << 24);
-        r->w = __float_as_uint(__ldg(a.tables + kTabAD + kTabCen + lmin));
+        uint32_t *c = (img ? a.col[1] : a.col[0]) + (size_t)y * a.pw + x;
+        *c = (*c & 0x00ffffffu) | (uint32_t(lmin) << 24);
     }
 }
 
-// ------------------------------------------------------------------ k_hagg
-// Block = one row segment of one reference view for one group of 32
-// disparities.  Stage 0 copies (cp.async) the tables, the reference records
-// of the prefix range [xa, xb) (the output columns plus an L1 reach on both
-// sides), the candidate records of the whole group (census and colour apart,
-// even and odd candidate indices apart) and the output columns' arms into
-// shared memory.  Then:
-//   A. each half-warp walks a segment of 16 columns; lane j of the half holds
-//      the disparity pair (dlo + 2j, dlo + 2j + 1): Eq. 1 costs rounded to
-//      fixed point, local inclusive prefixes into P[x - xa][d - dlo].  The
-//      candidate of d + 1 at column x + 1 is the candidate of d at x (the
-//      other way round in the right-reference view), so each column step
-//      loads one new candidate record for two evaluations;
-//   B. the exclusive prefix of the segment totals (segment offsets);
-//   C. every output column xo: S_H = F(xo + r) - F(xo - l - 1) (the
-//      horizontal part of Eq. 2), F the row prefix: the difference of the
-//      local prefixes plus the difference of their segments' offsets.
-// Unsigned wrap-around makes the differences exact segment sums.
-constexpr int kTabBytes = (kTabAD + kTabCen) * 4;
-
+// ------------------------------------------------------------ copies, waits
 __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 {
     const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
@@ -536,31 +512,304 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t n,
                  : "memory");
 }
 
-// byte offsets of the H block's shared-memory regions.  Candidate indices
-// run over [0, len + 31); index i sits at position i >> 1 of the even (i & 1
-// = 0) or odd array, hh positions each.  The arrays arrive by bulk copies
-// that start on 16-byte boundaries of the candidate planes, so each half has
-// room for the alignment shift: census halves hhc entries (up to one more
-// than hh, even), colour halves hhk (up to three more, a multiple of 4), the
-// arms up to three entries more.
-struct HSmem {
-    int ref, oth, hh, hhc, hhk, col, arm, p, t, total;
-    __host__ __device__ HSmem(int len, int chunk, int nw)
-    {
-        ref = kTabBytes;
-        oth = ref + len * 16;                   // census: uint2 [2][hhc]; then the segment offsets
-        hh = (len + 33) / 2;
-        hhc = (hh + 3) & ~1;
-        hhk = (hh + 9) & ~3;
-        col = oth + hhc * 16;                   // colour: uint32 [2][hhk]
-        arm = col + hhk * 8;
-        p = arm + ((chunk + 9) & ~3) * 4 + 128; // one zero row in front: P[-1]
-        t = p + len * 128;
-        total = t + 2 * nw * 128;               // segment totals [2 nw][32]
-    }
+// ------------------------------------------------------------------ k_hagg
+// Eq. 1 costs and their horizontal segment sums (the first 1-D sum of Eq. 2).
+// Block = (row, view, 32 disparities, a range of columns), sixteen warps: warp
+// = (four disparities, half of the range).  The records of both images, the
+// arms and the tables arrive in shared memory by bulk copies on one mbarrier
+// (bounded wait).  Then:
+//   A. a warp walks its half in segments of 160 columns (a short end in one of
+//      32), lane = five (one)
+//      consecutive columns x four disparities: the reference records stay in
+//      registers and each candidate loaded serves up to four costs; costs
+//      rounded to fixed point, prefixes within the lane, a scan of the lanes'
+//      totals, and the prefixes stored as one 16-byte word per column
+//      (G[quad][x], lanes five words apart: no bank conflicts);
+//   B. every output column: S_H = G(end) - G(start), eight lanes (quads) per
+//      column, a 128-byte line of the slice per column; the planes' stride
+//      puts the eight quads of a column on distinct banks whatever the arms.
+// Bound by the shared-memory data path (15 M wavefronts at 640x480, D = 64, 87 %
+// of the L1 throughput, a third of them the table gathers of Eq. 1).  Against
+// one block per task with a disparity pair per lane and sixteen-column
+// segments: 45 M instead of 52 M instructions; 640x480, D = 64, one pass 70 -> 66
+// us (the default was two passes: 82), 1280x720, D = 128 481 -> 423 us,
+// 1920x1080, D = 256 1960 -> 1875 us; rows that fill their segments badly lose
+// (333x211, D = 50 22.3 -> 23.8 us).  Both views in one block from one
+// evaluation of every pixel pair (16 disparities, 96 registers, one set of
+// table gathers for two costs) took 72-75 us: 13.5 M wavefronts, but sixteen
+// warps per SM, and right-view windows that move with the disparity.
+constexpr int kHD = 32;        // disparities per block
+constexpr int kHQuads = kHD / 4;
+constexpr int kHWarps = 2 * kHQuads;
+constexpr int kHCols = 5;      // columns per lane (odd: conflict-free stores)
+constexpr int kHSegCols = 32 * kHCols;
+constexpr int kHScan = 40;     // words per value of the scan of the lanes' totals (eight lanes' 16-byte reads hit distinct banks)
+constexpr int kHMaxPairs = 4 * kHSegCols;   // reference columns per block (two blocks per SM)
+constexpr int kHPlane = kHMaxPairs + 1;     // 16-byte words per plane: odd
+constexpr int kTabBytes = kTabFloats * 4;
+
+// Byte offsets of the block's shared memory (the same for every launch): each
+// copied range has room for its 16-byte alignment; the arms of two tasks.
+namespace hsm {
+constexpr int e = kHMaxPairs + 4, f = kHMaxPairs + kHD + 4;   // reference and candidate columns
+// (a second copy of the AD table for every other lane: 67.7 against 65.8 us at
+// 640x480, D = 64: neighbouring columns often read the same entry)
+constexpr int rcen = kTabBytes, ccen = rcen + 8 * e, rcol = ccen + 8 * f, ccol = rcol + 4 * e;
+constexpr int arm = ccol + 4 * f, arms = 4 * e, g = arm + 2 * arms;
+constexpr int total = g + kHQuads * kHPlane * 16;
+}   // namespace hsm
+
+// one unit of a block's work: a range of output columns of a row, view and group
+struct HTask {
+    int live;
+    int W, p0, n, q0, nq;      // reference columns p0 .. p0 + n - 1, candidates q0 .. q0 + nq - 1
+    int m, lead;               // output columns, the first at relative column `lead`
+    int view, dlo, dend, arm;  // arm: entries before the first output's arm word in the copy
+    float S;
+    uint32_t Sint;
+    size_t ds4;                // slice words of a pixel / 4
+    uint4 *out;                // slice of the first output column, this group
+    unsigned long long *init;  // keys to set (null: none)
 };
 
-// Phase C of a horizontal pass: every output column c (n_out of them,
+// Blocks are resident (two per SM) and take tasks in turn: the next task's
+// copies are in flight during phase B, which does not read the records.
+// find(t, bx, by, bz): the arguments of task t and its place in their grid.
+template <class Find>
+__device__ __forceinline__ void hagg_tasks(int ntasks, Find find)
+{
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    __shared__ __align__(8) unsigned long long hbar_s;
+    __shared__ HTask task_s[2];
+    __shared__ uint4 half_s[kHQuads];   // totals of the first half
+    __shared__ int lost_s;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&hbar_s);
+    const float *sTC = reinterpret_cast<const float *>(smem_raw) + kTabAD, *sAl = sTC + kTabCen;
+
+    // thread 0: task t's description, and its copies.  Each starts on the
+    // 16-byte boundary at or below its first entry and ends on the one at or
+    // above its last.
+    auto prepare = [&](int t, int slot) {
+        HTask k;
+        k.live = t < ntasks;
+        if (!k.live) {
+            task_s[slot].live = 0;
+            return;
+        }
+        int y, part, bz;   // rows first, then ranges: the short last ranges come last
+        const HArgs &a = find(t, y, part, bz);
+        const int W = a.W, L1 = a.L1, xs = part ? a.first + (part - 1) * a.chunk : 0;
+        const int xe = min(W, part ? xs + a.chunk : a.first);
+        const int view = bz / a.ngroups, g32 = bz - view * a.ngroups, dlo = a.d0 + kHD * g32;
+        const int p0 = max(0, xs - L1), pe = min(W, xe + L1);
+        const int q0 = max(0, min(W, view ? p0 + dlo : p0 - dlo - (kHD - 1)));
+        const int q1 = max(q0, min(W, view ? pe + dlo + kHD - 1 : pe - dlo));
+        const size_t row = (size_t)y * a.pw, arow = (size_t)y * W, ga = (arow + xs) & ~(size_t)3;
+        k.W = W;
+        k.p0 = p0;
+        k.n = pe - p0;
+        k.q0 = q0;
+        k.nq = q1 - q0;
+        k.m = xe - xs;
+        k.lead = xs - p0;
+        k.view = view;
+        k.dlo = dlo;
+        k.dend = min(a.d0 + a.dc, a.D);
+        k.arm = (int)(arow + xs - ga);
+        k.S = a.S;
+        k.Sint = a.Sint;
+        k.ds4 = (size_t)a.dstride / 4;
+        k.out = reinterpret_cast<uint4 *>((view ? a.sh[1] : a.sh[0]) + (arow + xs) * a.dstride + kHD * g32);
+        unsigned long long *init = view ? a.init[1] : a.init[0];
+        k.init = init && g32 == 0 ? init + arow + xs : nullptr;
+        task_s[slot] = k;
+        auto bytes = [](int x0, int x1, int size) -> uint32_t {   // of entries [x0, x1) from the boundary below x0
+            const int per = 16 / size;
+            return x1 > x0 ? (uint32_t)((x1 - (x0 & ~(per - 1)) + per - 1) & ~(per - 1)) * size : 0u;
+        };
+        const uint32_t nrc = bytes(p0, pe, 8), ncc = bytes(q0, q1, 8), nrk = bytes(p0, pe, 4), nck = bytes(q0, q1, 4);
+        const uint32_t na = 4u * ((uint32_t)(arow + xe - ga + 3) & ~3u);
+        mbar_expect_tx(bar, nrc + ncc + nrk + nck + na);
+        if (a.skip_copy) return;   // (the failure test arms the barrier and issues nothing)
+        const uint2 *cr = view ? a.cen[1] : a.cen[0], *cc = view ? a.cen[0] : a.cen[1];
+        const uint32_t *kr = view ? a.col[1] : a.col[0], *kc = view ? a.col[0] : a.col[1];
+        bulk_g2s(smem_raw + hsm::rcen, cr + row + (p0 & ~1), nrc, bar);
+        bulk_g2s(smem_raw + hsm::rcol, kr + row + (p0 & ~3), nrk, bar);
+        if (ncc) bulk_g2s(smem_raw + hsm::ccen, cc + row + (q0 & ~1), ncc, bar);
+        if (nck) bulk_g2s(smem_raw + hsm::ccol, kc + row + (q0 & ~3), nck, bar);
+        bulk_g2s(smem_raw + hsm::arm + slot * hsm::arms, (view ? a.arms[1] : a.arms[0]) + ga, na, bar);
+    };
+    int next = blockIdx.x;
+    if (threadIdx.x == 0) {
+        mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        lost_s = 0;
+        prepare(next, 0);
+    }
+    if (next < ntasks) {
+        int bx, by, bz;
+        const float *tables = find(next, bx, by, bz).tables;   // (one set per handle: the same for every task)
+        for (int i = threadIdx.x; i < kTabFloats; i += blockDim.x) reinterpret_cast<float *>(smem_raw)[i] = __ldg(tables + i);
+    }
+    for (int it = 0;; it++) {
+        const int slot = it & 1;
+        if (threadIdx.x == 0 && task_s[slot].live) {
+            int bx, by, bz;
+            const HArgs &a = find(next, bx, by, bz);
+            if (!mbar_wait(bar, (uint32_t)slot, a.wait_limit)) {
+                // report, and wait (bounded) once more before the block's shared memory is released
+                if (a.status) atomicOr(a.status, kStatusCopyTimeout);
+                mbar_wait(bar, (uint32_t)slot, a.wait_limit);
+                lost_s = 1;
+            }
+        }
+        __syncthreads();   // (also: the last task's outputs have been read from G)
+        const HTask &k = task_s[slot];
+        if (!k.live || lost_s) return;
+        if (unsigned long long *init = k.init)   // the keys the V pass minimises into
+            for (int i = threadIdx.x; i < k.m; i += blockDim.x) init[i] = ~0ull;
+
+        // ---- A: prefixes of the warp's quad over its half of the columns
+        const int n = k.n, view = k.view;
+        // first column of the second half: whole segments, of which an end of
+        // at most 32 columns does not count
+        const int nseg = max(1, (n + kHSegCols - 33) / kHSegCols), split = min(n, (nseg + 1) / 2 * kHSegCols);
+        {
+            const int quad = warp & (kHQuads - 1), half = warp / kHQuads, d0 = k.dlo + 4 * quad;
+            const int W = k.W, p0 = k.p0, q0 = k.q0, nq = k.nq;
+            const uint2 *rcen = reinterpret_cast<const uint2 *>(smem_raw + hsm::rcen) + (p0 & 1);
+            const uint32_t *rcol = reinterpret_cast<const uint32_t *>(smem_raw + hsm::rcol) + (p0 & 3);
+            // indexed by candidate column - q0
+            const uint2 *ccen = reinterpret_cast<const uint2 *>(smem_raw + hsm::ccen) + (q0 & 1);
+            const uint32_t *ccol = reinterpret_cast<const uint32_t *>(smem_raw + hsm::ccol) + (q0 & 3);
+            uint4 *g = reinterpret_cast<uint4 *>(smem_raw + hsm::g) + quad * kHPlane;
+            const float S = k.S;
+            const uint32_t one = k.Sint;
+            // Cost j of column c meets candidate c + 3 - j of the lane's eight:
+            // disparity d0 + j in the left view, d0 + 3 - j in the right one.
+            const int cand = view ? p0 + d0 - q0 : p0 - d0 - 3 - q0;   // of relative column 0, relative to q0
+            uint32_t carry = 0;   // of cost lane & 3: the prefix before the segment
+            // columns s .. s + 159 (relative); kEdge: some lie past the range, or
+            // meet candidates outside the image
+            auto segment = [&](int s, auto cols_c, auto edge_c) {
+                constexpr int kCols = decltype(cols_c)::value;
+                constexpr bool kEdge = decltype(edge_c)::value;
+                const int x = s + kCols * lane;   // the lane's first column
+                uint32_t lo[kCols], hi[kCols], rgb[kCols];
+                float av[kCols];
+#pragma unroll
+                for (int c = 0; c < kCols; c++) {
+                    const int i = kEdge ? min(x + c, n - 1) : x + c;
+                    const uint2 ce = rcen[i];
+                    lo[c] = ce.x;
+                    hi[c] = ce.y;
+                    rgb[c] = rcol[i];
+                    av[c] = sAl[rgb[c] >> 24];
+                }
+                // c - j of the costs inside the image: [first, last)
+                const int first = view ? -4 : d0 - p0 - x, last = view ? W - p0 - x - d0 - 3 : kCols;
+                uint32_t pl[kCols][4];   // prefixes within the lane
+#pragma unroll
+                for (int i = 0; i < kCols + 3; i++) {
+                    const int r = kEdge ? max(0, min(cand + x + i, nq - 1)) : cand + x + i;
+                    const uint2 ce = ccen[r];
+                    const uint32_t rc = ccol[r];
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const int c = i - 3 + j;
+                        if (c < 0 || c >= kCols) continue;   // (resolved at compile time)
+                        const int h = __popc(lo[c] ^ ce.x) + __popc(hi[c] ^ ce.y);
+                        const uint32_t k4 = __dp4a(__vabsdiffu4(rgb[c], rc), 0x00040404u, 0u);   // byte offset
+                        const float ta = *reinterpret_cast<const float *>(smem_raw + k4), tc = sTC[h];
+                        uint32_t q = __float2uint_rn(fmaf(av[c], ta, (S - av[c]) * tc));
+                        if (kEdge && (c - j < first || c - j >= last)) q = one;   // match outside the image: cost 1
+                        pl[c][j] = c ? pl[c ? c - 1 : 0][j] + q : q;
+                    }
+                }
+                // offsets of the lanes: exclusive scan of their four totals, by way
+                // of shared memory (the segment's own columns of G, not yet
+                // written): lane = (value, four lanes' worth of it)
+                uint32_t *scan = reinterpret_cast<uint32_t *>(g + s + 1);
+#pragma unroll
+                for (int j = 0; j < 4; j++) scan[j * kHScan + lane] = pl[kCols - 1][j];
+                __syncwarp();
+                uint4 *mine = reinterpret_cast<uint4 *>(scan + (lane & 3) * kHScan + (lane >> 2) * 4);
+                const uint4 t = *mine;
+                const uint32_t a2 = t.x + t.y, a3 = a2 + t.z, a4 = a3 + t.w;
+                uint32_t incl = a4;
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) {
+                    const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += u;
+                }
+                const uint32_t before = carry + incl - a4;
+                *mine = make_uint4(before, before + t.x, before + a2, before + a3);
+                carry += __shfl_sync(0xffffffffu, incl, 28 + (lane & 3));
+                __syncwarp();
+                uint32_t off[4];
+#pragma unroll
+                for (int j = 0; j < 4; j++) off[j] = scan[j * kHScan + lane];
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < kCols; c++) {
+                    if (kEdge && x + c >= n) break;
+                    const uint4 v = make_uint4(pl[c][0] + off[0], pl[c][1] + off[1], pl[c][2] + off[2], pl[c][3] + off[3]);
+                    g[x + c + 1] = view ? make_uint4(v.w, v.z, v.y, v.x) : v;
+                }
+            };
+            if (d0 < k.dend) {
+                const int s1 = half ? n : split;
+                for (int s = half ? split : 0; s < s1; s += kHSegCols) {
+                    const bool inside = view ? p0 + s + kHSegCols + d0 + 3 <= W : p0 + s >= d0 + 3;
+                    if (s1 - s <= 32) segment(s, std::integral_constant<int, 1>{}, std::true_type{});
+                    else if (inside && s + kHSegCols <= n) segment(s, std::integral_constant<int, kHCols>{}, std::false_type{});
+                    else segment(s, std::integral_constant<int, kHCols>{}, std::true_type{});
+                }
+                if (half == 0) {
+                    if (lane == 0) g[0] = make_uint4(0u, 0u, 0u, 0u);
+                    if (lane < 4) reinterpret_cast<uint32_t *>(&half_s[quad])[view ? 3 - lane : lane] = carry;
+                }
+            }
+        }
+        __syncthreads();
+        next += gridDim.x;
+        if (threadIdx.x == 0) prepare(next, slot ^ 1);
+
+        // ---- B: segment sums; lane = (column, quad)
+        const int quad = lane & (kHQuads - 1), c0 = 32 / kHQuads * warp;
+        if (k.dlo + 4 * quad < k.dend) {
+            constexpr int kStep = kHWarps * 32 / kHQuads;
+            const int lead = k.lead, cross = split - lead, m = k.m, col = lane / kHQuads;
+            const uint4 *g = reinterpret_cast<const uint4 *>(smem_raw + hsm::g) + quad * kHPlane + lead + col;
+            const uchar4 *arm = reinterpret_cast<const uchar4 *>(smem_raw + hsm::arm + slot * hsm::arms) + k.arm + col;
+            const size_t ds4 = k.ds4, ostep = kStep * ds4;
+            uint4 *o = k.out + (c0 + col) * ds4 + quad;
+            const uint4 tot = half_s[quad];
+            // columns i + col
+            auto sum = [&](int i) {
+                const uchar4 am = arm[i];
+                const int hi = i + am.y + 1, lo = i - am.x;
+                const uint4 h = g[hi], w = g[lo];
+                uint4 v = make_uint4(h.x - w.x, h.y - w.y, h.z - w.z, h.w - w.w);
+                if (i + kMaxL1 + 4 > cross && i - kMaxL1 <= cross) {   // near the halves' border (the same in the warp)
+                    if (hi + col > cross && lo + col <= cross) v = make_uint4(v.x + tot.x, v.y + tot.y, v.z + tot.z, v.w + tot.w);
+                }
+                return v;
+            };
+            int i = c0;
+            for (; i + kStep + 3 < m; i += 2 * kStep, o += 2 * ostep) {
+                const uint4 v0 = sum(i), v1 = sum(i + kStep);
+                o[0] = v0;
+                o[ostep] = v1;
+            }
+            for (; i + col < m; i += kStep, o += ostep) o[0] = sum(i);
+        }
+    }
+}
+
+// The output phase of a pass whose lanes hold one disparity each (k_vcost):
+// every output position c (n_out of them,
 // prefix index base + c): S_H = F(c + r) - F(c - l - 1), F the prefix of the
 // costs along the scan.  P holds prefixes local to segments of 1 << kSegLog
 // positions and OFF the exclusive prefix of the segment totals, so
@@ -604,7 +853,7 @@ __device__ __forceinline__ void hagg_out_quads(const uint32_t *P, const uint32_t
     if (i < n_out) o4[(size_t)i * ds4] = column(i);
 }
 
-// Phases B and C of a horizontal pass (k_vcost, k_hvote) whose warps each
+// Segment offsets and outputs of a pass (k_vcost) whose warps each
 // scanned one segment of 1 << kSegLog positions: P holds every warp's local
 // inclusive prefix of its segment, T the segment totals (visible after a
 // barrier).
@@ -624,195 +873,13 @@ __device__ __forceinline__ void hagg_tail(const uint32_t *P, uint32_t *T, const 
     hagg_out_quads<kSegLog>(P, T, sarm, n_out, base, o, ds);
 }
 
-// Phase A of k_hagg for one half-warp segment [sa, sb) (relative to xa) of
-// view kView.  Lane j of the half (hl) holds the disparities da = dlo + 2 hl
-// and da + 1, the prefixes run_a, run_b.  The candidate index of the record
-// loaded new at column x is x + nb (odd at even x): view 0 pairs it with da
-// and the previous one with da + 1, view 1 the other way round.  A match
-// outside the image costs 1 (Sint): view 0 needs x >= va / vb, view 1 x < va / vb.
-template <int kView>
-__device__ __forceinline__ void hagg_costs(const uint4 *sref, const uint2 *cenE, const uint2 *cenO,
-                                           const uint32_t *colE, const uint32_t *colO, const float *sTA,
-                                           const float *sTC, uint32_t *P, int sa, int sb, int hl, int va, int vb,
-                                           float Sf, uint32_t Sint, uint32_t &run_a, uint32_t &run_b)
-{
-    const int nb = kView ? 1 + 2 * hl : 31 - 2 * hl;
-    const int p0 = (sa + nb - 1) >> 1;
-    const uint2 *cE = cenE + p0 + 1, *cO = cenO + p0;   // new records at odd / even steps
-    const uint32_t *kE = colE + p0 + 1, *kO = colO + p0;
-    uint2 pc = cenE[p0];
-    uint32_t pk = colE[p0];
-    uint2 *Pp = reinterpret_cast<uint2 *>(P) + hl;
-    auto cost = [&](const uint4 &pr, float av, float sav, uint2 c, uint32_t col) -> uint32_t {
-        const int h = __popc(pr.x ^ c.x) + __popc(pr.y ^ c.y);
-        const int k = (int)__dp4a(__vabsdiffu4(pr.z, col), 0x00010101u, 0u);
-        return __float2uint_rn(fmaf(av, sTA[k], sav * sTC[h]));
-    };
-    auto step = [&](int x, uint2 nc, uint32_t nk) {
-        const uint4 pr = sref[x];
-        const float av = __uint_as_float(pr.w), sav = Sf - av;
-        const uint32_t qa = kView ? cost(pr, av, sav, pc, pk) : cost(pr, av, sav, nc, nk);
-        const uint32_t qb = kView ? cost(pr, av, sav, nc, nk) : cost(pr, av, sav, pc, pk);
-        run_a += (kView ? x < va : x >= va) ? qa : Sint;
-        run_b += (kView ? x < vb : x >= vb) ? qb : Sint;
-        Pp[x * 16] = make_uint2(run_a, run_b);
-        pc = nc;
-        pk = nk;
-    };
-    if (sb - sa == 16) {
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-            step(sa + 2 * k, cO[k], kO[k]);
-            step(sa + 2 * k + 1, cE[k], kE[k]);
-        }
-    } else {
-        for (int k = 0; sa + 2 * k < sb; k++) {
-            step(sa + 2 * k, cO[k], kO[k]);
-            if (sa + 2 * k + 1 < sb) step(sa + 2 * k + 1, cE[k], kE[k]);
-        }
-    }
-}
-
-__device__ __forceinline__ void hagg_body(const HArgs &a, int bx, int by, int bz)
-{
-    extern __shared__ __align__(16) uint8_t smem_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int W = a.W, L1 = a.L1;
-    const int y = by;
-    const int view = bz / a.ngroups, g = bz % a.ngroups;
-    const int xs = bx * a.chunk, xe = min(W, xs + a.chunk);
-    const int xa = max(0, xs - L1), xb = min(W, xe + L1), len = xb - xa;
-    const HSmem L(len, a.chunk, nw);
-    float *sTA = reinterpret_cast<float *>(smem_raw);
-    float *sTC = sTA + kTabAD;
-    uint4 *sref = reinterpret_cast<uint4 *>(smem_raw + L.ref);
-    uint2 *scen = reinterpret_cast<uint2 *>(smem_raw + L.oth);       // candidate census [2][hhc]
-    uint32_t *scol = reinterpret_cast<uint32_t *>(smem_raw + L.col); // candidate colour + Lmin [2][hhk]
-    uchar4 *sarm = reinterpret_cast<uchar4 *>(smem_raw + L.arm);
-    uint32_t *P = reinterpret_cast<uint32_t *>(smem_raw + L.p);   // [len][32], P[-1] = 0
-    uint32_t *T = reinterpret_cast<uint32_t *>(smem_raw + L.t);   // [2 nw][32]
-    if (threadIdx.x < 32) P[(int)threadIdx.x - 32] = 0u;
-
-    // first disparity of this group
-    const int dlo = a.d0 + 32 * g;
-    // candidate index i <-> column olo + i, i in [0, len + 31): every
-    // disparity of the 32-wide group (the costs of dead disparities are
-    // computed from whatever the shared words hold and never read)
-    const int olo = view ? xa + dlo : xa - dlo - 31;
-    const uint4 *rref = (view ? a.rec[1] : a.rec[0]) + (size_t)y * a.rpitch;
-
-    // ---- 0: stage by bulk copies, issued by one thread on one mbarrier:
-    // the tables, the reference records, the arms and the candidates.  The
-    // even-index candidates i = 2m are the columns olo + 2m, entry
-    // (olo >> 1) + m of one half of the other view's plane row, the odd ones
-    // olo + 1 + 2m of the other half; only the in-image columns are copied
-    // (the others cost 1 whatever they hold).  Each copy starts on the 16-byte
-    // boundary at or below its first entry, and candidate m of a half sits at
-    // shared position o + m, o (0-3) chosen so the copy's destination is
-    // 16-byte aligned too.
-    __shared__ __align__(8) unsigned long long hbar_s;
-    __shared__ int hoff_s[5];   // the halves' shared offsets o, then the lost flag
-    const uint32_t hbar = (uint32_t)__cvta_generic_to_shared(&hbar_s);
-    const size_t ga = (size_t)y * W + xs, gas = ga & ~(size_t)3;
-    if (threadIdx.x == 0) {
-        struct Half {
-            int base, mlo, mhi;   // plane entry of m = 0 (may be negative), in-image m range
-        };
-        auto cand_half = [&](int c0) {   // the candidates c0 + 2m, m < hh
-            Half h;
-            h.base = (c0 & 1) * a.phw + (c0 >> 1);
-            h.mlo = max(0, (1 - c0) >> 1);          // first m with c0 + 2m >= 0
-            h.mhi = min(L.hh, (W - c0 + 1) >> 1);   // first m with c0 + 2m >= W
-            return h;
-        };
-        const Half hE = cand_half(olo), hO = cand_half(olo + 1);
-        // q entries per 16 bytes: the copy starts `shift` entries below the
-        // first in-image one; o makes (o + mlo - shift) a multiple of q
-        auto shift = [](const Half &h, int q) { return h.mlo < h.mhi ? (h.base + h.mlo) & (q - 1) : 0; };
-        auto offs = [&](const Half &h, int q) { return (shift(h, q) - h.mlo) & (q - 1); };
-        auto count = [&](const Half &h, int q) {
-            return h.mlo < h.mhi ? (uint32_t)(h.mhi - h.mlo + shift(h, q) + q - 1) & ~(uint32_t)(q - 1) : 0u;
-        };
-        const uint2 *cpl = (view ? a.cen[0] : a.cen[1]) + (size_t)y * 2 * a.phw;
-        const uint32_t *kpl = (view ? a.col[0] : a.col[1]) + (size_t)y * 2 * a.phw;
-        const uint32_t nA = (uint32_t)(xe - xs + (int)(ga - gas) + 3) & ~3u;
-        const uint32_t nCE = count(hE, 2), nCO = count(hO, 2), nKE = count(hE, 4), nKO = count(hO, 4);
-        const int oCE = offs(hE, 2), oCO = offs(hO, 2), oKE = offs(hE, 4), oKO = offs(hO, 4);
-        mbar_init(hbar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-        mbar_expect_tx(hbar, (uint32_t)kTabBytes + 16u * (uint32_t)len + 8u * (nCE + nCO) + 4u * (nKE + nKO) + 4u * nA);
-        if (!a.skip_copy) {   // (the failure test arms the barrier and issues nothing)
-            bulk_g2s(smem_raw, a.tables, kTabBytes, hbar);
-            bulk_g2s(sref, rref + xa, 16u * (uint32_t)len, hbar);
-            bulk_g2s(sarm, (view ? a.arms[1] : a.arms[0]) + gas, 4u * nA, hbar);
-            if (nCE) bulk_g2s(scen + oCE + hE.mlo - shift(hE, 2), cpl + hE.base + hE.mlo - shift(hE, 2), 8u * nCE, hbar);
-            if (nCO)
-                bulk_g2s(scen + L.hhc + oCO + hO.mlo - shift(hO, 2), cpl + hO.base + hO.mlo - shift(hO, 2), 8u * nCO, hbar);
-            if (nKE) bulk_g2s(scol + oKE + hE.mlo - shift(hE, 4), kpl + hE.base + hE.mlo - shift(hE, 4), 4u * nKE, hbar);
-            if (nKO)
-                bulk_g2s(scol + L.hhk + oKO + hO.mlo - shift(hO, 4), kpl + hO.base + hO.mlo - shift(hO, 4), 4u * nKO, hbar);
-        }
-        hoff_s[0] = oCE;
-        hoff_s[1] = oCO;
-        hoff_s[2] = oKE;
-        hoff_s[3] = oKO;
-        const bool ok = mbar_wait(hbar, 0u, a.wait_limit);
-        if (!ok) {   // report, and wait (bounded) once more before the block's shared memory is released
-            if (a.status) atomicOr(a.status, kStatusCopyTimeout);
-            mbar_wait(hbar, 0u, a.wait_limit);
-        }
-        hoff_s[4] = !ok;
-    }
-    __syncthreads();
-    if (hoff_s[4]) return;
-    const uint2 *cenE = scen + hoff_s[0], *cenO = scen + L.hhc + hoff_s[1];
-    const uint32_t *colE = scol + hoff_s[2], *colO = scol + L.hhk + hoff_s[3];
-    const uchar4 *sarm0 = sarm + (ga - gas);   // arm of output column xs
-    unsigned long long *init = view ? a.init[1] : a.init[0];
-    if (init && g == 0)   // the keys the V pass minimises into
-        for (int i = threadIdx.x; i < xe - xs; i += blockDim.x) init[ga + i] = ~0ull;
-
-    // ---- A: costs and local prefixes of this half-warp's segment
-    const int half = lane >> 4, hl = lane & 15;
-    const int s = 2 * warp + half;
-    const int sa = 16 * s, sb = min(len, sa + 16);
-    const int da = dlo + 2 * hl;
-    // columns x (relative to xa) whose match x -/+ d lies in the image
-    const int va = view ? W - xa - da : da - xa, vb = view ? va - 1 : va + 1;
-    uint32_t run_a = 0, run_b = 0;
-    if (sa < len) {
-        if (view)
-            hagg_costs<1>(sref, cenE, cenO, colE, colO, sTA, sTC, P, sa, sb, hl, va, vb, a.S, a.Sint, run_a, run_b);
-        else
-            hagg_costs<0>(sref, cenE, cenO, colE, colO, sTA, sTC, P, sa, sb, hl, va, vb, a.S, a.Sint, run_a, run_b);
-    }
-    reinterpret_cast<uint2 *>(T + s * 32)[hl] = make_uint2(run_a, run_b);
-    __syncthreads();
-
-    // ---- B: exclusive offsets of the segments holding columns (lane =
-    // disparity), written over the candidate records, which are no longer read
-    uint32_t *OFF = reinterpret_cast<uint32_t *>(smem_raw + L.oth);   // [ceil(len / 16)][32]
-    if (32 * warp < len) {
-        uint32_t offs = 0;
-#pragma unroll 4
-        for (int s2 = 0; s2 < 2 * warp; s2++) offs += T[s2 * 32 + lane];
-        OFF[2 * warp * 32 + lane] = offs;
-        if (32 * warp + 16 < len) OFF[(2 * warp + 1) * 32 + lane] = offs + T[2 * warp * 32 + lane];
-    }
-    __syncthreads();
-
-    // ---- C
-    hagg_out_quads<4>(P, OFF, sarm0, xe - xs, xs - xa,
-                      (view ? a.sh[1] : a.sh[0]) + ((size_t)y * W + xs) * a.dstride + g * 32, a.dstride);
-}
-
 // ---------------------------------------------------------------- k_vcost
 // The other aggregation order, first pass: Eq. 1 costs and their vertical
 // segment sums S_V(q, d) over q's vertical arm.  Block = one column x (a
 // chunk of rows) of one reference view for one group of 32 disparities;
 // lane = disparity.  The reference records of the column are staged in
-// shared memory; the candidates of each row (32 neighbouring records of the
-// other view's row) are read straight from the record rows.  Then the
+// shared memory; the candidates of each row (32 neighbouring pixels of the
+// other view's row) are read straight from the planes.  Then the
 // phases of a horizontal pass along the column: local prefixes over warp
 // segments of 32 rows, segment offsets, segment sums (hagg_tail, with the
 // up / down arms), written to the same slice layout.
@@ -844,8 +911,8 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
     uchar4 *sarm = reinterpret_cast<uchar4 *>(smem_raw + L.arm);   // (up, down) of the output rows
     uint32_t *P = reinterpret_cast<uint32_t *>(smem_raw + L.p);    // [len][32], P[-1] = 0
     uint32_t *T = reinterpret_cast<uint32_t *>(smem_raw + L.t);
-    const uint4 *rref = view ? a.rec[1] : a.rec[0];   // padded rows, pitch rpitch
-    const uint4 *roth = view ? a.rec[0] : a.rec[1];
+    const uint2 *cref = (view ? a.cen[1] : a.cen[0]) + x, *coth = view ? a.cen[0] : a.cen[1];
+    const uint32_t *kref = (view ? a.col[1] : a.col[0]) + x, *koth = view ? a.col[0] : a.col[1];
     const uchar4 *aref = view ? a.arms[1] : a.arms[0];
     unsigned long long *init = view ? a.init[1] : a.init[0];
     if (init && g == 0)   // the keys the second pass minimises into
@@ -853,7 +920,11 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
 
     for (int i = threadIdx.x; i < kTabBytes / 16; i += blockDim.x)
         cp_async16(smem_raw + 16 * i, reinterpret_cast<const uint8_t *>(a.tables) + 16 * i);
-    for (int i = threadIdx.x; i < len; i += blockDim.x) cp_async16(sref + i, rref + (size_t)(ya + i) * a.rpitch + x);
+    for (int i = threadIdx.x; i < len; i += blockDim.x) {
+        const uint2 ce = cref[(size_t)(ya + i) * a.pw];
+        const uint32_t c = kref[(size_t)(ya + i) * a.pw];
+        sref[i] = make_uint4(ce.x, ce.y, c, __float_as_uint(__ldg(a.tables + kTabAD + kTabCen + (c >> 24))));
+    }
     for (int i = threadIdx.x; i < ye - ys; i += blockDim.x) {
         const uchar4 am = aref[(size_t)(ys + i) * W + x];
         sarm[i] = make_uchar4(am.z, am.w, 0, 0);   // backward = up, forward = down
@@ -866,9 +937,10 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
     const int dhi = min(min(a.d0 + a.dc, a.D), dlo + 32) - 1;
     const int d = dlo + lane;
     const int dd = d <= dhi ? d : dlo;                // dead lanes read a real candidate, results unused
-    const int xo = view ? x + dd : x - dd;            // candidate column, -255 .. W + 254 (padded rows)
+    const int xo = view ? x + dd : x - dd;            // candidate column
     const bool outside = xo < 0 || xo >= W;           // match outside the image: cost 1
-    const uint4 *cand = roth + xo;
+    const uint2 *ccand = coth + max(0, min(xo, W - 1));
+    const uint32_t *kcand = koth + max(0, min(xo, W - 1));
     const float Sf = a.S;
     const uint32_t Sint = a.Sint;
 
@@ -877,14 +949,18 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
     uint32_t run = 0;
     int u = sa;
     for (; u + 4 <= sb; u += 4) {
-        uint4 po[4];
+        uint2 pc[4];
+        uint32_t po[4];
 #pragma unroll
-        for (int k = 0; k < 4; k++) po[k] = __ldg(cand + (size_t)(ya + u + k) * a.rpitch);
+        for (int k = 0; k < 4; k++) {
+            pc[k] = __ldg(ccand + (size_t)(ya + u + k) * a.pw);
+            po[k] = __ldg(kcand + (size_t)(ya + u + k) * a.pw);
+        }
 #pragma unroll
         for (int k = 0; k < 4; k++) {
             const uint4 pr = sref[u + k];
-            const int hm = __popc(pr.x ^ po[k].x) + __popc(pr.y ^ po[k].y);
-            const int kk = (int)__dp4a(__vabsdiffu4(pr.z, po[k].z), 0x00010101u, 0u);
+            const int hm = __popc(pr.x ^ pc[k].x) + __popc(pr.y ^ pc[k].y);
+            const int kk = (int)__dp4a(__vabsdiffu4(pr.z, po[k]), 0x00010101u, 0u);
             const float av = __uint_as_float(pr.w);
             const uint32_t q = __float2uint_rn(fmaf(av, sTA[kk], (Sf - av) * sTC[hm]));
             run += outside ? Sint : q;
@@ -892,10 +968,11 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
         }
     }
     for (; u < sb; u++) {
-        const uint4 po = __ldg(cand + (size_t)(ya + u) * a.rpitch);
+        const uint2 pc = __ldg(ccand + (size_t)(ya + u) * a.pw);
+        const uint32_t po = __ldg(kcand + (size_t)(ya + u) * a.pw);
         const uint4 pr = sref[u];
-        const int hm = __popc(pr.x ^ po.x) + __popc(pr.y ^ po.y);
-        const int kk = (int)__dp4a(__vabsdiffu4(pr.z, po.z), 0x00010101u, 0u);
+        const int hm = __popc(pr.x ^ pc.x) + __popc(pr.y ^ pc.y);
+        const int kk = (int)__dp4a(__vabsdiffu4(pr.z, po), 0x00010101u, 0u);
         const float av = __uint_as_float(pr.w);
         const uint32_t q = __float2uint_rn(fmaf(av, sTA[kk], (Sf - av) * sTC[hm]));
         run += outside ? Sint : q;
@@ -1471,14 +1548,13 @@ __global__ void __launch_bounds__(kTX * kTY) k_prep(const __grid_constant__ Batc
     prep_body<CW, CH>(b.p[i], bx, by, bz);
 }
 
-// kWide: blocks of more than kHNarrow warps (rows wider than 640 columns)
-template <int N, bool kWide>
-__global__ void __launch_bounds__(kWide ? 1024 : kHNarrow * 32) k_hagg(const __grid_constant__ Batch<HArgs, N> b)
+template <int N>
+__global__ void __launch_bounds__(kHWarps * 32, 2) k_hagg(const __grid_constant__ Batch<HArgs, N> b)
 {
     pdl_enter();
-    int bx, by, bz;
-    const int i = batch_pair(b, blockIdx.x, bx, by, bz);
-    hagg_body(b.p[i], bx, by, bz);
+    hagg_tasks(b.off[b.n], [&](int t, int &bx, int &by, int &bz) -> const HArgs & {
+        return b.p[batch_pair(b, t, bx, by, bz)];
+    });
 }
 
 template <int N, bool kMax, bool kRow, bool kVol>
@@ -1539,12 +1615,11 @@ __global__ void __launch_bounds__(256) k_vote_end(const __grid_constant__ Batch<
     a.out[k] = v >= a.dmin && v < a.D ? (int16_t)(a.best[k] & 0xffffu) : (int16_t)-1;
 }
 
-__global__ void k_extract_census(const uint4 *__restrict__ rec, int W, int H, int rpitch,
-                                 unsigned long long *out)
+__global__ void k_extract_census(const uint2 *__restrict__ cen, int W, int H, int pw, unsigned long long *out)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (size_t)W * H) return;
-    const uint4 r = rec[(i / W) * rpitch + i % W];
+    const uint2 r = cen[(i / W) * pw + i % W];
     out[i] = ((unsigned long long)r.y << 32) | r.x;
 }
 
@@ -1576,8 +1651,8 @@ struct Derived {
 };
 
 struct Layout {
-    size_t rgbx[2], grey[2], rec[2], cen[2], col[2], arms[2], atmp[2], best[2], sh[2], total;
-    int dc, dstride, npass, rpitch, phw;
+    size_t rgbx[2], grey[2], cen[2], col[2], arms[2], atmp[2], best[2], sh[2], total;
+    int dc, dstride, npass, pw;
 };
 
 constexpr size_t kAlign = 256;
@@ -1625,35 +1700,37 @@ bool dims_valid(int W, int H, int D, int dmin = 0)
     return W >= 1 && H >= 1 && W <= 16384 && H <= 16384 && D >= 1 && dmin >= 0 && dmin + D <= 256 && dmin + D <= W;
 }
 
-Layout make_layout(int W, int H, int D, const dco_params &p, int dc_override = 0)
+// Automatic pass width: both views' slices of a pass within `cap` bytes, at
+// least one group of 32 disparities.  Wide passes are fewer, larger launches of
+// the two aggregation kernels and whole 128-byte lines per pixel and group:
+// first and second pass together at 640x480, D = 64 in one pass 117 us, in two
+// 128; 1280x720, D = 128 in two passes 663 us, in four 722.  The narrow cap
+// (about the L2) is what the serving lanes admit frames by, and the fallback
+// where the device cannot allocate the wide one.
+constexpr size_t kSlicesWide = 512u << 20, kSlicesNarrow = 96u << 20;
+int auto_width(int W, int H, int D, size_t cap)
+{
+    const size_t per = 8 * (size_t)W * H;   // slice bytes per disparity
+    if (per * ((size_t)(D + 31) / 32 * 32) <= cap) return D;
+    return (int)std::min<size_t>(D, std::max<size_t>(32, cap / per / 32 * 32));
+}
+
+Layout make_layout(int W, int H, int D, const dco_params &p, int dc_override = 0, size_t cap = kSlicesWide)
 {
     Layout L{};
     const size_t npx = (size_t)W * H;
     int dc = dc_override > 0 ? dc_override : p.d_chunk;
-    if (dc <= 0) {
-        // automatic: slices of both views within ~96 MB so the producer and
-        // consumer of a pass meet in L2; at least one warp of disparities
-        const size_t cap = 96u << 20;
-        int full = (D + 31) / 32 * 32;
-        if (8 * npx * (size_t)full <= cap) dc = D;
-        else {
-            size_t fit = cap / (8 * npx);
-            dc = (int)std::max<size_t>(32, fit / 32 * 32);
-        }
-    }
+    if (dc <= 0) dc = auto_width(W, H, D, cap);
     dc = std::min(dc, D);
     L.dc = dc;
     L.dstride = (dc + 31) / 32 * 32;
     L.npass = (D + dc - 1) / dc;
     size_t off = 0;
-    L.rpitch = W + 2 * kRPad;
-    L.phw = ((W + 1) / 2 + 3) / 4 * 4;
+    L.pw = (W + 3) / 4 * 4;
     for (int v = 0; v < 2; v++) { L.rgbx[v] = off; off = align_up(off + 4 * npx); }
     for (int v = 0; v < 2; v++) { L.grey[v] = off; off = align_up(off + npx); }
-    for (int v = 0; v < 2; v++) { L.rec[v] = off; off = align_up(off + 16 * (size_t)H * L.rpitch); }
-    // candidate planes, 16 bytes of slack each (the bulk copies end on 16-byte boundaries)
-    for (int v = 0; v < 2; v++) { L.cen[v] = off; off = align_up(off + 8 * (size_t)H * 2 * L.phw + 16); }
-    for (int v = 0; v < 2; v++) { L.col[v] = off; off = align_up(off + 4 * (size_t)H * 2 * L.phw + 16); }
+    for (int v = 0; v < 2; v++) { L.cen[v] = off; off = align_up(off + 8 * (size_t)H * L.pw); }
+    for (int v = 0; v < 2; v++) { L.col[v] = off; off = align_up(off + 4 * (size_t)H * L.pw); }
     // arms: 16 bytes of slack, read by the cost pass's bulk copies past the last pixel
     for (int v = 0; v < 2; v++) { L.arms[v] = off; off = align_up(off + 4 * npx + 16); }
     for (int v = 0; v < 2; v++) { L.atmp[v] = off; off = align_up(off + (p.smooth_arms ? 4 * npx : 0)); }
@@ -1663,8 +1740,7 @@ Layout make_layout(int W, int H, int D, const dco_params &p, int dc_override = 0
     return L;
 }
 
-// H geometry: one block per (row, chunk of output columns, view, group);
-// the block's prefix range is the chunk plus an L1 reach on both sides
+// geometry of a pass over lines: output positions per block, warps, grid
 struct HGeom {
     int chunk, nw;
     size_t smem;
@@ -1696,15 +1772,41 @@ HGeom vcost_geom(int W, int H, int dc, int L1, int want)
     return g;
 }
 
-HGeom hagg_geom(int W, int H, int dc, int L1, int want)
+// the vote's horizontal pass: one block per (row, chunk of output columns, group)
+HGeom hvote_geom(int W, int H, int dc, int L1, int want)
 {
     HGeom g{};
     g.chunk = first_pass_chunk(W, L1, want);
     const int len = std::min(W, g.chunk + 2 * L1);
-    g.nw = (len + kHSegCost - 1) / kHSegCost;
-    g.smem = HSmem(len, g.chunk, g.nw).total;
-    const int ngroups = (dc + 31) / 32;
-    g.grid = dim3((W + g.chunk - 1) / g.chunk, H, 2 * ngroups);
+    g.nw = (len + kHSeg - 1) / kHSeg;
+    g.smem = HVSmem(len, g.chunk, g.nw).total;
+    g.grid = dim3((W + g.chunk - 1) / g.chunk, H, (dc + 31) / 32);
+    return g;
+}
+
+// k_hagg: one task per (row, view, 32 disparities, range of output columns): whole
+// rows up to kHMaxPairs columns, else ranges that fill it with their L1 reach
+// on both sides (the first has a reach on one side only)
+struct HaggGeom {
+    int first, chunk;
+    dim3 grid;   // of tasks: rows, ranges, views and groups
+};
+
+HaggGeom hagg_geom(int W, int H, int dc, int L1, int want)
+{
+    HaggGeom g{};
+    if (W <= kHMaxPairs && (want <= 0 || want >= W)) {
+        g.first = g.chunk = W;
+    } else {
+        g.chunk = kHMaxPairs - 2 * L1;
+        g.first = kHMaxPairs - L1;
+        if (want > 0) {   // (ranges of equal length)
+            const int parts = (W + std::min(want, g.chunk) - 1) / std::min(want, g.chunk);
+            g.first = g.chunk = (W + parts - 1) / parts;
+        }
+    }
+    const int parts = g.first >= W ? 1 : 1 + (W - g.first + g.chunk - 1) / g.chunk;
+    g.grid = dim3(H, parts, 2 * ((dc + kHD - 1) / kHD));
     return g;
 }
 
@@ -1963,7 +2065,7 @@ struct Item {
 
 template <class A, int N, class K>
 dco_status launch_group(dco_stereo *h, cudaStream_t s, const char *name, K kernel, const Item<A> *it, int n,
-                        int block, size_t smem)
+                        int block, size_t smem, int most = INT_MAX)
 {
     Batch<A, N> b;
     std::memset(&b, 0, sizeof b);
@@ -1981,7 +2083,7 @@ dco_status launch_group(dco_stereo *h, cudaStream_t s, const char *name, K kerne
         if (st != DCO_OK) return st;
     }
     ProfScope ps(h, s, name);
-    cudaError_t e = launch_pdl(kernel, dim3((unsigned)b.off[n]), dim3((unsigned)block), smem, s, b);
+    cudaError_t e = launch_pdl(kernel, dim3((unsigned)std::min(b.off[n], most)), dim3((unsigned)block), smem, s, b);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         h->last_error = std::string(name) + " launch (" + std::to_string(n) + " pairs, " + std::to_string(b.off[n]) +
@@ -1992,18 +2094,19 @@ dco_status launch_group(dco_stereo *h, cudaStream_t s, const char *name, K kerne
     return DCO_OK;
 }
 
+// most: blocks of a launch whose kernel takes its blocks' tasks in turn
 // one launch for a single pair (small parameter block), else groups of
 // kBatchMax (kn is the kernel instance for that many)
 template <class A, class K1, class KN>
 dco_status launch_items(dco_stereo *h, cudaStream_t s, const char *name, K1 k1, KN kn,
-                        const std::vector<Item<A>> &items, int block, size_t smem)
+                        const std::vector<Item<A>> &items, int block, size_t smem, int most = INT_MAX)
 {
     constexpr int nmax = kBatchMax;
     if (items.empty()) return DCO_OK;
-    if (items.size() == 1) return launch_group<A, 1>(h, s, name, k1, items.data(), 1, block, smem);
+    if (items.size() == 1) return launch_group<A, 1>(h, s, name, k1, items.data(), 1, block, smem, most);
     for (size_t i = 0; i < items.size(); i += nmax) {
         const int n = (int)std::min<size_t>(nmax, items.size() - i);
-        dco_status st = launch_group<A, nmax>(h, s, name, kn, items.data() + i, n, block, smem);
+        dco_status st = launch_group<A, nmax>(h, s, name, kn, items.data() + i, n, block, smem, most);
         if (st != DCO_OK) return st;
     }
     return DCO_OK;
@@ -2028,7 +2131,7 @@ struct Job {
 
 // workspace plan for all jobs; the pass width shrinks (same for all pairs)
 // until the plan fits the handle's budget
-dco_status plan_jobs(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs, size_t &total)
+dco_status plan_jobs(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs, size_t &total, size_t cap = kSlicesWide)
 {
     // a pair's own pass width (j.dchunk > 0) replaces the call's; a budget
     // override caps both
@@ -2037,7 +2140,7 @@ dco_status plan_jobs(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs,
         for (auto &j : jobs) {
             int dc = j.dchunk > 0 ? j.dchunk : 0;
             if (dc_override > 0) dc = dc > 0 ? std::min(dc, dc_override) : dc_override;
-            j.L = make_layout(j.W, j.H, j.D, p, dc);
+            j.L = make_layout(j.W, j.H, j.D, p, dc, cap);
             j.base = t;
             t = align_up(t + j.L.total);
         }
@@ -2050,6 +2153,21 @@ dco_status plan_jobs(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs,
         for (int dc = widest; dc >= 32 && total > h->budget; dc -= 32) total = plan(dc);
     }
     return DCO_OK;
+}
+
+// workspace for the planned jobs, behind `front` bytes of the call's own.  Wide
+// passes are a choice: where the device or the budget cannot hold them, the
+// jobs are planned again with narrow ones.
+dco_status plan_ws(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs, size_t &total, size_t front = 0)
+{
+    dco_status st = ensure_ws(h, total + front);
+    if (st == DCO_ENOMEM || st == DCO_EBUDGET) {
+        plan_jobs(h, p, jobs, total, kSlicesNarrow);
+        for (auto &j : jobs) j.base += front;
+        return ensure_ws(h, total + front);
+    }
+    for (auto &j : jobs) j.base += front;
+    return st;
 }
 
 template <class T>
@@ -2098,15 +2216,13 @@ dco_status launch_prep(dco_stereo *h, const dco_params &p, const Derived &dv, co
         for (int v = 0; v < 2; v++) {
             b.a.rgbx[v] = jptr<uint32_t>(h, j, j.L.rgbx[v]);
             b.a.grey[v] = jptr<uint8_t>(h, j, j.L.grey[v]);
-            b.a.rec[v] = jptr<uint4>(h, j, j.L.rec[v]) + kRPad;
             b.a.cen[v] = jptr<uint2>(h, j, j.L.cen[v]);
             b.a.col[v] = jptr<uint32_t>(h, j, j.L.col[v]);
             b.a.arms[v] = jptr<uchar4>(h, j, j.L.arms[v]);
         }
-        b.a.phw = j.L.phw;
+        b.a.pw = j.L.pw;
         if (j.arms0) b.a.arms[0] = j.arms0;
-        b.a.tables = h->d_tables;
-        b.a.W = j.W; b.a.H = j.H; b.a.rpitch = j.L.rpitch;
+        b.a.W = j.W; b.a.H = j.H;
         b.a.cw = p.census_w; b.a.ch = p.census_h;
         b.a.L1 = dv.L1; b.a.L2 = p.arm_l2; b.a.tau1 = p.tau1; b.a.tau2 = p.tau2;
         b.gx = (j.W + kTX - 1) / kTX;
@@ -2132,15 +2248,14 @@ dco_status launch_prep(dco_stereo *h, const dco_params &p, const Derived &dv, co
             e.a.src[v] = pr[k].a.arms[v];
             e.a.dst[v] = jptr<uchar4>(h, j, j.L.atmp[v]);
         }
-        e.a.tables = h->d_tables;
-        e.a.W = j.W; e.a.H = j.H; e.a.rpitch = j.L.rpitch;
+        e.a.W = j.W; e.a.H = j.H; e.a.pw = j.L.pw;
         e.gx = (j.W * j.H + 255) / 256; e.gy = nimg; e.gz = 1;
         er.push_back(e);
         Item<SmoothArgs> d = e;
         for (int v = 0; v < 2; v++) {
             d.a.src[v] = e.a.dst[v];
             d.a.dst[v] = pr[k].a.arms[v];
-            d.a.rec[v] = pr[k].a.rec[v];
+            d.a.col[v] = pr[k].a.col[v];
         }
         di.push_back(d);
     }
@@ -2173,9 +2288,10 @@ void deal_v_blocks(const dco_stereo *h, std::vector<Item<VArgs>> &it, int L1, bo
 
 dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> &jobs, int pass, cudaStream_t s)
 {
-    std::map<int, std::vector<Item<HArgs>>> hb;
+    std::map<int, std::vector<Item<HArgs>>> cb;   // k_vcost, by warps per block
+    std::map<int, size_t> csm;
+    std::vector<Item<HArgs>> hb;
     std::vector<Item<VArgs>> vb, vvol;
-    std::map<int, size_t> hsm;
     const size_t vsm = vagg_smem_bytes(dv.L1);
     const bool vh = dv.order == 1;   // vertical segment sums first (k_vcost), then rows (k_vagg<.., kRow>)
     for (const Job &j : jobs) {
@@ -2183,19 +2299,16 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
         const int ng = (dc + 31) / 32;
         const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk, vw = j.vchunk > 0 ? j.vchunk : dv.vchunk;
-        const HGeom hg = vh ? vcost_geom(j.W, j.H, dc, dv.L1, hw) : hagg_geom(j.W, j.H, dc, dv.L1, hw);
         const bool single = j.L.npass == 1 && ng == 1;
-        hsm[hg.nw] = std::max(hsm[hg.nw], hg.smem);
         Item<HArgs> a{};
         for (int v = 0; v < 2; v++) {
-            a.a.rec[v] = jptr<uint4>(h, j, j.L.rec[v]) + kRPad;
             a.a.cen[v] = jptr<uint2>(h, j, j.L.cen[v]);
             a.a.col[v] = jptr<uint32_t>(h, j, j.L.col[v]);
             a.a.arms[v] = jptr<uchar4>(h, j, j.L.arms[v]);
             a.a.sh[v] = jptr<uint32_t>(h, j, j.L.sh[v]);
             a.a.init[v] = pass == 0 && !single ? jptr<unsigned long long>(h, j, j.L.best[v]) : nullptr;
         }
-        a.a.phw = j.L.phw;
+        a.a.pw = j.L.pw;
         a.a.status = h->d_status;
         {   // bounded staging waits; the lost-copy failure test arms the barrier without copies
             const bool lose = (h->test_flags & DCO_TEST_LOSE_TILE_COPIES) != 0;
@@ -2203,12 +2316,22 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
             a.a.skip_copy = lose ? 1 : 0;
         }
         a.a.tables = h->d_tables;
-        a.a.W = j.W; a.a.H = j.H; a.a.D = dv.dmin + j.D; a.a.rpitch = j.L.rpitch;
+        a.a.W = j.W; a.a.H = j.H; a.a.D = dv.dmin + j.D;
         a.a.d0 = d0; a.a.dc = dc; a.a.dstride = j.L.dstride;
         a.a.ngroups = ng;
-        a.a.L1 = dv.L1; a.a.chunk = hg.chunk; a.a.S = dv.S; a.a.Sint = dv.Sint;
-        a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = hg.grid.z;
-        hb[hg.nw].push_back(a);
+        a.a.L1 = dv.L1; a.a.S = dv.S; a.a.Sint = dv.Sint;
+        if (vh) {
+            const HGeom hg = vcost_geom(j.W, j.H, dc, dv.L1, hw);
+            a.a.chunk = hg.chunk;
+            a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = hg.grid.z;
+            csm[hg.nw] = std::max(csm[hg.nw], hg.smem);
+            cb[hg.nw].push_back(a);
+        } else {
+            const HaggGeom hg = hagg_geom(j.W, j.H, dc, dv.L1, hw);
+            a.a.chunk = hg.chunk; a.a.first = hg.first;
+            a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = hg.grid.z;
+            hb.push_back(a);
+        }
         Item<VArgs> b{};
         for (int v = 0; v < 2; v++) {
             b.a.sh[v] = a.a.sh[v];
@@ -2226,21 +2349,15 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
     }
     deal_v_blocks(h, vb, dv.L1, vh);
     deal_v_blocks(h, vvol, dv.L1, vh);
-    for (auto &kv : hb) {
-        if (vh) {
-            dco_status st = launch_items(h, s, "k_vcost", k_vcost<1>, k_vcost<kBatchMax>, kv.second, kv.first * 32,
-                                         hsm[kv.first]);
-            if (st != DCO_OK) return st;
-            continue;
-        }
-        dco_status st = kv.first <= kHNarrow
-                            ? launch_items(h, s, "k_hagg", k_hagg<1, false>, k_hagg<kBatchMax, false>, kv.second,
-                                           kv.first * 32, hsm[kv.first])
-                            : launch_items(h, s, "k_hagg", k_hagg<1, true>, k_hagg<kBatchMax, true>, kv.second,
-                                           kv.first * 32, hsm[kv.first]);
-        if (st != DCO_OK) return st;
-    }
-    dco_status st = vh ? launch_items(h, s, "k_hwta", k_vagg<1, false, true, false>,
+    dco_status st;
+    for (auto &kv : cb)
+        if ((st = launch_items(h, s, "k_vcost", k_vcost<1>, k_vcost<kBatchMax>, kv.second, kv.first * 32,
+                               csm[kv.first])) != DCO_OK)
+            return st;
+    if ((st = launch_items(h, s, "k_hagg", k_hagg<1>, k_hagg<kBatchMax>, hb, kHWarps * 32, hsm::total,
+                           2 * h->nsm)) != DCO_OK)
+        return st;
+    st = vh ? launch_items(h, s, "k_hwta", k_vagg<1, false, true, false>,
                                       k_vagg<kBatchMax, false, true, false>, vb, kVThreads, vsm)
                        : launch_items(h, s, "k_vagg", k_vagg<1, false, false, false>,
                                       k_vagg<kBatchMax, false, false, false>, vb, kVThreads, vsm);
@@ -2274,11 +2391,9 @@ dco_status launch_vote_pass(dco_stereo *h, const Derived &dv, const std::vector<
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
         const int ng = (dc + 31) / 32;
         const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk, vw = j.vchunk > 0 ? j.vchunk : dv.vchunk;
-        const HGeom hg = hagg_geom(j.W, j.H, dc, dv.L1, hw);
+        const HGeom hg = hvote_geom(j.W, j.H, dc, dv.L1, hw);
         const bool single = j.L.npass == 1 && ng == 1;
-        const int hlen = std::min(j.W, hg.chunk + 2 * dv.L1);
-        const int hnw = (hlen + kHSeg - 1) / kHSeg;   // the vote pass walks 64-column segments
-        hsm[hnw] = std::max(hsm[hnw], (size_t)HVSmem(hlen, hg.chunk, hnw).total);
+        hsm[hg.nw] = std::max(hsm[hg.nw], hg.smem);
         Item<HVArgs> a{};
         a.a.disp = j.out;
         a.a.keys = j.vkeys;
@@ -2288,8 +2403,8 @@ dco_status launch_vote_pass(dco_stereo *h, const Derived &dv, const std::vector<
         a.a.sh = jptr<uint32_t>(h, j, j.L.sh[0]);
         a.a.W = j.W; a.a.H = j.H; a.a.d0 = d0; a.a.dstride = j.L.dstride;
         a.a.L1 = dv.L1; a.a.chunk = hg.chunk;
-        a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = ng;
-        hb[hnw].push_back(a);
+        a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = hg.grid.z;
+        hb[hg.nw].push_back(a);
         Item<VArgs> b{};
         b.a.sh[0] = a.a.sh;
         b.a.arms[0] = a.a.arms;
@@ -2385,7 +2500,7 @@ dco_status run_jobs(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs, 
     dco_status st = plan_jobs(h, p, jobs, total);
     if (st != DCO_OK) return st;
     if (!h->budget || total <= h->budget || jobs.size() == 1) {
-        if ((st = ensure_ws(h, total)) != DCO_OK) return st;
+        if ((st = plan_ws(h, p, jobs, total)) != DCO_OK) return st;
         if ((st = ensure_tables(h, p, dv, s)) != DCO_OK) return st;
         return launch_jobs(h, p, dv, jobs, s);
     }
@@ -2552,7 +2667,12 @@ dco_status dco_stereo_reserve(dco_stereo *h, int W, int H, int D, const dco_para
     dco_status st = check_common(h, pin, p);
     if (st != DCO_OK) return st;
     if (!dims_valid(W, H, D, p.d_min)) return DCO_EINVAL;
-    return ensure_ws(h, make_layout(W, H, D, p).total);
+    // under a budget, the widest automatic passes that fit it
+    std::vector<Job> jobs(1);
+    jobs[0].W = W; jobs[0].H = H; jobs[0].D = D;
+    size_t total = make_layout(W, H, D, p).total;
+    if (p.d_chunk == 0 && h->budget && total > h->budget) plan_jobs(h, p, jobs, total);
+    return ensure_ws(h, total);
 }
 
 dco_status dco_stereo_match_views(dco_stereo *h, const uint8_t *left, const uint8_t *right, int W, int H,
@@ -2663,8 +2783,7 @@ dco_status dco_stereo_census(dco_stereo *h, const uint8_t *rgb, int W, int H, co
     const Job &j = jobs[0];
     const size_t n = (size_t)W * H;
     ProfScope ps(h, s, "k_extract_census");
-    k_extract_census<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(jptr<uint4>(h, j, j.L.rec[0]) + kRPad, W, H,
-                                                                  j.L.rpitch,
+    k_extract_census<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(jptr<uint2>(h, j, j.L.cen[0]), W, H, j.L.pw,
                                                                   reinterpret_cast<unsigned long long *>(census_out));
     DCO_CUDA(h, cudaGetLastError());
     return DCO_OK;
@@ -2696,7 +2815,7 @@ dco_status dco_stereo_vote(dco_stereo *h, const uint8_t *rgb, const int16_t *dis
     j.left = rgb; j.right = rgb; j.W = W; j.H = H; j.D = D; j.out = disp_out;
     size_t total = 0;
     if ((st = plan_jobs(h, p, jobs, total)) != DCO_OK) return st;
-    if ((st = ensure_ws(h, total)) != DCO_OK) return st;
+    if ((st = plan_ws(h, p, jobs, total)) != DCO_OK) return st;
     if ((st = ensure_tables(h, p, dv, s)) != DCO_OK) return st;
     if ((st = launch_prep(h, p, dv, jobs, 1, s)) != DCO_OK) return st;   // arms of rgb
     if (disp_in != disp_out)
@@ -2737,8 +2856,7 @@ dco_status dco_stereo_depth(dco_stereo *h, const uint8_t *left, const uint8_t *r
     if ((st = plan_jobs(h, p, jobs, total)) != DCO_OK) return st;
     // in front of the pair's workspace: the two half-size images and the map
     const size_t img = align_up(3 * (size_t)Wh * Hh), front = 2 * img + align_up(2 * (size_t)Wh * Hh);
-    j.base = front;
-    if ((st = ensure_ws(h, total + front)) != DCO_OK) return st;
+    if ((st = plan_ws(h, p, jobs, total, front)) != DCO_OK) return st;
     if ((st = ensure_tables(h, p, dv, s)) != DCO_OK) return st;
     DownArgs da{};
     da.src[0] = left; da.src[1] = right;

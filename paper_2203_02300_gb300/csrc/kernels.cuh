@@ -3,9 +3,9 @@
 // Data layout in HBM (row-major, pixel index i = y*W + x):
 //   rgbx[i]  uint32 r | g<<10 | b<<20          colour in three 10-bit fields (arm tests)
 //   grey[i]  uint8  (77R + 150G + 29B + 128) >> 8
-//   rec[y*rpitch + x]  uint4 {census bits 0-31, census bits 32-63,
-//                    r | g<<8 | b<<16 | Lmin<<24, float bits of alpha(Lmin)*S}
-//                    rows padded by kRPad records on both sides
+//   cen[y*pw + x]  uint2 {census bits 0-31, census bits 32-63}
+//   col[y*pw + x]  uint32 r | g<<8 | b<<16 | Lmin<<24   (pw: W rounded up to a
+//                    multiple of 4, so that every row starts on a 16-byte boundary)
 //   arms[i]  uchar4 {left, right, up, down}
 //   sh[i*dstride + j]  uint32 horizontal segment sum (fixed point) of
 //                    disparity d0 + j (one pass of the d range)
@@ -30,25 +30,11 @@ constexpr int kTabCen = 96;   // entries of the census table (Hamming 0..64)
 constexpr int kTabAlpha = 64; // alpha*S by Lmin, 0..kMaxL1
 constexpr int kTabFloats = kTabAD + kTabCen + kTabAlpha;
 
-// Record rows are padded by kRPad records on both sides, so a candidate
-// x +- d with 0 <= d < 256 never leaves the allocation (its value is then
-// discarded: the cost of a match outside the image is 1).
-constexpr int kRPad = 256;
-
-// Candidate planes (read by the cost pass's bulk copies): per image and
-// row, the census words (uint2) and the colours (uint32) of the even
-// columns, then of the odd columns, each half phw entries long (ceil(W / 2)
-// rounded up to a multiple of 4, so every half starts on a 16-byte
-// boundary); 16 bytes of slack after the last row.
-
-// The cost H pass gives each warp kHSegCost columns of the prefix range (two
-// half-warp segments of 16; one chunk per row up to kHMaxLen columns, else
-// 512-column chunks), k_vcost each warp kHSegCost rows, the vote H pass
-// segments of kHSeg.
+// k_vcost gives each warp kHSegCost rows of the prefix range, the vote H pass
+// segments of kHSeg columns.
 constexpr int kHSegLog = 6, kHSeg = 1 << kHSegLog;
 constexpr int kHSegCost = 32;
-constexpr int kHNarrow = 20;     // warps of the cost H instantiation kept at two blocks per SM
-constexpr int kHMaxLen = 1024;   // prefix columns one H block holds
+constexpr int kHMaxLen = 1024;   // prefix positions one k_vcost or k_hvote block holds
 
 struct PackArgs {
     const uint8_t *rgb[2];
@@ -61,22 +47,19 @@ struct PackArgs {
 struct PrepArgs {
     const uint32_t *rgbx[2];
     const uint8_t *grey[2];
-    uint4 *rec[2];         // first real record of row 0; row pitch rpitch
-    uint2 *cen[2];         // candidate planes (census, colour): row y, column x at
-    uint32_t *col[2];      //   y * 2 phw + (x & 1) * phw + (x >> 1)
-    int phw;
+    uint2 *cen[2];         // planes, row pitch pw
+    uint32_t *col[2];
+    int pw;
     uchar4 *arms[2];
-    const float *tables;   // alpha*S table at offset kTabAD + kTabCen
-    int W, H, rpitch;
+    int W, H;
     int cw, ch;            // census window (odd)
     int L1, L2, tau1, tau2;
 };
 
 struct HArgs {
-    const uint4 *rec[2];   // padded rows, pitch rpitch
-    const uint2 *cen[2];   // candidate planes (PrepArgs)
+    const uint2 *cen[2];   // planes, row pitch pw
     const uint32_t *col[2];
-    int phw;
+    int pw;
     int *status;           // device status word (a lost staging copy sets bit 0)
     int wait_limit;        // mbarrier polls before the staging copies are declared lost
     int skip_copy;         // failure test: arm the staging barrier but issue no copy
@@ -84,12 +67,13 @@ struct HArgs {
     uint32_t *sh[2];
     unsigned long long *init[2];   // first pass: keys to set to the maximum (null: none)
     const float *tables;
-    int W, H, D, rpitch;
+    int W, H, D;
     int d0, dc;            // this pass covers d in [d0, d0 + dc)
     int dstride;           // uint32 per pixel in sh (dc rounded up to 32)
     int ngroups;           // 32-disparity groups in the pass
     int L1;
-    int chunk;             // output columns per block
+    int chunk;             // output positions per block (k_hagg: per task, `first` in a row's first)
+    int first;
     float S;               // fixed-point scale (integer valued)
     uint32_t Sint;
 };
@@ -125,9 +109,8 @@ struct DepthArgs {
 struct SmoothArgs {
     const uchar4 *src[2];
     uchar4 *dst[2];
-    uint4 *rec[2];         // dilation pass: records whose L_min and alpha*S follow the new arms
-    const float *tables;
-    int W, H, rpitch;
+    uint32_t *col[2];      // dilation pass: colour words whose L_min follows the new arms
+    int W, H, pw;
 };
 
 struct VArgs {

@@ -324,6 +324,11 @@ dco_status dco_server_create(dco_server **out, int device, const dco_stream_desc
     s->params = p;
     s->max_batch = max_batch;
     s->streams.assign(streams, streams + nstreams);
+    // frames are admitted by the workspace of narrow passes: a lane's share
+    // holds as many of them, whatever widths single calls would take
+    if (p.d_chunk == 0)
+        for (auto &d : s->streams)
+            if (d.d_chunk == 0) d.d_chunk = auto_width(d.W, d.H, d.D, kSlicesNarrow);
     size_t total = 0, largest = 0;
     for (const auto &d : s->streams) {
         s->ws.push_back(stream_ws(p, d));

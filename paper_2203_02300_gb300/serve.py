@@ -62,6 +62,15 @@ class _Lane:
         self.busy = False
 
 
+def _narrow_width(W: int, H: int, D: int) -> int:
+    """The pass width whose slices of both views stay within 96 MiB (at least
+    32 disparities)."""
+    per = 8 * W * H
+    if per * (-(-D // 32) * 32) <= 96 << 20:
+        return D
+    return min(D, max(32, (96 << 20) // per // 32 * 32))
+
+
 class Server:
     def __init__(self, shapes: Sequence[tuple[int, int, int]], budget_bytes: Optional[int] = None,
                  lanes: int = 2, slots_per_stream: int = 3, max_batch: int = 16,
@@ -73,8 +82,12 @@ class Server:
         self.shapes = [tuple(int(v) for v in s) for s in shapes]
         self.params = params
         self.max_batch = max_batch
-        # each stream's tiles (e.g. tune.tune_batch); 0 fields = the params' own
+        # each stream's tiles (e.g. tune.tune_batch); 0 fields = the params' own.
+        # Frames are admitted by the workspace of narrow passes.
         self.tiles = [Tile.of(v) for v in (tiles or [None] * len(self.shapes))]
+        if not (params and params.d_chunk):
+            self.tiles = [t if t.d_chunk else t._replace(d_chunk=_narrow_width(*s))
+                          for t, s in zip(self.tiles, self.shapes)]
 
         def ws_of(s):
             W, H, D = self.shapes[s]
