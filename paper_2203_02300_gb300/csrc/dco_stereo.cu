@@ -255,6 +255,7 @@ __device__ __forceinline__ void pack_rows_body(const PackArgs &a, int t, int img
 // compares four neighbours per SIMD byte comparison.
 constexpr int kTX = 32, kTY = 8;
 constexpr int kMaxCW = 15, kMaxCH = 15;
+constexpr int kArmRun = 8;   // candidates of an arm walk loaded together
 constexpr int kGW = 48;   // grey tile row pitch (>= kTX + kMaxCW - 1, multiple of 4)
 
 // 4 flags f_i = [byte_i(w) < byte_i(c4)] -> bits f0 | f1<<1 | f2<<2 | f3<<3.
@@ -344,12 +345,40 @@ __device__ __forceinline__ void prep_body(const PrepArgs &a, int bx, int by, int
     auto kfield = [](int tau) { return 0x00100401u * (uint32_t)(min(tau, 256) + 511); };
     const uint32_t k1 = kfield(a.tau1), k2 = kfield(min(a.tau1, a.tau2));
     const uint32_t K1p = k1 - p, pK1 = p + k1, K2p = k2 - p, pK2 = p + k2;
-    auto pass = [](uint32_t c, uint32_t Kp, uint32_t pK, uint32_t ew, uint32_t bit) {
-        return ((((c + Kp) & (pK - c)) & kM9 | (ew & bit)) == (kM9 | bit));
+    auto fails = [](uint32_t c, uint32_t Kp, uint32_t pK, uint32_t ew, uint32_t bit) {
+        return ((~((c + Kp) & (pK - c)) & kM9) | (~ew & bit)) != 0u;
     };
-    // the first kArmBatch candidates of all four directions are loaded at
-    // once (in-image addresses only), so a typical pixel pays one load latency
-    constexpr int kArmBatch = 2;
+    // Steps n + 1 .. end of one direction, with one pair of constants; true if
+    // all of them pass.  kArmRun candidates are loaded together, and tested one
+    // by one with a way out after each, so a step costs its load, the two sums
+    // and the two logic operations of its test and a branch.
+    auto walk = [&](auto own_c, const uint32_t *&q, ptrdiff_t st, uint32_t &prev, int &n, int end, uint32_t Kp, uint32_t pK,
+                    uint32_t bit) -> bool {
+        constexpr bool kOwn = decltype(own_c)::value;   // right, down: the candidate's own edge bit; left, up: its predecessor's
+        for (; n + kArmRun <= end; n += kArmRun) {
+            uint32_t c[kArmRun];
+#pragma unroll
+            for (int u = 0; u < kArmRun; u++) c[u] = __ldg(q + (u + 1) * st);
+#pragma unroll
+            for (int u = 0; u < kArmRun; u++)
+                if (fails(c[u], Kp, pK, kOwn ? c[u] : u ? c[u ? u - 1 : 0] : prev, bit)) {
+                    n += u;
+                    return false;
+                }
+            prev = c[kArmRun - 1];
+            q += kArmRun * st;
+        }
+        for (; n < end; n++) {
+            q += st;
+            const uint32_t c = __ldg(q);
+            if (fails(c, Kp, pK, kOwn ? c : prev, bit)) return false;
+            prev = c;
+        }
+        return true;
+    };
+    // the first candidate of all four directions is loaded at once (in-image
+    // addresses only)
+    constexpr int kArmBatch = 1;
     int arm[4];
     uint32_t cand[4][kArmBatch];
     int lim[4];
@@ -375,47 +404,22 @@ __device__ __forceinline__ void prep_body(const PrepArgs &a, int bx, int by, int
             const int j = u + 1;
             const bool far = j > L2;
             const uint32_t c = cand[e][u];
-            if (open && j <= lim[e] && pass(c, far ? K2p : K1p, far ? pK2 : pK1, own ? c : prev, bit)) {
+            if (open && j <= lim[e] && !fails(c, far ? K2p : K1p, far ? pK2 : pK1, own ? c : prev, bit)) {
                 n = j;
                 prev = c;
             } else {
                 open = false;
             }
         }
-        // longer arms: one candidate at a time, up to L2 then beyond
-        if (open) {
+        if (open) {   // longer arms: up to L2, then beyond
             const uint32_t *q = rgbx + i + (ptrdiff_t)n * step[e];
-            int j = n + 1;
             if (own) {
-                for (const int l = min(lim[e], L2); j <= l; j++) {
-                    q += step[e];
-                    const uint32_t c = __ldg(q);
-                    if (!pass(c, K1p, pK1, c, bit)) { open = false; break; }
-                }
-                if (open) {
-                    for (; j <= lim[e]; j++) {
-                        q += step[e];
-                        const uint32_t c = __ldg(q);
-                        if (!pass(c, K2p, pK2, c, bit)) break;
-                    }
-                }
+                if (walk(std::true_type{}, q, step[e], prev, n, min(lim[e], L2), K1p, pK1, bit))
+                    walk(std::true_type{}, q, step[e], prev, n, lim[e], K2p, pK2, bit);
             } else {
-                for (const int l = min(lim[e], L2); j <= l; j++) {
-                    q += step[e];
-                    const uint32_t c = __ldg(q);
-                    if (!pass(c, K1p, pK1, prev, bit)) { open = false; break; }
-                    prev = c;
-                }
-                if (open) {
-                    for (; j <= lim[e]; j++) {
-                        q += step[e];
-                        const uint32_t c = __ldg(q);
-                        if (!pass(c, K2p, pK2, prev, bit)) break;
-                        prev = c;
-                    }
-                }
+                if (walk(std::false_type{}, q, step[e], prev, n, min(lim[e], L2), K1p, pK1, bit))
+                    walk(std::false_type{}, q, step[e], prev, n, lim[e], K2p, pK2, bit);
             }
-            n = j - 1;
         }
         arm[e] = n;
     }
@@ -425,6 +429,137 @@ __device__ __forceinline__ void prep_body(const PrepArgs &a, int bx, int by, int
     (img ? a.cen[1] : a.cen[0])[pe] = make_uint2((uint32_t)bits, (uint32_t)(bits >> 32));
     (img ? a.col[1] : a.col[0])[pe] = colour;
     (img ? a.arms[1] : a.arms[0])[i] = make_uchar4((uint8_t)arm[0], (uint8_t)arm[1], (uint8_t)arm[2], (uint8_t)arm[3]);
+}
+
+// The same for launches that leave most of the SMs idle, where the time is that
+// of one pixel's four walks: block = a 32 x 4 tile, four threads per pixel,
+// warp = (direction, row).  Every thread walks one arm of its pixel and takes
+// two rows of its census window; one warp per row puts the parts together.
+// 96x64 13.0 -> 9.9 us, 320x240 18.8 us either way, 640x480 46.7 against 35.3 us
+// (four times the set-up per pixel): the line lies at two blocks of prep_body
+// per SM.
+constexpr int kTYd = 4, kDirs = 4, kPrepThreads = kTX * kTYd * kDirs;
+constexpr int kArmRunDirs = 4;
+
+template <int CW, int CH>
+__device__ __forceinline__ void prep_dirs_body(const PrepArgs &a, int bx, int by, int img)
+{
+    __shared__ __align__(16) uint8_t gs[kTYd + kMaxCH - 1][kGW];
+    __shared__ uint2 part_s[kDirs][kTYd][kTX];   // census bits
+    __shared__ uint8_t arm_s[kDirs][kTYd][kTX];
+    constexpr bool kStd = CW == 9 && CH == 7;
+    const uint32_t *__restrict__ rgbx = img ? a.rgbx[1] : a.rgbx[0];
+    const uint8_t *__restrict__ grey = img ? a.grey[1] : a.grey[0];
+    const int W = a.W, H = a.H;
+    const int cw = CW ? CW : a.cw, ch = CH ? CH : a.ch;
+    const int rx = cw / 2, ry = ch / 2;
+    const int x0 = bx * kTX, y0 = by * kTYd;
+    const int warp = threadIdx.x >> 5, tx = threadIdx.x & 31, ty = warp % kTYd, dir = warp / kTYd;   // left, right, up, down
+    const int x = x0 + tx, y = y0 + ty;
+    const bool in = x < W && y < H;
+    const size_t i = (size_t)min(y, H - 1) * W + min(x, W - 1);
+    const uint32_t praw = __ldg(rgbx + i);   // colours are stored spread (k_pack), with edge bits
+    for (int r = warp; r < kTYd + 2 * ry; r += kTYd * kDirs) {
+        const uint8_t *g = grey + (size_t)min(max(y0 - ry + r, 0), H - 1) * W;
+        for (int c = tx; c < kTX + 2 * rx; c += kTX) gs[r][c] = __ldg(g + min(max(x0 - rx + c, 0), W - 1));
+    }
+
+    // the arm: the rule of prep_body
+    {
+        const uint32_t p = praw & kColour;
+        auto kfield = [](int tau) { return 0x00100401u * (uint32_t)(min(tau, 256) + 511); };
+        const uint32_t k1 = kfield(a.tau1), k2 = kfield(min(a.tau1, a.tau2));
+        const uint32_t bit = dir < 2 ? kEdgeL : kEdgeU;
+        const int st = dir == 0 ? -1 : dir == 1 ? 1 : dir == 2 ? -W : W;
+        const int room = dir == 0 ? x : dir == 1 ? W - 1 - x : dir == 2 ? y : H - 1 - y;
+        const int lim = in ? min(a.L1, room) : 0;
+        const uint32_t *q = rgbx + i;
+        uint32_t prev = praw;
+        int n = 0;
+        auto fails = [&](uint32_t c, uint32_t Kp, uint32_t pK, uint32_t ew) {
+            return ((~((c + Kp) & (pK - c)) & kM9) | (~ew & bit)) != 0u;
+        };
+        // steps n + 1 .. end; true if all of them pass
+        auto walk = [&](auto own_c, int end, uint32_t k) -> bool {
+            constexpr bool kOwn = decltype(own_c)::value;
+            const uint32_t Kp = k - p, pK = p + k;
+            for (; n + kArmRunDirs <= end; n += kArmRunDirs) {
+                uint32_t c[kArmRunDirs];
+#pragma unroll
+                for (int u = 0; u < kArmRunDirs; u++) {
+                    q += st;
+                    c[u] = __ldg(q);
+                }
+#pragma unroll
+                for (int u = 0; u < kArmRunDirs; u++)
+                    if (fails(c[u], Kp, pK, kOwn ? c[u] : u ? c[u ? u - 1 : 0] : prev)) {
+                        n += u;
+                        return false;
+                    }
+                prev = c[kArmRunDirs - 1];
+            }
+            for (; n < end; n++) {
+                q += st;
+                const uint32_t c = __ldg(q);
+                if (fails(c, Kp, pK, kOwn ? c : prev)) return false;
+                prev = c;
+            }
+            return true;
+        };
+        if (dir & 1) {
+            if (walk(std::true_type{}, min(lim, a.L2), k1)) walk(std::true_type{}, lim, k2);
+        } else {
+            if (walk(std::false_type{}, min(lim, a.L2), k1)) walk(std::false_type{}, lim, k2);
+        }
+        arm_s[dir][ty][tx] = (uint8_t)n;
+    }
+    __syncthreads();   // (the grey tile)
+
+    // census: bit k = [Y(n) < Y(p)], window row-major, centre skipped
+    const uint32_t yc = gs[ty + ry][tx + rx];
+    if (kStd) {
+        const uint32_t c4 = yc * 0x01010101u, c4lo = c4 & 0x7f7f7f7fu;
+        const int al = tx & ~3, sh = 8 * (tx & 3);
+        auto row_bits = [&](int dy) -> uint32_t {
+            const uint32_t *row = reinterpret_cast<const uint32_t *>(&gs[ty + dy][al]);
+            const uint32_t a0 = row[0], a1 = row[1], a2 = row[2];
+            const uint32_t w0 = __funnelshift_r(a0, a1, sh);   // bytes dx 0..3
+            const uint32_t w1 = __funnelshift_r(a1, a2, sh);   // bytes dx 4..7
+            const uint32_t b8 = (__funnelshift_r(a2, 0u, sh) & 0xffu) < yc ? 1u : 0u;   // dx 8
+            const uint32_t f0 = lt4(w0, c4, c4lo), f1 = lt4(w1, c4, c4lo);
+            return dy == 3 ? f0 | ((f1 >> 1) << 4) | (b8 << 7)   // centre row: dx 4 is the centre itself
+                           : f0 | (f1 << 4) | (b8 << 8);
+        };
+        // window rows 2 dir, 2 dir + 1; rows start at bits 0, 9, 18, 27, 35, 44, 53
+        const int first = 18 * dir - (dir > 1), second = dir == 1 ? 27 : first + 9;
+        unsigned long long bits = (unsigned long long)row_bits(2 * dir) << first;
+        if (dir < 3) bits |= (unsigned long long)row_bits(2 * dir + 1) << second;
+        part_s[dir][ty][tx] = make_uint2((uint32_t)bits, (uint32_t)(bits >> 32));
+    }
+    __syncthreads();
+    if (dir != 0 || !in) return;
+    uint2 census;
+    if (kStd) {
+        const uint2 b0 = part_s[0][ty][tx], b1 = part_s[1][ty][tx], b2 = part_s[2][ty][tx], b3 = part_s[3][ty][tx];
+        census = make_uint2(b0.x | b1.x | b2.x | b3.x, b0.y | b1.y | b2.y | b3.y);
+    } else {
+        unsigned long long bits = 0ull;
+        int k = 0;
+        for (int dy = 0; dy < ch; dy++) {
+            for (int dx = 0; dx < cw; dx++) {
+                if (dy == ry && dx == rx) continue;
+                if (gs[ty + dy][tx + dx] < yc) bits |= 1ull << k;
+                k++;
+            }
+        }
+        census = make_uint2((uint32_t)bits, (uint32_t)(bits >> 32));
+    }
+    const int l = arm_s[0][ty][tx], r = arm_s[1][ty][tx], u = arm_s[2][ty][tx], d = arm_s[3][ty][tx];
+    const uint32_t lmin = (uint32_t)min(min(l, r), min(u, d));
+    const size_t pe = (size_t)y * a.pw + x;
+    (img ? a.cen[1] : a.cen[0])[pe] = census;
+    (img ? a.col[1] : a.col[0])[pe] = unspread10(praw) | (lmin << 24);
+    (img ? a.arms[1] : a.arms[0])[i] = make_uchar4((uint8_t)l, (uint8_t)r, (uint8_t)u, (uint8_t)d);
 }
 
 // --------------------------------------------------------------- k_smooth
@@ -1157,6 +1292,7 @@ __device__ __forceinline__ uint32_t region_size(const uchar4 *arms, int W, size_
     const uchar4 p = arms[i];
     uint32_t n = 0;
     if (!row_order)
+#pragma unroll 8
         for (int k = -(int)p.z; k <= (int)p.w; k++) {
             const uchar4 q = arms[(ptrdiff_t)i + (ptrdiff_t)k * W];
             n += q.x + q.y + 1u;
@@ -1410,13 +1546,13 @@ __device__ __forceinline__ void lr_body(const LrArgs &a, size_t i)
 // disparities and minimum costs (where asked for) and the consistency map.
 // The region size N(p) of a cost is summed on the spot: only callers that
 // ask for costs pay for it.
-__device__ __forceinline__ void end_body(const EndArgs &a, size_t i)
+__device__ __forceinline__ void end_body(const EndArgs &a, size_t i, int view)   // view -1: both
 {
     if (i >= (size_t)a.W * a.H) return;
     const int x = int(i % a.W);
     const unsigned long long kl = a.best[0][i];
     const int d = (int)(kl & 0xffffu);
-    if (a.out) {
+    if (a.out && view <= 0) {
         int16_t r = -1;
         if (a.tol < 0) r = (int16_t)d;
         else if (x - d >= 0 && abs(d - (int)(a.best[1][i - d] & 0xffffu)) <= a.tol) r = (int16_t)d;
@@ -1424,7 +1560,7 @@ __device__ __forceinline__ void end_body(const EndArgs &a, size_t i)
     }
 #pragma unroll
     for (int v = 0; v < 2; v++) {
-        if (!a.disp[v] && !a.cost[v]) continue;
+        if ((!a.disp[v] && !a.cost[v]) || view == 1 - v) continue;
         const unsigned long long k = v ? a.best[1][i] : kl;
         if (a.disp[v]) a.disp[v][i] = (int16_t)(k & 0xffffu);
         if (a.cost[v])
@@ -1548,6 +1684,15 @@ __global__ void __launch_bounds__(kTX * kTY) k_prep(const __grid_constant__ Batc
     prep_body<CW, CH>(b.p[i], bx, by, bz);
 }
 
+template <int CW, int CH, int N>
+__global__ void __launch_bounds__(kPrepThreads) k_prep_dirs(const __grid_constant__ Batch<PrepArgs, N> b)
+{
+    pdl_enter();
+    int bx, by, bz;
+    const int i = batch_pair(b, blockIdx.x, bx, by, bz);
+    prep_dirs_body<CW, CH>(b.p[i], bx, by, bz);
+}
+
 template <int N>
 __global__ void __launch_bounds__(kHWarps * 32, 2) k_hagg(const __grid_constant__ Batch<HArgs, N> b)
 {
@@ -1599,7 +1744,7 @@ __global__ void __launch_bounds__(256) k_end(const __grid_constant__ Batch<EndAr
     pdl_enter();
     int bx, by, bz;
     const int i = batch_pair(b, blockIdx.x, bx, by, bz);
-    end_body(b.p[i], (size_t)bx * 256 + threadIdx.x);
+    end_body(b.p[i], (size_t)bx * 256 + threadIdx.x, b.p[i].views == 2 ? by : -1);
 }
 
 template <int N>
@@ -2234,7 +2379,17 @@ dco_status launch_prep(dco_stereo *h, const dco_params &p, const Derived &dv, co
     if (st != DCO_OK) return st;
     st = launch_items(h, s, "k_pack", k_pack<1, kPackHostRows>, k_pack<kBatchMax, kPackHostRows>, pk_host, 256, 0);
     if (st != DCO_OK) return st;
-    if (p.census_w == 9 && p.census_h == 7)
+    int blocks = 0;
+    for (const auto &b : pr) blocks += b.gx * b.gy * b.gz;
+    const bool dirs = blocks <= 2 * h->nsm;   // a thread per arm instead of one per pixel
+    if (dirs)
+        for (auto &b : pr) b.gy = (b.a.H + kTYd - 1) / kTYd;
+    const bool std_census = p.census_w == 9 && p.census_h == 7;
+    if (dirs && std_census)
+        st = launch_items(h, s, "k_prep", k_prep_dirs<9, 7, 1>, k_prep_dirs<9, 7, kBatchMax>, pr, kPrepThreads, 0);
+    else if (dirs)
+        st = launch_items(h, s, "k_prep", k_prep_dirs<0, 0, 1>, k_prep_dirs<0, 0, kBatchMax>, pr, kPrepThreads, 0);
+    else if (std_census)
         st = launch_items(h, s, "k_prep", k_prep<9, 7, 1>, k_prep<9, 7, kBatchMax>, pr, kTX * kTY, 0);
     else
         st = launch_items(h, s, "k_prep", k_prep<0, 0, 1>, k_prep<0, 0, kBatchMax>, pr, kTX * kTY, 0);
@@ -2480,7 +2635,8 @@ dco_status launch_jobs(dco_stereo *h, const dco_params &p, const Derived &dv, st
         it.a.disp[0] = j.disp_l; it.a.disp[1] = j.disp_r; it.a.out = j.out;
         it.a.cost[0] = j.cost_l; it.a.cost[1] = j.cost_r;
         it.a.W = j.W; it.a.H = j.H; it.a.tol = p.lr_tol; it.a.order = dv.order; it.a.S = dv.S;
-        it.gx = (j.W * j.H + 255) / 256; it.gy = 1; it.gz = 1;
+        it.a.views = j.cost_l || j.cost_r ? 2 : 1;   // blocks of their own for each view's region sums
+        it.gx = (j.W * j.H + 255) / 256; it.gy = it.a.views; it.gz = 1;
         end.push_back(it);
     }
     if ((st = launch_items(h, s, "k_end", k_end<1>, k_end<kBatchMax>, end, 256, 0)) != DCO_OK) return st;

@@ -139,6 +139,7 @@ struct EndArgs {
     int16_t *disp[2], *out;
     float *cost[2];
     int W, H, tol, order;
+    int views;             // blocks per pixel range: 1, or one per view
     float S;
 };
 
