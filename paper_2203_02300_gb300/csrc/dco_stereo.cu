@@ -568,25 +568,36 @@ __device__ __forceinline__ void prep_dirs_body(const PrepArgs &a, int bx, int by
 // maximum (kMax = true), windows cut to the image.  An opening never
 // lengthens an arm, so arms stay inside the image and <= L1.  The maximum
 // pass also rewrites the colour word's L_min (Eq. 1's weight).
+// A thread takes four pixels of a column, six rows of three arm words: the
+// four arms of a word are compared at once (byte-wise minimum or maximum), and
+// coordinates past the border repeat the border, which changes neither.
+// 640x480: 13.4 -> KSM us (nine words per pixel, arm by arm, before).
+constexpr int kSmRows = 4;
 template <bool kMax>
-__device__ __forceinline__ void smooth_body(const SmoothArgs &a, int i, int img)
+__device__ __forceinline__ void smooth_body(const SmoothArgs &a, int t, int img)
 {
-    if (i >= a.W * a.H) return;
-    const int x = i % a.W, y = i / a.W;
-    const uchar4 *src = img ? a.src[1] : a.src[0];
-    int v[4] = {kMax ? 0 : 255, kMax ? 0 : 255, kMax ? 0 : 255, kMax ? 0 : 255};
-    for (int yy = max(0, y - 1); yy <= min(a.H - 1, y + 1); yy++)
-        for (int xx = max(0, x - 1); xx <= min(a.W - 1, x + 1); xx++) {
-            const uchar4 q = src[(size_t)yy * a.W + xx];
-            const int c[4] = {q.x, q.y, q.z, q.w};
+    const int W = a.W, H = a.H, x = t % W, y0 = kSmRows * (t / W);
+    if (y0 >= H) return;
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(img ? a.src[1] : a.src[0]);
+    const int xl = max(x - 1, 0), xr = min(x + 1, W - 1);
+    auto pick = [](uint32_t u, uint32_t v) { return kMax ? __vmaxu4(u, v) : __vminu4(u, v); };
+    uint32_t row[kSmRows + 2];   // of the three words of each row
 #pragma unroll
-            for (int k = 0; k < 4; k++) v[k] = kMax ? max(v[k], c[k]) : min(v[k], c[k]);
+    for (int k = 0; k < kSmRows + 2; k++) {
+        const uint32_t *p = src + (size_t)min(max(y0 - 1 + k, 0), H - 1) * W;
+        row[k] = pick(pick(p[xl], p[x]), p[xr]);
+    }
+#pragma unroll
+    for (int k = 0; k < kSmRows; k++) {
+        const int y = y0 + k;
+        if (y >= H) break;
+        const uint32_t v = pick(pick(row[k], row[k + 1]), row[k + 2]);
+        reinterpret_cast<uint32_t *>(img ? a.dst[1] : a.dst[0])[(size_t)y * W + x] = v;
+        if (kMax) {
+            const uint32_t lmin = min(min(v & 0xffu, (v >> 8) & 0xffu), min((v >> 16) & 0xffu, v >> 24));
+            uint32_t *c = (img ? a.col[1] : a.col[0]) + (size_t)y * a.pw + x;
+            *c = (*c & 0x00ffffffu) | (lmin << 24);
         }
-    (img ? a.dst[1] : a.dst[0])[i] = make_uchar4((uint8_t)v[0], (uint8_t)v[1], (uint8_t)v[2], (uint8_t)v[3]);
-    if (kMax) {
-        const int lmin = min(min(v[0], v[1]), min(v[2], v[3]));
-        uint32_t *c = (img ? a.col[1] : a.col[0]) + (size_t)y * a.pw + x;
-        *c = (*c & 0x00ffffffu) | (uint32_t(lmin) << 24);
     }
 }
 
@@ -1292,7 +1303,7 @@ __device__ __forceinline__ uint32_t region_size(const uchar4 *arms, int W, size_
     const uchar4 p = arms[i];
     uint32_t n = 0;
     if (!row_order)
-#pragma unroll 8
+#pragma unroll 16
         for (int k = -(int)p.z; k <= (int)p.w; k++) {
             const uchar4 q = arms[(ptrdiff_t)i + (ptrdiff_t)k * W];
             n += q.x + q.y + 1u;
@@ -2404,7 +2415,7 @@ dco_status launch_prep(dco_stereo *h, const dco_params &p, const Derived &dv, co
             e.a.dst[v] = jptr<uchar4>(h, j, j.L.atmp[v]);
         }
         e.a.W = j.W; e.a.H = j.H; e.a.pw = j.L.pw;
-        e.gx = (j.W * j.H + 255) / 256; e.gy = nimg; e.gz = 1;
+        e.gx = (j.W * ((j.H + kSmRows - 1) / kSmRows) + 255) / 256; e.gy = nimg; e.gz = 1;
         er.push_back(e);
         Item<SmoothArgs> d = e;
         for (int v = 0; v < 2; v++) {
