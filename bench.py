@@ -97,7 +97,7 @@ def source_digest() -> str:
         cu = fh.read()
     host = cu.index("// ====================================================================== host")
     parts.append(cu[:host])
-    parts.append(cu[cu.index("struct HGeom {"):cu.index("// ---- TMA tile maps")])
+    parts.append(cu[cu.index("struct HGeom {"):cu.index("struct dco_stereo {")])
     h = hashlib.sha256()
     for part in parts:
         h.update(strip(part).encode())
@@ -191,13 +191,13 @@ def algorithmic_bytes(kernel: str, npx: int, ev_pass: int, npass: int) -> float:
     if kernel == "k_pack":
         return 2 * npx * (3 + 4 + 1)                       # rgb in, rgbx + grey out
     if kernel == "k_prep":
-        return 2 * npx * (4 + 1 + 16 + 4)                  # rgbx + grey in, record + arms out
+        return 2 * npx * (4 + 1 + 12 + 4)                  # rgbx + grey in, census, colour + arms out
     if kernel == "k_hagg":
-        return 4 * ev_pass + 2 * npx * (16 + 16 + 4)       # slice out; records + arms in
+        return 4 * ev_pass + 2 * npx * (12 + 12 + 4)       # slice out; both images' planes + arms in
     if kernel == "k_vagg":
-        return 4 * ev_pass + 2 * npx * (4 + 2 + (16 if npass > 1 else 0))   # slice in; arms in, disparity/state out
-    if kernel == "k_lr":
-        return npx * (2 + 2 + 2)
+        return 4 * ev_pass + 2 * npx * (4 + 8 * (2 if npass > 1 else 1))   # slice + arms in, keys out (and in)
+    if kernel == "k_end":
+        return npx * (8 + 8 + 2)                           # keys in, map out
     return 0.0
 
 
@@ -441,7 +441,7 @@ def vote_config2(torch, binding, st, L, R, D, dchunk, flush, dev, reps: int = 20
     pk, _ = peaks()
     dc = dchunk or D
     alg = {"k_hvote": lambda: npx * (2 + 4) + 4 * npx * dc,        # map + arms in, count slice out
-           "k_vvote": lambda: 4 * npx * dc + npx * (4 + 2 + 2)}   # slice + arms + mask in, map out
+           "k_vvote": lambda: 4 * npx * dc + npx * (4 + 8)}   # slice + arms in, keys out
     kern = {}
     round_us = 0.0
     for k in ("k_hvote", "k_vvote"):

@@ -1297,7 +1297,7 @@ __host__ __device__ inline size_t vagg_smem_bytes(int L1)
 }
 static_assert(((2 * kMaxL1 + kVSub) / kVSub * kVSub + kVStep) * kVRow <= 1 << 16, "k_vagg: ring offsets in 16 bits");
 
-// N(p) of Eq. 2: the segment lengths along p's second arm
+// N(p) of Eq. 2: the segment lengths along p's second arm (cost volumes)
 __device__ __forceinline__ uint32_t region_size(const uchar4 *arms, int W, size_t i, bool row_order)
 {
     const uchar4 p = arms[i];
@@ -1555,27 +1555,67 @@ __device__ __forceinline__ void lr_body(const LrArgs &a, size_t i)
 // -------------------------------------------------------------------- k_end
 // The per-pixel end of a match: the winners' keys become the two views'
 // disparities and minimum costs (where asked for) and the consistency map.
-// The region size N(p) of a cost is summed on the spot: only callers that
-// ask for costs pay for it.
-__device__ __forceinline__ void end_body(const EndArgs &a, size_t i, int view)   // view -1: both
+__device__ __forceinline__ int16_t checked(const EndArgs &a, size_t i, int x, int d)
+{
+    if (a.tol < 0) return (int16_t)d;
+    if (x - d >= 0 && abs(d - (int)(a.best[1][i - d] & 0xffffu)) <= a.tol) return (int16_t)d;
+    return -1;
+}
+
+__device__ __forceinline__ void end_body(const EndArgs &a, size_t i)
 {
     if (i >= (size_t)a.W * a.H) return;
-    const int x = int(i % a.W);
-    const unsigned long long kl = a.best[0][i];
-    const int d = (int)(kl & 0xffffu);
-    if (a.out && view <= 0) {
-        int16_t r = -1;
-        if (a.tol < 0) r = (int16_t)d;
-        else if (x - d >= 0 && abs(d - (int)(a.best[1][i - d] & 0xffffu)) <= a.tol) r = (int16_t)d;
-        a.out[i] = r;
-    }
+    const int d = (int)(a.best[0][i] & 0xffffu);
+    if (a.out) a.out[i] = checked(a, i, int(i % a.W), d);
+    if (a.disp[0]) a.disp[0][i] = (int16_t)d;
+    if (a.disp[1]) a.disp[1][i] = (int16_t)(a.best[1][i] & 0xffffu);
+}
+
+// The same with costs, for one view: a cost is the key's sum over the region
+// size N(p) of Eq. 2, the segment lengths along p's second arm.  Block = a 32 x
+// 8 tile; the lengths of the tile and its reach along the walk are staged in
+// shared memory, every load of a thread in flight at once (bound by latency).
+constexpr int kEX = 32, kEY = 8;
+template <bool kRow>
+__device__ __forceinline__ void end_costs_body(const EndArgs &a, int bx, int by, int view)
+{
+    constexpr int kPitch = kRow ? kEX + 2 * kMaxL1 : kEX;
+    constexpr int kLoads = kRow ? (kEX + 2 * kMaxL1 + 31) / 32 : (kEY + 2 * kMaxL1 + kEY - 1) / kEY;
+    __shared__ uint16_t len_s[kRow ? kEY * kPitch : (kEY + 2 * kMaxL1) * kPitch];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int W = a.W, H = a.H, L1 = a.L1, x = kEX * bx + lane, y = kEY * by + warp;
+    const uchar4 *arms = view ? a.arms[1] : a.arms[0];
+    uchar4 q[kLoads];
 #pragma unroll
-    for (int v = 0; v < 2; v++) {
-        if ((!a.disp[v] && !a.cost[v]) || view == 1 - v) continue;
-        const unsigned long long k = v ? a.best[1][i] : kl;
-        if (a.disp[v]) a.disp[v][i] = (int16_t)(k & 0xffffu);
-        if (a.cost[v])
-            a.cost[v][i] = float(uint32_t(k >> 32)) / (float(region_size(a.arms[v], a.W, i, a.order == 1)) * a.S);
+    for (int j = 0; j < kLoads; j++) {
+        const int k = (kRow ? lane : warp) + (kRow ? 32 : kEY) * j;   // position in the walk's reach
+        const int qx = kRow ? kEX * bx - L1 + k : x, qy = kRow ? y : kEY * by - L1 + k;
+        q[j] = make_uchar4(0, 0, 0, 0);
+        if (k < (kRow ? kEX : kEY) + 2 * L1 && qx >= 0 && qx < W && qy >= 0 && qy < H)
+            q[j] = arms[(size_t)qy * W + qx];
+    }
+    const bool in = x < W && y < H;
+    const size_t i = (size_t)min(y, H - 1) * W + min(x, W - 1);
+    const unsigned long long key = view ? a.best[1][i] : a.best[0][i];
+    const uchar4 p = arms[i];
+#pragma unroll
+    for (int j = 0; j < kLoads; j++) {
+        const int k = (kRow ? lane : warp) + (kRow ? 32 : kEY) * j;
+        if (k < (kRow ? kEX : kEY) + 2 * L1)
+            len_s[kRow ? warp * kPitch + k : k * kPitch + lane] = kRow ? q[j].z + q[j].w + 1 : q[j].x + q[j].y + 1;
+    }
+    __syncthreads();
+    if (!in) return;
+    const int d = (int)(key & 0xffffu);
+    if (int16_t *disp = view ? a.disp[1] : a.disp[0]) disp[i] = (int16_t)d;
+    if (view == 0 && a.out) a.out[i] = checked(a, i, x, d);
+    if (float *cost = view ? a.cost[1] : a.cost[0]) {
+        const int first = kRow ? -(int)p.x : -(int)p.z, last = kRow ? p.y : p.w;
+        const uint16_t *n = kRow ? len_s + warp * kPitch + L1 + lane : len_s + (L1 + warp) * kPitch + lane;
+        uint32_t size = 0;
+#pragma unroll 8
+        for (int k = first; k <= last; k++) size += n[k * (kRow ? 1 : kPitch)];
+        cost[i] = float(uint32_t(key >> 32)) / (float(size) * a.S);
     }
 }
 
@@ -1755,7 +1795,16 @@ __global__ void __launch_bounds__(256) k_end(const __grid_constant__ Batch<EndAr
     pdl_enter();
     int bx, by, bz;
     const int i = batch_pair(b, blockIdx.x, bx, by, bz);
-    end_body(b.p[i], (size_t)bx * 256 + threadIdx.x, b.p[i].views == 2 ? by : -1);
+    end_body(b.p[i], (size_t)bx * 256 + threadIdx.x);
+}
+
+template <int N, bool kRow>
+__global__ void __launch_bounds__(kEX * kEY) k_end_costs(const __grid_constant__ Batch<EndArgs, N> b)
+{
+    pdl_enter();
+    int bx, by, bz;
+    const int i = batch_pair(b, blockIdx.x, bx, by, bz);
+    end_costs_body<kRow>(b.p[i], bx, by, bz);
 }
 
 template <int N>
@@ -2635,7 +2684,7 @@ dco_status launch_jobs(dco_stereo *h, const dco_params &p, const Derived &dv, st
     if ((st = launch_prep(h, p, dv, jobs, 2, s)) != DCO_OK) return st;
     for (int pass = 0; pass < maxpass; pass++)
         if ((st = launch_pass(h, dv, jobs, pass, s)) != DCO_OK) return st;
-    std::vector<Item<EndArgs>> end;
+    std::vector<Item<EndArgs>> end, end_costs;
     for (const Job &j : jobs) {
         if (!j.out && !j.disp_l && !j.disp_r && !j.cost_l && !j.cost_r) continue;
         Item<EndArgs> it{};
@@ -2645,11 +2694,20 @@ dco_status launch_jobs(dco_stereo *h, const dco_params &p, const Derived &dv, st
         }
         it.a.disp[0] = j.disp_l; it.a.disp[1] = j.disp_r; it.a.out = j.out;
         it.a.cost[0] = j.cost_l; it.a.cost[1] = j.cost_r;
-        it.a.W = j.W; it.a.H = j.H; it.a.tol = p.lr_tol; it.a.order = dv.order; it.a.S = dv.S;
-        it.a.views = j.cost_l || j.cost_r ? 2 : 1;   // blocks of their own for each view's region sums
-        it.gx = (j.W * j.H + 255) / 256; it.gy = it.a.views; it.gz = 1;
-        end.push_back(it);
+        it.a.W = j.W; it.a.H = j.H; it.a.tol = p.lr_tol; it.a.L1 = dv.L1; it.a.S = dv.S;
+        if (j.cost_l || j.cost_r) {
+            it.gx = (j.W + kEX - 1) / kEX; it.gy = (j.H + kEY - 1) / kEY; it.gz = 2;
+            end_costs.push_back(it);
+        } else {
+            it.gx = (j.W * j.H + 255) / 256; it.gy = 1; it.gz = 1;
+            end.push_back(it);
+        }
     }
+    st = dv.order == 1 ? launch_items(h, s, "k_end", k_end_costs<1, true>, k_end_costs<kBatchMax, true>, end_costs,
+                                      kEX * kEY, 0)
+                       : launch_items(h, s, "k_end", k_end_costs<1, false>, k_end_costs<kBatchMax, false>, end_costs,
+                                      kEX * kEY, 0);
+    if (st != DCO_OK) return st;
     if ((st = launch_items(h, s, "k_end", k_end<1>, k_end<kBatchMax>, end, 256, 0)) != DCO_OK) return st;
     return p.vote_iters > 0 ? run_vote(h, p, dv, jobs, s) : DCO_OK;
 }

@@ -138,8 +138,7 @@ struct EndArgs {
     const uchar4 *arms[2];
     int16_t *disp[2], *out;
     float *cost[2];
-    int W, H, tol, order;
-    int views;             // blocks per pixel range: 1, or one per view
+    int W, H, tol, L1;
     float S;
 };
 
