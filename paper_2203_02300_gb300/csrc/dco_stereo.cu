@@ -2063,6 +2063,7 @@ VGeom vagg_geom(int E, int F, int layers, int want, int blocks)
 struct dco_stereo {
     int device = 0;
     int nsm = 152;                           // multiprocessors of the device
+    bool yield = false;                      // launches of blocks that end after one unit of work (serving, see srv_launch)
     size_t budget = 0;
     char *ws = nullptr;
     size_t ws_cap = 0;
@@ -2494,7 +2495,8 @@ void deal_v_blocks(const dco_stereo *h, std::vector<Item<VArgs>> &it, int L1, bo
         all += double(vagg_units(row_scan ? b.a.H : b.a.W, b.gz)) * (row_scan ? b.a.W : b.a.H);
     for (auto &b : it) {
         const int E = row_scan ? b.a.W : b.a.H, F = row_scan ? b.a.H : b.a.W;
-        const int mine = std::max(1, (int)(slots * (double(vagg_units(F, b.gz)) * E / all)));
+        int mine = std::max(1, (int)(slots * (double(vagg_units(F, b.gz)) * E / all)));
+        if (h->yield) mine = std::max(mine, (int)vagg_units(F, b.gz));   // a strip each
         const VGeom g = vagg_geom(E, F, b.gz, b.gy, mine);
         b.a.strips = g.strips;
         b.a.nblk = g.nblk; b.a.rounds = g.rounds; b.a.rest = g.rest; b.a.share = g.share; b.a.bands = g.bands;
@@ -2572,7 +2574,7 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
                                csm[kv.first])) != DCO_OK)
             return st;
     if ((st = launch_items(h, s, "k_hagg", k_hagg<1>, k_hagg<kBatchMax>, hb, kHWarps * 32, hsm::total,
-                           2 * h->nsm)) != DCO_OK)
+                           h->yield ? INT_MAX : 2 * h->nsm)) != DCO_OK)
         return st;
     st = vh ? launch_items(h, s, "k_hwta", k_vagg<1, false, true, false>,
                                       k_vagg<kBatchMax, false, true, false>, vb, kVThreads, vsm)
