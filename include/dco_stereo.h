@@ -146,7 +146,8 @@ void dco_stereo_destroy(dco_stereo *h);
 size_t dco_stereo_workspace_bytes(int W, int H, int D, const dco_params *p);
 
 /* Allocate the workspace for (W, H, D, p) now.  DCO_EBUDGET if it exceeds
- * the handle's budget. */
+ * the handle's budget.  Automatic passes (d_chunk 0) are narrowed where the
+ * budget or the device cannot hold the wide ones. */
 dco_status dco_stereo_reserve(dco_stereo *h, int W, int H, int D, const dco_params *p);
 
 /*
@@ -378,11 +379,14 @@ dco_status dco_stereo_stream_status(dco_stereo *h, dco_stream stream);
  * DCO_ETIMEOUT.  DCO_TEST_LOSE_GRID_ARRIVAL: in the one-launch
  * densification solve, block 0 never arrives at the first grid barrier and
  * every barrier waits only a few polls, so all blocks give up and return;
- * dco_stereo_densify returns DCO_ETIMEOUT.  0 restores normal operation.
+ * dco_stereo_densify returns DCO_ETIMEOUT.  DCO_TEST_REFUSE_WIDE: workspace
+ * of automatic passes wider than 96 MiB of slices is refused as if the device
+ * could not allocate it.  0 restores normal operation.
  * Unknown bits: DCO_EINVAL.
  */
 #define DCO_TEST_LOSE_TILE_COPIES 1
 #define DCO_TEST_LOSE_GRID_ARRIVAL 4
+#define DCO_TEST_REFUSE_WIDE 8
 dco_status dco_stereo_set_test_flags(dco_stereo *h, int flags);
 
 /*

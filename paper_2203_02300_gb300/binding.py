@@ -25,6 +25,7 @@ STATUS = {0: "DCO_OK", 1: "DCO_EINVAL", 2: "DCO_ENOMEM", 3: "DCO_EBUDGET", 4: "D
 DCO_OK, DCO_EINVAL, DCO_ENOMEM, DCO_EBUDGET, DCO_ECUDA, DCO_ETIMEOUT, DCO_EDEVICE = range(7)
 DCO_TEST_LOSE_TILE_COPIES = 1   # failure test flags (include/dco_stereo.h)
 DCO_TEST_LOSE_GRID_ARRIVAL = 4
+DCO_TEST_REFUSE_WIDE = 8
 
 
 class Params(ctypes.Structure):

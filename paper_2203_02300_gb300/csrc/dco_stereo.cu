@@ -1915,6 +1915,11 @@ bool dims_valid(int W, int H, int D, int dmin = 0)
 // (about the L2) is what the serving lanes admit frames by, and the fallback
 // where the device cannot allocate the wide one.
 constexpr size_t kSlicesWide = 512u << 20, kSlicesNarrow = 96u << 20;
+// all pairs of a call together: from 33 pairs on, the wide cap of each is its
+// part of this (at least the narrow one), so that a batch's workspace stays
+// bounded by what narrow passes or 16 GiB of slices take
+constexpr size_t kSlicesCall = size_t(16) << 30;
+size_t wide_cap(size_t pairs) { return std::max(kSlicesNarrow, std::min(kSlicesWide, kSlicesCall / std::max<size_t>(1, pairs))); }
 int auto_width(int W, int H, int D, size_t cap)
 {
     const size_t per = 8 * (size_t)W * H;   // slice bytes per disparity
@@ -2067,6 +2072,7 @@ struct dco_stereo {
     size_t budget = 0;
     char *ws = nullptr;
     size_t ws_cap = 0;
+    size_t ws_refused = SIZE_MAX;            // smallest workspace of wide passes that the device could not allocate
     int *d_status = nullptr;
     float *d_tables = nullptr;
     float *h_tables = nullptr;   // pinned staging of the tables
@@ -2187,7 +2193,8 @@ struct ProfScope {
     }
 };
 
-dco_status ensure_ws(dco_stereo *h, size_t need)
+// keep: a workspace that the device cannot enlarge stays as it is
+dco_status ensure_ws(dco_stereo *h, size_t need, bool keep = false)
 {
     if (need <= h->ws_cap) return DCO_OK;
     if (h->budget && need > h->budget) {
@@ -2195,13 +2202,24 @@ dco_status ensure_ws(dco_stereo *h, size_t need)
                         std::to_string(h->budget);
         return DCO_EBUDGET;
     }
-    if (h->ws) {
+    char *old = h->ws;
+    if (old && !keep) {
         DCO_CUDA(h, cudaDeviceSynchronize());
-        cudaFree(h->ws);
-        h->ws = nullptr;
+        cudaFree(old);
+        h->ws = old = nullptr;
         h->ws_cap = 0;
     }
-    DCO_CUDA(h, cudaMalloc((void **)&h->ws, need));
+    char *ws = nullptr;
+    DCO_CUDA(h, cudaMalloc((void **)&ws, need));
+    if (old) {
+        const cudaError_t e = cudaDeviceSynchronize();
+        if (e != cudaSuccess) {
+            cudaFree(ws);
+            return cuda_fail(h, e, "cudaDeviceSynchronize()");
+        }
+        cudaFree(old);
+    }
+    h->ws = ws;
     h->ws_cap = need;
     return DCO_OK;
 }
@@ -2339,7 +2357,7 @@ struct Job {
 
 // workspace plan for all jobs; the pass width shrinks (same for all pairs)
 // until the plan fits the handle's budget
-dco_status plan_jobs(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs, size_t &total, size_t cap = kSlicesWide)
+size_t plan_jobs(const dco_stereo *h, const dco_params &p, std::vector<Job> &jobs, size_t cap)
 {
     // a pair's own pass width (j.dchunk > 0) replaces the call's; a budget
     // override caps both
@@ -2354,28 +2372,80 @@ dco_status plan_jobs(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs,
         }
         return t;
     };
-    total = plan(0);
+    size_t total = plan(0);
     if (h->budget && total > h->budget) {
         int widest = 32;
         for (auto &j : jobs) widest = std::max(widest, (j.L.dc + 31) / 32 * 32);
         for (int dc = widest; dc >= 32 && total > h->budget; dc -= 32) total = plan(dc);
     }
+    return total;
+}
+
+// Jobs that run together, and the workspace that the largest group needs.  On
+// a handle with a budget, jobs whose workspaces do not fit it together (even
+// at the narrowest pass width) are admitted in consecutive groups that do.
+struct Plan {
+    std::vector<std::vector<Job>> groups;
+    size_t need = 0;
+};
+
+dco_status make_plan(dco_stereo *h, const dco_params &p, const std::vector<Job> &jobs, size_t cap, size_t front, Plan &plan)
+{
+    plan.groups.assign(1, jobs);
+    plan.need = plan_jobs(h, p, plan.groups[0], cap);
+    if (h->budget && plan.need > h->budget && jobs.size() > 1) {
+        plan.groups.clear();
+        plan.need = 0;
+        for (size_t i = 0; i < jobs.size();) {
+            std::vector<Job> g{jobs[i]};
+            size_t t = plan_jobs(h, p, g, cap);
+            if (t > h->budget) {
+                h->last_error = "pair " + std::to_string(i) + " needs " + std::to_string(t) +
+                                " bytes of workspace, more than the budget of " + std::to_string(h->budget);
+                return DCO_EBUDGET;
+            }
+            size_t j = i + 1;
+            for (; j < jobs.size(); j++) {
+                std::vector<Job> g2 = g;
+                g2.push_back(jobs[j]);
+                const size_t t2 = plan_jobs(h, p, g2, cap);
+                if (t2 > h->budget) break;
+                g.swap(g2);
+                t = t2;
+            }
+            plan.need = std::max(plan.need, t);
+            plan.groups.push_back(std::move(g));
+            i = j;
+        }
+    }
+    plan.need += front;
+    for (auto &g : plan.groups)
+        for (auto &j : g) j.base += front;
     return DCO_OK;
 }
 
-// workspace for the planned jobs, behind `front` bytes of the call's own.  Wide
-// passes are a choice: where the device or the budget cannot hold them, the
-// jobs are planned again with narrow ones.
-dco_status plan_ws(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs, size_t &total, size_t front = 0)
+// Plan of a call and its workspace, behind `front` bytes of the call's own.
+// Wide passes are a choice: where the device or the budget cannot hold them,
+// the call runs with narrow ones.  A size that the device refused is not asked
+// for again while the workspace holds the narrow plan, so a call that has run
+// once allocates nothing the next time; a call that needs more than there is in any
+// case, and dco_stereo_reserve, try the wide plan afresh.
+dco_status plan_ws(dco_stereo *h, const dco_params &p, const std::vector<Job> &jobs, Plan &plan, size_t front = 0)
 {
-    dco_status st = ensure_ws(h, total + front);
-    if (st == DCO_ENOMEM || st == DCO_EBUDGET) {
-        plan_jobs(h, p, jobs, total, kSlicesNarrow);
-        for (auto &j : jobs) j.base += front;
-        return ensure_ws(h, total + front);
+    dco_status st = make_plan(h, p, jobs, wide_cap(jobs.size()), front, plan);
+    if (st == DCO_OK && plan.need <= h->ws_cap) return DCO_OK;
+    Plan narrow;
+    const dco_status nst = make_plan(h, p, jobs, kSlicesNarrow, front, narrow);
+    const bool choice = nst == DCO_OK && narrow.need < plan.need, fits = choice && narrow.need <= h->ws_cap;
+    if (st == DCO_OK) {
+        if (choice && (h->test_flags & DCO_TEST_REFUSE_WIDE)) st = DCO_ENOMEM;
+        else if (fits && plan.need >= h->ws_refused) st = DCO_ENOMEM;
+        else st = ensure_ws(h, plan.need, fits);
+        if (st == DCO_ENOMEM && choice) h->ws_refused = std::min(h->ws_refused, plan.need);
     }
-    for (auto &j : jobs) j.base += front;
-    return st;
+    if (!choice || (st != DCO_ENOMEM && st != DCO_EBUDGET)) return st;
+    plan = std::move(narrow);
+    return ensure_ws(h, plan.need);
 }
 
 template <class T>
@@ -2716,52 +2786,20 @@ dco_status launch_jobs(dco_stereo *h, const dco_params &p, const Derived &dv, st
     return p.vote_iters > 0 ? run_vote(h, p, dv, jobs, s) : DCO_OK;
 }
 
-// the whole path for a set of independent pairs: one launch per stage.  On a
-// handle with a budget, pairs whose workspaces do not fit it together (even
-// at the narrowest pass width) are admitted in consecutive groups that do;
-// the groups run one after the other on the stream, each reusing the same
-// workspace.  Every group is planned before anything is enqueued.
-dco_status run_jobs(dco_stereo *h, const dco_params &p, std::vector<Job> &jobs, cudaStream_t s)
+// the whole path for a set of independent pairs: one launch per stage.  The
+// groups that a budget makes run one after the other on the stream, each
+// reusing the same workspace.  Every group is planned before anything is
+// enqueued.
+dco_status run_jobs(dco_stereo *h, const dco_params &p, const std::vector<Job> &jobs, cudaStream_t s)
 {
     Derived dv;
     derive(p, dv);
-    size_t total = 0;
-    dco_status st = plan_jobs(h, p, jobs, total);
+    Plan plan;
+    dco_status st = plan_ws(h, p, jobs, plan);
     if (st != DCO_OK) return st;
-    if (!h->budget || total <= h->budget || jobs.size() == 1) {
-        if ((st = plan_ws(h, p, jobs, total)) != DCO_OK) return st;
-        if ((st = ensure_tables(h, p, dv, s)) != DCO_OK) return st;
-        return launch_jobs(h, p, dv, jobs, s);
-    }
-    std::vector<std::vector<Job>> groups;
-    size_t need = 0;
-    for (size_t i = 0; i < jobs.size();) {
-        std::vector<Job> g{jobs[i]};
-        size_t t = 0;
-        plan_jobs(h, p, g, t);
-        if (t > h->budget) {
-            h->last_error = "pair " + std::to_string(i) + " needs " + std::to_string(t) +
-                            " bytes of workspace, more than the budget of " + std::to_string(h->budget);
-            return DCO_EBUDGET;
-        }
-        size_t j = i + 1;
-        for (; j < jobs.size(); j++) {
-            std::vector<Job> g2 = g;
-            g2.push_back(jobs[j]);
-            size_t t2 = 0;
-            plan_jobs(h, p, g2, t2);
-            if (t2 > h->budget) break;
-            g.swap(g2);
-            t = t2;
-        }
-        need = std::max(need, t);
-        groups.push_back(std::move(g));
-        i = j;
-    }
-    if ((st = ensure_ws(h, need)) != DCO_OK) return st;
     if ((st = ensure_tables(h, p, dv, s)) != DCO_OK) return st;
-    h->groups_last = (int)groups.size();
-    for (auto &g : groups)
+    if (plan.groups.size() > 1) h->groups_last = (int)plan.groups.size();
+    for (auto &g : plan.groups)
         if ((st = launch_jobs(h, p, dv, g, s)) != DCO_OK) return st;
     return DCO_OK;
 }
@@ -2896,12 +2934,13 @@ dco_status dco_stereo_reserve(dco_stereo *h, int W, int H, int D, const dco_para
     dco_status st = check_common(h, pin, p);
     if (st != DCO_OK) return st;
     if (!dims_valid(W, H, D, p.d_min)) return DCO_EINVAL;
-    // under a budget, the widest automatic passes that fit it
+    if (p.d_chunk > 0) return ensure_ws(h, make_layout(W, H, D, p).total);
+    // the widest automatic passes that the budget and the device allow
     std::vector<Job> jobs(1);
     jobs[0].W = W; jobs[0].H = H; jobs[0].D = D;
-    size_t total = make_layout(W, H, D, p).total;
-    if (p.d_chunk == 0 && h->budget && total > h->budget) plan_jobs(h, p, jobs, total);
-    return ensure_ws(h, total);
+    h->ws_refused = SIZE_MAX;
+    Plan plan;
+    return plan_ws(h, p, jobs, plan);
 }
 
 dco_status dco_stereo_match_views(dco_stereo *h, const uint8_t *left, const uint8_t *right, int W, int H,
@@ -2991,10 +3030,8 @@ static dco_status prep_one(dco_stereo *h, const dco_params &p, const uint8_t *rg
     jobs.assign(1, Job{});
     Job &j = jobs[0];
     j.left = rgb; j.right = rgb; j.W = W; j.H = H; j.D = 1; j.arms0 = arms_out;
-    size_t total = 0;
-    dco_status st = plan_jobs(h, p, jobs, total);
+    dco_status st = ensure_ws(h, plan_jobs(h, p, jobs, kSlicesNarrow));
     if (st != DCO_OK) return st;
-    if ((st = ensure_ws(h, total)) != DCO_OK) return st;
     if ((st = ensure_tables(h, p, dv, s)) != DCO_OK) return st;
     return launch_prep(h, p, dv, jobs, 1, s);
 }
@@ -3042,14 +3079,13 @@ dco_status dco_stereo_vote(dco_stereo *h, const uint8_t *rgb, const int16_t *dis
     std::vector<Job> jobs(1);
     Job &j = jobs[0];
     j.left = rgb; j.right = rgb; j.W = W; j.H = H; j.D = D; j.out = disp_out;
-    size_t total = 0;
-    if ((st = plan_jobs(h, p, jobs, total)) != DCO_OK) return st;
-    if ((st = plan_ws(h, p, jobs, total)) != DCO_OK) return st;
+    Plan plan;
+    if ((st = plan_ws(h, p, jobs, plan)) != DCO_OK) return st;
     if ((st = ensure_tables(h, p, dv, s)) != DCO_OK) return st;
-    if ((st = launch_prep(h, p, dv, jobs, 1, s)) != DCO_OK) return st;   // arms of rgb
+    if ((st = launch_prep(h, p, dv, plan.groups[0], 1, s)) != DCO_OK) return st;   // arms of rgb
     if (disp_in != disp_out)
         DCO_CUDA(h, cudaMemcpyAsync(disp_out, disp_in, sizeof(int16_t) * W * H, cudaMemcpyDeviceToDevice, s));
-    return run_vote(h, p, dv, jobs, s);
+    return run_vote(h, p, dv, plan.groups[0], s);
 }
 
 dco_status dco_stereo_downscale(dco_stereo *h, const uint8_t *rgb, int W, int H, uint8_t *out, dco_stream stream)
@@ -3079,13 +3115,12 @@ dco_status dco_stereo_depth(dco_stereo *h, const uint8_t *left, const uint8_t *r
     Derived dv;
     derive(p, dv);
     std::vector<Job> jobs(1);
-    Job &j = jobs[0];
-    j.W = Wh; j.H = Hh; j.D = D;
-    size_t total = 0;
-    if ((st = plan_jobs(h, p, jobs, total)) != DCO_OK) return st;
+    jobs[0].W = Wh; jobs[0].H = Hh; jobs[0].D = D;
+    Plan plan;
     // in front of the pair's workspace: the two half-size images and the map
     const size_t img = align_up(3 * (size_t)Wh * Hh), front = 2 * img + align_up(2 * (size_t)Wh * Hh);
-    if ((st = plan_ws(h, p, jobs, total, front)) != DCO_OK) return st;
+    if ((st = plan_ws(h, p, jobs, plan, front)) != DCO_OK) return st;
+    Job &j = plan.groups[0][0];
     if ((st = ensure_tables(h, p, dv, s)) != DCO_OK) return st;
     DownArgs da{};
     da.src[0] = left; da.src[1] = right;
@@ -3098,7 +3133,7 @@ dco_status dco_stereo_depth(dco_stereo *h, const uint8_t *left, const uint8_t *r
         launch_pdl(k_down, dim3((unsigned)((Wh + 255) / 256), (unsigned)Hh, 2), dim3(256), 0, s, da);
         DCO_CUDA(h, cudaGetLastError());
     }
-    if ((st = launch_jobs(h, p, dv, jobs, s)) != DCO_OK) return st;
+    if ((st = launch_jobs(h, p, dv, plan.groups[0], s)) != DCO_OK) return st;
     DepthArgs za{};
     za.disp = j.out; za.out = depth_out; za.W = W; za.H = H; za.fb = (float)(f_px * baseline);
     ProfScope ps(h, s, "k_depth");
@@ -3183,7 +3218,7 @@ dco_status dco_stereo_stream_status(dco_stereo *h, dco_stream stream)
 
 dco_status dco_stereo_set_test_flags(dco_stereo *h, int flags)
 {
-    if (!h || (flags & ~(DCO_TEST_LOSE_TILE_COPIES | DCO_TEST_LOSE_GRID_ARRIVAL))) return DCO_EINVAL;
+    if (!h || (flags & ~(DCO_TEST_LOSE_TILE_COPIES | DCO_TEST_LOSE_GRID_ARRIVAL | DCO_TEST_REFUSE_WIDE))) return DCO_EINVAL;
     h->test_flags = flags;
     return DCO_OK;
 }
