@@ -1285,6 +1285,7 @@ constexpr int kVSub = 8;         // rows per warp and step
 constexpr int kVStep = kVWarps * kVSub;
 constexpr int kVRow = 512;       // ring bytes per row: 32 lanes x 16
 constexpr int kVTile = 128;      // reduction tile: bytes per output row (4 columns x 8 words)
+constexpr int kVResident = 4;   // blocks per SM that the registers allow (128 each)
 constexpr int kVHalf = 2;        // output rows whose window ends are loaded together (4 and 8: 1-2 % slower)
 // the output rows of a step read back to 2 L1 + 1 rows above it
 __host__ __device__ inline uint32_t vagg_ring_bytes(int L1)
@@ -1756,7 +1757,7 @@ __global__ void __launch_bounds__(kHWarps * 32, 2) k_hagg(const __grid_constant_
 }
 
 template <int N, bool kMax, bool kRow, bool kVol>
-__global__ void __launch_bounds__(kVThreads, 4) k_vagg(const __grid_constant__ Batch<VArgs, N> b)
+__global__ void __launch_bounds__(kVThreads, kVResident) k_vagg(const __grid_constant__ Batch<VArgs, N> b)
 {
     pdl_enter();
     int bx, by, bz;
@@ -2552,29 +2553,43 @@ dco_status launch_prep(dco_stereo *h, const dco_params &p, const Derived &dv, co
     return launch_items(h, s, "k_smooth", k_smooth<1, true>, k_smooth<kBatchMax, true>, di, 256, 0);
 }
 
-// pass `pass` (disparities [pass*dc, pass*dc + dc)) of every job that has it.
-// Pairs are bucketed by block size (warps per block) so no block carries
-// idle warps for a larger pair; one launch per bucket and stage.
-// Deals the resident V blocks of a launch out to its pairs by their work
-// (strips x rows; a pair's own v_chunk in it[].gy, the layers in it[].gz).
+// blocks of k_vagg that are resident at once: by the ring in shared memory, and
+// by the registers (the deal for arm_l1 <= 19 counted five to eight blocks per SM by the
+// ring alone: 640x480, D = 64, arm_l1 = 17 51.4 us, with four 43.2)
+int vagg_slots(const dco_stereo *h, int L1)
+{
+    return h->nsm * std::max(1, std::min(kVResident, (int)(kSmShared / (vagg_smem_bytes(L1) + kBlockShared))));
+}
+
+// Deals the resident V blocks of a launch (of at most kBatchMax pairs) out to its
+// pairs by their work (strips x rows; a pair's own v_chunk in it[].gy, the layers
+// in it[].gz).
 void deal_v_blocks(const dco_stereo *h, std::vector<Item<VArgs>> &it, int L1, bool row_scan)
 {
-    const int slots = h->nsm * std::max(1, (int)(kSmShared / (vagg_smem_bytes(L1) + kBlockShared)));
-    double all = 0.0;
-    for (auto &b : it)
-        all += double(vagg_units(row_scan ? b.a.H : b.a.W, b.gz)) * (row_scan ? b.a.W : b.a.H);
-    for (auto &b : it) {
-        const int E = row_scan ? b.a.W : b.a.H, F = row_scan ? b.a.H : b.a.W;
-        int mine = std::max(1, (int)(slots * (double(vagg_units(F, b.gz)) * E / all)));
-        if (h->yield) mine = std::max(mine, (int)vagg_units(F, b.gz));   // a strip each
-        const VGeom g = vagg_geom(E, F, b.gz, b.gy, mine);
-        b.a.strips = g.strips;
-        b.a.nblk = g.nblk; b.a.rounds = g.rounds; b.a.rest = g.rest; b.a.share = g.share; b.a.bands = g.bands;
-        b.gx = g.nblk;
-        b.gy = b.gz = 1;
+    const int slots = vagg_slots(h, L1);
+    for (size_t i0 = 0; i0 < it.size(); i0 += kBatchMax) {
+        const size_t i1 = std::min(it.size(), i0 + kBatchMax);
+        double all = 0.0;
+        for (size_t i = i0; i < i1; i++) {
+            const Item<VArgs> &b = it[i];
+            all += double(vagg_units(row_scan ? b.a.H : b.a.W, b.gz)) * (row_scan ? b.a.W : b.a.H);
+        }
+        for (size_t i = i0; i < i1; i++) {
+            Item<VArgs> &b = it[i];
+            const int E = row_scan ? b.a.W : b.a.H, F = row_scan ? b.a.H : b.a.W;
+            int mine = std::max(1, (int)(slots * (double(vagg_units(F, b.gz)) * E / all)));
+            if (h->yield) mine = std::max(mine, (int)vagg_units(F, b.gz));   // a strip each
+            const VGeom g = vagg_geom(E, F, b.gz, b.gy, mine);
+            b.a.strips = g.strips;
+            b.a.nblk = g.nblk; b.a.rounds = g.rounds; b.a.rest = g.rest; b.a.share = g.share; b.a.bands = g.bands;
+            b.gx = g.nblk;
+            b.gy = b.gz = 1;
+        }
     }
 }
 
+// pass `pass` (disparities [pass*dc, pass*dc + dc)) of every job that has it.
+// k_vcost: pairs are bucketed by warps per block, one launch per bucket.
 dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> &jobs, int pass, cudaStream_t s)
 {
     std::map<int, std::vector<Item<HArgs>>> cb;   // k_vcost, by warps per block

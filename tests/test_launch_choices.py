@@ -1,0 +1,73 @@
+"""The choice of kernels and the deal of their blocks by the size of a launch:
+maps and costs are the same whichever runs, and no size pays for the rule of
+another (ratios of kernel times of the same process).
+"""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2203_02300_gb300 import scenes
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2203_02300_gb300 import binding
+    if not torch.cuda.is_available():
+        pytest.fail("no CUDA device")
+    st = binding.Stereo(0)
+    yield torch, binding, st
+    st.close()
+
+
+def _pair(torch, W, H, D, seed=1, d_min=0):
+    if W < 16:
+        left, right = scenes.random_pair(W, H, W + H)
+    else:
+        s = scenes.plane_scene(W, H, d_min + D, 4, seed=scenes.seed_for(8, 100 + seed), noise_sigma=2.0, texture="mixed",
+                               drange=(d_min, d_min + D - 1))
+        left, right = s.left, s.right
+    return left, right, torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda()
+
+
+def _us(torch, st, kernels, call, reps=9):
+    """Device time of one call's launches of these kernels: the shortest of three means."""
+    call()
+    torch.cuda.synchronize()
+    st.set_profiling(True)
+    best = float("inf")
+    for _ in range(3):
+        st.profile_reset()
+        for _ in range(reps):
+            call()
+        prof = st.profile()
+        best = min(best, 1e3 * sum(prof[k][1] for k in kernels.split()) / reps)
+    st.set_profiling(False)
+    return best
+
+
+def test_short_arms_are_dealt_to_the_blocks_that_are_resident(env):
+    # a shorter ring must not be slower for being dealt to blocks that the
+    # registers do not let in: 0.98 of the long arms' time when it was, 0.85 since
+    torch, binding, st = env
+    _, _, L, R = _pair(torch, 640, 480, 64)
+    t = {L1: _us(torch, st, "k_vagg", lambda p=binding.Params.default(arm_l1=L1, arm_l2=L1 // 2): st.match(L, R, 64, p))
+         for L1 in (8, 34)}
+    assert t[8] < 0.92 * t[34], t
+
+
+def test_batches_beyond_one_launch_keep_the_device_full(env):
+    # pairs 65 .. 128 are a launch of their own: 1.76 times two launches of 64 when
+    # the blocks were dealt over the call
+    torch, binding, st = env
+    _, _, L, R = _pair(torch, 320, 240, 32)
+    pairs = [(L, R, 32, torch.empty((240, 320), dtype=torch.int16, device="cuda")) for _ in range(128)]
+    t = {n: _us(torch, st, "k_vagg", lambda n=n: st.match_batch(pairs[:n])) for n in (64, 128)}
+    assert t[128] < 2 * 1.3 * t[64], t
+    for p in pairs[1:]:
+        assert torch.equal(p[3], pairs[0][3])
