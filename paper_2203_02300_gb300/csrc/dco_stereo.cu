@@ -1298,26 +1298,7 @@ __host__ __device__ inline size_t vagg_smem_bytes(int L1)
 }
 static_assert(((2 * kMaxL1 + kVSub) / kVSub * kVSub + kVStep) * kVRow <= 1 << 16, "k_vagg: ring offsets in 16 bits");
 
-// N(p) of Eq. 2: the segment lengths along p's second arm (cost volumes)
-__device__ __forceinline__ uint32_t region_size(const uchar4 *arms, int W, size_t i, bool row_order)
-{
-    const uchar4 p = arms[i];
-    uint32_t n = 0;
-    if (!row_order)
-#pragma unroll 16
-        for (int k = -(int)p.z; k <= (int)p.w; k++) {
-            const uchar4 q = arms[(ptrdiff_t)i + (ptrdiff_t)k * W];
-            n += q.x + q.y + 1u;
-        }
-    else
-        for (int k = -(int)p.x; k <= (int)p.y; k++) {
-            const uchar4 q = arms[(ptrdiff_t)i + k];
-            n += q.z + q.w + 1u;
-        }
-    return n;
-}
-
-template <bool kMax, bool kRow, bool kVol>
+template <bool kMax, bool kRow>
 __device__ __forceinline__ void vagg_body(const VArgs &a, int blk)
 {
     extern __shared__ __align__(128) uint8_t vring[];
@@ -1481,16 +1462,6 @@ __device__ __forceinline__ void vagg_body(const VArgs &a, int blk)
                     for (int u = 0; u < kVHalf; u++) {
                         const int r = r0 + u;
                         uint32_t c[4] = {hi[u].x - lo[u].x, hi[u].y - lo[u].y, hi[u].z - lo[u].z, hi[u].w - lo[u].w};
-                        if (kVol && view == a.vol_view && line < F && y + r < ye) {
-                            const size_t p = pix0 + (size_t)(y + r) * pstep;
-                            const uint32_t n =
-                                region_size(reinterpret_cast<const uchar4 *>(view ? a.arms[1] : a.arms[0]), a.W, p, kRow);
-#pragma unroll
-                            for (int j = 0; j < 4; j++)
-                                if (4 * dq + j < nlive)
-                                    a.vol[(size_t)(dbase + 4 * dq + j - a.dmin) * a.H * a.W + p] =
-                                        float(c[j]) / (float(n) * a.S);
-                        }
 #pragma unroll
                         for (int j = 0; j < 4; j++)
                             if (kMax) c[j] = 0x7fffffffu - c[j];
@@ -1536,6 +1507,144 @@ __device__ __forceinline__ void vagg_body(const VArgs &a, int blk)
         }
         __syncthreads();   // the ring is the next run's
     }
+}
+
+// ------------------------------------------------------------------ k_vcol
+// The same second sum and winner, a block per line, for cost volumes.  Block = one column x of one view (kRow: one
+// row y), a chunk of output rows and their reach; a warp per 32 rows.  Per
+// group of 32 disparities:
+//   0. the warp's 32 slice rows (128 bytes each) into its rows of Q by 16-byte
+//      asynchronous copies, all in flight;
+//   A. lane = disparity: the rows into registers, their sum exchanged with the
+//      other warps, and the column prefix in their place;
+//   C. lane = output row: V(d) = Q(y + down, d) - Q(y - up - 1, d), four
+//      disparities per 16-byte load, the running minimum with the smallest d
+//      on ties in registers across the groups.
+// One store per pixel and pass (a line belongs to one block), and N(p) of
+// Eq. 2 from a prefix of the segment lengths.  Q rows are 36 words: 32 rows of 16-byte loads spread over the banks.
+// A cost volume of 640x480, D = 64 takes 162 us here; summing N(p) from the arms
+// for every group, as the strips would have to, 369.
+constexpr int kQS = 36;        // Q row stride in words
+constexpr int kColSeg = 32;    // rows per warp
+constexpr int kColMax = 512;   // rows of a block's prefix range (16 warps)
+// words: Q[-1] (zeros), Q [nw * 32], T [nw][32], NQ [nw * 32], NT [nw]
+__host__ __device__ inline size_t vcol_smem_bytes(int nw) { return 4 * (size_t)(kQS + nw * (kColSeg * (kQS + 2) + 1)); }
+
+template <bool kMax, bool kRow>
+__device__ __forceinline__ void vcol_body(const VArgs &a, int fix, int view, int part)
+{
+    extern __shared__ __align__(16) uint32_t vsmem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int W = a.W, H = a.H, L1 = a.L1;
+    const int E = kRow ? W : H;
+    const int ys = part * a.chunk, ye = min(E, ys + a.chunk);
+    const int ya = max(0, ys - L1), len = min(E, ye + L1) - ya;
+    const size_t pix0 = kRow ? (size_t)fix * W : (size_t)fix, pstep = kRow ? 1 : (size_t)W;   // pixels along the line
+    uint32_t *Q = vsmem + kQS, *T = Q + nw * kColSeg * kQS, *NQ = T + nw * 32, *NT = NQ + nw * kColSeg;
+    const uint32_t *arms = reinterpret_cast<const uint32_t *>(view ? a.arms[1] : a.arms[0]) + pix0;
+    const size_t step = pstep * (size_t)a.dstride;
+    const int r = warp * kColSeg + lane;   // the lane's row, relative to ya
+    // group g's rows of the warp into its rows of Q: eight lanes per row, four
+    // rows per instruction.  Rows past the range keep what they held: they are
+    // summed after its last row, and the last warp's total is read by no other.
+    const uint32_t *src = (view ? a.sh[1] : a.sh[0]) +
+                          (pix0 + (size_t)(ya + warp * kColSeg + (lane >> 3)) * pstep) * a.dstride + 4 * (lane & 7);
+    uint32_t *dst = Q + (warp * kColSeg + (lane >> 3)) * kQS + 4 * (lane & 7);
+    const int nrow = len - warp * kColSeg - (lane >> 3);   // copied: the lane's rows 4 i < nrow
+    auto load = [&](int g) {
+#pragma unroll
+        for (int i = 0; i < kColSeg / 4; i++)
+            if (4 * i < nrow) cp_async16(dst + 4 * i * kQS, src + (size_t)(4 * i) * step + 32 * g);
+    };
+    load(0);
+    const uint32_t aw = r < len ? __ldg(arms + (size_t)(ya + r) * pstep) : 0u;
+    const int back = kRow ? aw & 0xffu : (aw >> 16) & 0xffu, fwd = kRow ? (aw >> 8) & 0xffu : aw >> 24;
+    const bool vol = a.vol != nullptr && view == a.vol_view;
+    if (vol) {   // the prefix of the segment lengths (the other arms)
+        uint32_t n = r >= len ? 0u : kRow ? ((aw >> 16) & 0xffu) + (aw >> 24) + 1u : (aw & 0xffu) + ((aw >> 8) & 0xffu) + 1u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, n, o);
+            if (lane >= o) n += t;
+        }
+        if (lane == 31) NT[warp] = n;
+        __syncthreads();
+        for (int w = 0; w < warp; w++) n += NT[w];
+        NQ[r] = n;   // (read after the barriers below)
+    }
+    if (warp == 0) vsmem[lane] = 0u;   // Q[-1]: read by rows whose arm reaches the line's start
+    const bool out = r < len && ya + r >= ys && ya + r < ye;
+    const uint4 *qh = reinterpret_cast<const uint4 *>(Q + (r + fwd) * kQS);
+    const uint4 *ql = reinterpret_cast<const uint4 *>(Q + (r - back - 1) * kQS);
+    uint32_t bv = 0xffffffffu, bd = 0;
+    for (int g = 0; g < a.ng; g++) {
+        // ---- A
+        cp_async_wait_all();
+        __syncwarp();
+        uint32_t *q = Q + warp * kColSeg * kQS + lane;
+        uint32_t v[kColSeg], tot = 0;
+#pragma unroll
+        for (int u = 0; u < kColSeg; u++) {
+            v[u] = q[u * kQS];
+            tot += v[u];
+        }
+        T[warp * 32 + lane] = tot;
+        __syncthreads();
+        uint32_t run = 0;
+        for (int w = 0; w < warp; w++) run += T[w * 32 + lane];
+#pragma unroll
+        for (int u = 0; u < kColSeg; u++) {
+            run += v[u];
+            q[u * kQS] = run;
+        }
+        __syncthreads();
+        // ---- C
+        const int dbase = a.d0 + 32 * g, nlive = min(32, min(a.dc - 32 * g, a.D - dbase));
+        if (out) {
+            uint32_t bj = 0xffffffffu, bmin = bv;   // strict <: the smallest d on ties
+            auto quad = [&](int j4, int live) {
+                const uint4 h = qh[j4], l = ql[j4];
+                const uint32_t c[4] = {h.x - l.x, h.y - l.y, h.z - l.z, h.w - l.w};
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    const uint32_t s = k < live ? (kMax ? 0x7fffffffu - c[k] : c[k]) : 0xffffffffu;
+                    bj = s < bmin ? (uint32_t)(4 * j4 + k) : bj;
+                    bmin = min(bmin, s);
+                }
+                return make_uint4(c[0], c[1], c[2], c[3]);
+            };
+            if (vol) {
+                const float n = float(NQ[r + fwd] - (r > back ? NQ[r - back - 1] : 0u));
+                float *o = a.vol + (size_t)(dbase - a.dmin) * H * W + pix0 + (size_t)(ya + r) * pstep;
+                for (int j4 = 0; 4 * j4 < nlive; j4++) {
+                    const uint4 w = quad(j4, nlive - 4 * j4);
+                    const uint32_t c[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int k = 0; k < 4; k++)
+                        if (4 * j4 + k < nlive) o[(size_t)(4 * j4 + k) * H * W] = float(c[k]) / (n * a.S);
+                }
+            } else if (nlive == 32) {
+#pragma unroll 2
+                for (int j4 = 0; j4 < 8; j4++) quad(j4, 4);
+            } else {
+                for (int j4 = 0; 4 * j4 < nlive; j4++) quad(j4, nlive - 4 * j4);
+            }
+            if (bj != 0xffffffffu) {
+                bv = bmin;
+                bd = (uint32_t)dbase + bj;
+            }
+        }
+        if (g + 1 < a.ng) {
+            __syncthreads();   // Q and T are the next group's
+            load(g + 1);
+        }
+    }
+    if (!out) return;
+    const size_t i = pix0 + (size_t)(ya + r) * pstep;
+    unsigned long long *best = (view ? a.best[1] : a.best[0]) + i;
+    unsigned long long key = ((unsigned long long)bv << 32) | bd;
+    if (!a.first) key = min(key, *best);   // (of the earlier passes)
+    *best = key;
 }
 
 // ------------------------------------------------------------------ k_lr
@@ -1756,13 +1865,22 @@ __global__ void __launch_bounds__(kHWarps * 32, 2) k_hagg(const __grid_constant_
     });
 }
 
-template <int N, bool kMax, bool kRow, bool kVol>
+template <int N, bool kMax, bool kRow>
 __global__ void __launch_bounds__(kVThreads, kVResident) k_vagg(const __grid_constant__ Batch<VArgs, N> b)
 {
     pdl_enter();
     int bx, by, bz;
     const int i = batch_pair(b, blockIdx.x, bx, by, bz);
-    vagg_body<kMax, kRow, kVol>(b.p[i], bx);
+    vagg_body<kMax, kRow>(b.p[i], bx);
+}
+
+template <int N, bool kMax, bool kRow>
+__global__ void __launch_bounds__(kColMax, 2) k_vcol(const __grid_constant__ Batch<VArgs, N> b)
+{
+    pdl_enter();
+    int bx, by, bz;
+    const int i = batch_pair(b, blockIdx.x, bx, by, bz);
+    vcol_body<kMax, kRow>(b.p[i], bx, by, bz);
 }
 
 template <int N>
@@ -2588,29 +2706,81 @@ void deal_v_blocks(const dco_stereo *h, std::vector<Item<VArgs>> &it, int L1, bo
     }
 }
 
+// k_vcol's grids (b.gy: a pair's own v_chunk, b.gz: layers), by warps per block
+std::map<int, std::vector<Item<VArgs>>> deal_lines(const std::vector<Item<VArgs>> &it, int L1, bool row_scan)
+{
+    std::map<int, std::vector<Item<VArgs>>> out;
+    for (Item<VArgs> b : it) {
+        const int E = row_scan ? b.a.W : b.a.H, want = b.gy > 0 ? b.gy : E;
+        const int most = want >= E && E <= kColMax ? E : std::min(want, kColMax - 2 * L1);
+        const int parts = (E + most - 1) / most;   // balanced
+        b.a.chunk = (E + parts - 1) / parts;
+        b.gx = row_scan ? b.a.H : b.a.W;
+        b.gy = b.gz / b.a.ng;
+        b.gz = (E + b.a.chunk - 1) / b.a.chunk;
+        const int len = std::min(E, b.a.chunk + 2 * L1);
+        out[(len + kColSeg - 1) / kColSeg].push_back(b);
+    }
+    return out;
+}
+
+template <bool kMax, bool kRow>
+dco_status launch_second(dco_stereo *h, const char *name, std::vector<Item<VArgs>> &it, bool lines, int L1, cudaStream_t s)
+{
+    if (!lines) {
+        deal_v_blocks(h, it, L1, kRow);
+        return launch_items(h, s, name, k_vagg<1, kMax, kRow>, k_vagg<kBatchMax, kMax, kRow>, it, kVThreads,
+                            vagg_smem_bytes(L1));
+    }
+    for (const auto &kv : deal_lines(it, L1, kRow)) {
+        const dco_status st = launch_items(h, s, name, k_vcol<1, kMax, kRow>, k_vcol<kBatchMax, kMax, kRow>, kv.second,
+                                           32 * kv.first, vcol_smem_bytes(kv.first));
+        if (st != DCO_OK) return st;
+    }
+    return DCO_OK;
+}
+
 // pass `pass` (disparities [pass*dc, pass*dc + dc)) of every job that has it.
-// k_vcost: pairs are bucketed by warps per block, one launch per bucket.
+// k_vcost and k_vcol: pairs are bucketed by warps per block, one launch per bucket.
 dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> &jobs, int pass, cudaStream_t s)
 {
     std::map<int, std::vector<Item<HArgs>>> cb;   // k_vcost, by warps per block
     std::map<int, size_t> csm;
     std::vector<Item<HArgs>> hb;
     std::vector<Item<VArgs>> vb, vvol;
-    const size_t vsm = vagg_smem_bytes(dv.L1);
-    const bool vh = dv.order == 1;   // vertical segment sums first (k_vcost), then rows (k_vagg<.., kRow>)
+    const bool vh = dv.order == 1;   // vertical segment sums first (k_vcost), then rows (kRow)
     for (const Job &j : jobs) {
         if (pass >= j.L.npass) continue;
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
         const int ng = (dc + 31) / 32;
-        const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk, vw = j.vchunk > 0 ? j.vchunk : dv.vchunk;
-        const bool single = j.L.npass == 1 && ng == 1;
+        Item<VArgs> b{};
+        for (int v = 0; v < 2; v++) {
+            b.a.sh[v] = jptr<uint32_t>(h, j, j.L.sh[v]);
+            b.a.arms[v] = jptr<uchar4>(h, j, j.L.arms[v]);
+            b.a.best[v] = jptr<unsigned long long>(h, j, j.L.best[v]);
+        }
+        b.a.vol = j.vol; b.a.vol_view = j.vol_view;
+        b.a.W = j.W; b.a.H = j.H; b.a.D = dv.dmin + j.D; b.a.dmin = dv.dmin;
+        b.a.d0 = d0; b.a.dc = dc; b.a.dstride = j.L.dstride;
+        b.a.ng = ng; b.a.single = j.L.npass == 1 && ng == 1; b.a.first = pass == 0;
+        b.a.L1 = dv.L1; b.a.S = dv.S;
+        b.gy = j.vchunk > 0 ? j.vchunk : dv.vchunk;
+        b.gz = 2 * ng;
+        (j.vol ? vvol : vb).push_back(b);
+    }
+    for (const Job &j : jobs) {
+        if (pass >= j.L.npass) continue;
+        const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
+        const int ng = (dc + 31) / 32;
+        const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk;
+        const bool init = pass == 0 && !j.vol && !(j.L.npass == 1 && ng == 1);
         Item<HArgs> a{};
         for (int v = 0; v < 2; v++) {
             a.a.cen[v] = jptr<uint2>(h, j, j.L.cen[v]);
             a.a.col[v] = jptr<uint32_t>(h, j, j.L.col[v]);
             a.a.arms[v] = jptr<uchar4>(h, j, j.L.arms[v]);
             a.a.sh[v] = jptr<uint32_t>(h, j, j.L.sh[v]);
-            a.a.init[v] = pass == 0 && !single ? jptr<unsigned long long>(h, j, j.L.best[v]) : nullptr;
+            a.a.init[v] = init ? jptr<unsigned long long>(h, j, j.L.best[v]) : nullptr;
         }
         a.a.pw = j.L.pw;
         a.a.status = h->d_status;
@@ -2636,23 +2806,7 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
             a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = hg.grid.z;
             hb.push_back(a);
         }
-        Item<VArgs> b{};
-        for (int v = 0; v < 2; v++) {
-            b.a.sh[v] = a.a.sh[v];
-            b.a.arms[v] = a.a.arms[v];
-            b.a.best[v] = jptr<unsigned long long>(h, j, j.L.best[v]);
-        }
-        b.a.vol = j.vol; b.a.vol_view = j.vol_view;
-        b.a.W = j.W; b.a.H = j.H; b.a.D = dv.dmin + j.D; b.a.dmin = dv.dmin;
-        b.a.d0 = d0; b.a.dc = dc; b.a.dstride = j.L.dstride;
-        b.a.ng = ng; b.a.single = single;
-        b.a.L1 = dv.L1; b.a.S = dv.S;
-        b.gy = vw;
-        b.gz = 2 * ng;
-        (j.vol ? vvol : vb).push_back(b);
     }
-    deal_v_blocks(h, vb, dv.L1, vh);
-    deal_v_blocks(h, vvol, dv.L1, vh);
     dco_status st;
     for (auto &kv : cb)
         if ((st = launch_items(h, s, "k_vcost", k_vcost<1>, k_vcost<kBatchMax>, kv.second, kv.first * 32,
@@ -2661,18 +2815,12 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
     if ((st = launch_items(h, s, "k_hagg", k_hagg<1>, k_hagg<kBatchMax>, hb, kHWarps * 32, hsm::total,
                            h->yield ? INT_MAX : 2 * h->nsm)) != DCO_OK)
         return st;
-    st = vh ? launch_items(h, s, "k_hwta", k_vagg<1, false, true, false>,
-                                      k_vagg<kBatchMax, false, true, false>, vb, kVThreads, vsm)
-                       : launch_items(h, s, "k_vagg", k_vagg<1, false, false, false>,
-                                      k_vagg<kBatchMax, false, false, false>, vb, kVThreads, vsm);
-    if (st != DCO_OK) return st;
-    // (a cost volume is asked for one pair at a time)
-    for (const auto &it : vvol) {
-        st = vh ? launch_group<VArgs, 1>(h, s, "k_hwta", k_vagg<1, false, true, true>, &it, 1, kVThreads, vsm)
-                : launch_group<VArgs, 1>(h, s, "k_vagg", k_vagg<1, false, false, true>, &it, 1, kVThreads, vsm);
-        if (st != DCO_OK) return st;
+    if (vh) {
+        if ((st = launch_second<false, true>(h, "k_hwta", vb, false, dv.L1, s)) != DCO_OK) return st;
+        return launch_second<false, true>(h, "k_hwta", vvol, true, dv.L1, s);
     }
-    return DCO_OK;
+    if ((st = launch_second<false, false>(h, "k_vagg", vb, false, dv.L1, s)) != DCO_OK) return st;
+    return launch_second<false, false>(h, "k_vagg", vvol, true, dv.L1, s);
 }
 
 dco_status launch_lr(dco_stereo *h, const std::vector<Item<LrArgs>> &items, cudaStream_t s)
@@ -2689,19 +2837,34 @@ dco_status launch_vote_pass(dco_stereo *h, const Derived &dv, const std::vector<
     std::map<int, std::vector<Item<HVArgs>>> hb;
     std::vector<Item<VArgs>> vb;
     std::map<int, size_t> hsm;
-    const size_t vsm = vagg_smem_bytes(dv.L1);
     for (const Job &j : jobs) {
         if (!j.vbest || pass >= j.L.npass) continue;
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
         const int ng = (dc + 31) / 32;
-        const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk, vw = j.vchunk > 0 ? j.vchunk : dv.vchunk;
+        Item<VArgs> b{};
+        b.a.sh[0] = jptr<uint32_t>(h, j, j.L.sh[0]);
+        b.a.arms[0] = jptr<uchar4>(h, j, j.L.arms[0]);
+        b.a.best[0] = j.vbest;
+        b.a.W = j.W; b.a.H = j.H; b.a.D = dv.dmin + j.D; b.a.dmin = dv.dmin;
+        b.a.d0 = d0; b.a.dc = dc; b.a.dstride = j.L.dstride;
+        b.a.ng = ng; b.a.single = j.L.npass == 1 && ng == 1; b.a.first = pass == 0;
+        b.a.L1 = dv.L1; b.a.S = dv.S;
+        b.gy = j.vchunk > 0 ? j.vchunk : dv.vchunk;
+        b.gz = ng;   // the left view only
+        vb.push_back(b);
+    }
+    for (const Job &j : jobs) {
+        if (!j.vbest || pass >= j.L.npass) continue;
+        const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
+        const int ng = (dc + 31) / 32;
+        const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk;
         const HGeom hg = hvote_geom(j.W, j.H, dc, dv.L1, hw);
-        const bool single = j.L.npass == 1 && ng == 1;
+        const bool init = pass == 0 && !(j.L.npass == 1 && ng == 1);
         hsm[hg.nw] = std::max(hsm[hg.nw], hg.smem);
         Item<HVArgs> a{};
         a.a.disp = j.out;
         a.a.keys = j.vkeys;
-        a.a.init = pass == 0 && !single ? j.vbest : nullptr;
+        a.a.init = init ? j.vbest : nullptr;
         a.a.dmin = dv.dmin; a.a.D = dv.dmin + j.D;
         a.a.arms = jptr<uchar4>(h, j, j.L.arms[0]);
         a.a.sh = jptr<uint32_t>(h, j, j.L.sh[0]);
@@ -2709,26 +2872,13 @@ dco_status launch_vote_pass(dco_stereo *h, const Derived &dv, const std::vector<
         a.a.L1 = dv.L1; a.a.chunk = hg.chunk;
         a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = hg.grid.z;
         hb[hg.nw].push_back(a);
-        Item<VArgs> b{};
-        b.a.sh[0] = a.a.sh;
-        b.a.arms[0] = a.a.arms;
-        b.a.best[0] = j.vbest;
-        b.a.W = j.W; b.a.H = j.H; b.a.D = dv.dmin + j.D; b.a.dmin = dv.dmin;
-        b.a.d0 = d0; b.a.dc = dc; b.a.dstride = j.L.dstride;
-        b.a.ng = ng; b.a.single = single;
-        b.a.L1 = dv.L1; b.a.S = dv.S;
-        b.gy = vw;
-        b.gz = ng;   // the left view only
-        vb.push_back(b);
     }
-    deal_v_blocks(h, vb, dv.L1, false);
     for (auto &kv : hb) {
         dco_status st = launch_items(h, s, "k_hvote", k_hvote<1>, k_hvote<kBatchMax>, kv.second, kv.first * 32,
                                      hsm[kv.first]);
         if (st != DCO_OK) return st;
     }
-    return launch_items(h, s, "k_vvote", k_vagg<1, true, false, false>, k_vagg<kBatchMax, true, false, false>, vb, kVThreads,
-                        vsm);
+    return launch_second<true, false>(h, "k_vvote", vb, false, dv.L1, s);
 }
 
 // p.vote_iters rounds of Eq. 4 on every job's final map (j.out, in place).

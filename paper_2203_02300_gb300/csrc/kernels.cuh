@@ -123,7 +123,9 @@ struct VArgs {
     int dmin;              // smallest disparity of the search
     int d0, dc, dstride;   // this pass covers d in [d0, d0 + dc)
     int ng;                // 32-disparity groups in the pass
-    int single;            // the only pass and group: keys are stored, not minimised
+    int single;            // k_vagg: the only pass and group: keys are stored, not minimised
+    int first;             // k_vcol: the first pass: keys are stored, else minimised
+    int chunk;             // k_vcol: output rows per block
     int L1;
     int strips;            // strips of four columns per layer (group and view)
     int nblk, rounds;      // blocks; whole strips per block

@@ -71,3 +71,24 @@ def test_batches_beyond_one_launch_keep_the_device_full(env):
     assert t[128] < 2 * 1.3 * t[64], t
     for p in pairs[1:]:
         assert torch.equal(p[3], pairs[0][3])
+
+
+@pytest.mark.parametrize("W,H,D,d_min", [(33, 513, 7, 0), (40, 1100, 33, 2), (513, 31, 20, 0), (600, 20, 70, 5), (7, 3, 2, 0)])
+@pytest.mark.parametrize("order", [0, 1])
+def test_cost_volumes_of_long_lines_and_partial_groups(env, W, H, D, d_min, order):
+    torch, binding, st = env
+    left, right, L, R = _pair(torch, W, H, D, W, d_min)
+    ref = O.match(left, right, D, O.Params(agg_order=order, d_min=d_min), volume=True)
+    for d_chunk in (0, 32):   # one pass, and passes that merge their winners
+        p = binding.Params.default(agg_order=order, d_min=d_min, d_chunk=d_chunk)
+        for view, want in ((0, ref.vol_l), (1, ref.vol_r)):
+            parity.check_volume(st.cost_volume(L, R, D, view, p).cpu().numpy(), want,
+                                f"volume {W}x{H} D={D} order {order} view {view}")
+
+
+def test_a_cost_volume_takes_region_sizes_once(env):
+    # 7 times the match's second pass when N(p) was summed again for every group
+    torch, binding, st = env
+    _, _, L, R = _pair(torch, 640, 480, 64)
+    vol = _us(torch, st, "k_vagg", lambda: st.cost_volume(L, R, 64, 0))
+    assert vol < 5 * _us(torch, st, "k_vagg", lambda: st.match(L, R, 64))
