@@ -1510,7 +1510,9 @@ __device__ __forceinline__ void vagg_body(const VArgs &a, int blk)
 }
 
 // ------------------------------------------------------------------ k_vcol
-// The same second sum and winner, a block per line, for cost volumes.  Block = one column x of one view (kRow: one
+// The same second sum and winner, a block per line: for launches whose strips
+// of k_vagg do not fill the SMs (a walk is then one long chain of steps on an
+// idle chip), and for cost volumes.  Block = one column x of one view (kRow: one
 // row y), a chunk of output rows and their reach; a warp per 32 rows.  Per
 // group of 32 disparities:
 //   0. the warp's 32 slice rows (128 bytes each) into its rows of Q by 16-byte
@@ -1521,7 +1523,11 @@ __device__ __forceinline__ void vagg_body(const VArgs &a, int blk)
 //      disparities per 16-byte load, the running minimum with the smallest d
 //      on ties in registers across the groups.
 // One store per pixel and pass (a line belongs to one block), and N(p) of
-// Eq. 2 from a prefix of the segment lengths.  Q rows are 36 words: 32 rows of 16-byte loads spread over the banks.
+// Eq. 2 from a prefix of the segment lengths, so costs and volumes are written
+// here.  Q rows are 36 words: 32 rows of 16-byte loads spread over the banks.
+// Bound by latency: a copy, two block barriers and a row's window per group, all
+// blocks resident at once.  Against the strips (event times, us): 96x64, D = 16 8.3
+// -> 6.9; 320x240, D = 32 14.3 -> 11.9, D = 64 18.6 -> 16.3; 333x211, D = 50 18.4 -> 14.6.
 // A cost volume of 640x480, D = 64 takes 162 us here; summing N(p) from the arms
 // for every group, as the strips would have to, 369.
 constexpr int kQS = 36;        // Q row stride in words
@@ -1559,8 +1565,9 @@ __device__ __forceinline__ void vcol_body(const VArgs &a, int fix, int view, int
     load(0);
     const uint32_t aw = r < len ? __ldg(arms + (size_t)(ya + r) * pstep) : 0u;
     const int back = kRow ? aw & 0xffu : (aw >> 16) & 0xffu, fwd = kRow ? (aw >> 8) & 0xffu : aw >> 24;
+    float *cost = view ? a.cost[1] : a.cost[0];
     const bool vol = a.vol != nullptr && view == a.vol_view;
-    if (vol) {   // the prefix of the segment lengths (the other arms)
+    if (cost || vol) {   // the prefix of the segment lengths (the other arms)
         uint32_t n = r >= len ? 0u : kRow ? ((aw >> 16) & 0xffu) + (aw >> 24) + 1u : (aw & 0xffu) + ((aw >> 8) & 0xffu) + 1u;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1645,6 +1652,10 @@ __device__ __forceinline__ void vcol_body(const VArgs &a, int fix, int view, int
     unsigned long long key = ((unsigned long long)bv << 32) | bd;
     if (!a.first) key = min(key, *best);   // (of the earlier passes)
     *best = key;
+    if (cost) {
+        const uint32_t n = NQ[r + fwd] - (r > back ? NQ[r - back - 1] : 0u);
+        cost[i] = float(uint32_t(key >> 32)) / (float(n) * a.S);
+    }
 }
 
 // ------------------------------------------------------------------ k_lr
@@ -2470,6 +2481,7 @@ struct Job {
     int host_in = -1;                // images in host memory: 1, in device memory: 0, -1: ask the driver
     const unsigned long long *vkeys = nullptr;   // Eq. 4 round: the previous round's keys (null: first round)
     unsigned long long *vbest = nullptr;         //   and the keys it minimises into
+    bool costs_done = false;   // the second pass wrote the costs
     Layout L{};
     size_t base = 0;           // workspace offset of this pair
 };
@@ -2679,6 +2691,23 @@ int vagg_slots(const dco_stereo *h, int L1)
     return h->nsm * std::max(1, std::min(kVResident, (int)(kSmShared / (vagg_smem_bytes(L1) + kBlockShared))));
 }
 
+// The second pass of a launch: strips (k_vagg) or whole lines (k_vcol).  Lines where
+// every one fits a block (a v_chunk asks for strips) and their warps, counted once per
+// group, are at most 110 per SM (k_vcol holds 32 at once): the strips' long walks
+// then leave the chip idle.  Strips against lines, us, by that count: 69 (320x240,
+// D = 64) 18.6, 16.3; 105 (400x300, D = 64) 23.3, 20.7; 126 (480x320, D = 64) 24.8, 24.8;
+// 126 (640x480, D = 32) 25.4, 28.7; 152 (480x360, D = 64) 27.4, 31.0.
+bool whole_lines(const dco_stereo *h, const std::vector<Item<VArgs>> &it, bool row_scan)
+{
+    size_t warps = 0;
+    for (const auto &b : it) {
+        const int E = row_scan ? b.a.W : b.a.H, F = row_scan ? b.a.H : b.a.W;
+        if (b.gy > 0 || E > kColMax) return false;
+        warps += (size_t)F * b.gz * ((E + kColSeg - 1) / kColSeg);
+    }
+    return warps <= 110 * (size_t)h->nsm;
+}
+
 // Deals the resident V blocks of a launch (of at most kBatchMax pairs) out to its
 // pairs by their work (strips x rows; a pair's own v_chunk in it[].gy, the layers
 // in it[].gz).
@@ -2742,7 +2771,7 @@ dco_status launch_second(dco_stereo *h, const char *name, std::vector<Item<VArgs
 
 // pass `pass` (disparities [pass*dc, pass*dc + dc)) of every job that has it.
 // k_vcost and k_vcol: pairs are bucketed by warps per block, one launch per bucket.
-dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> &jobs, int pass, cudaStream_t s)
+dco_status launch_pass(dco_stereo *h, const Derived &dv, std::vector<Job> &jobs, int pass, cudaStream_t s)
 {
     std::map<int, std::vector<Item<HArgs>>> cb;   // k_vcost, by warps per block
     std::map<int, size_t> csm;
@@ -2768,12 +2797,23 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
         b.gz = 2 * ng;
         (j.vol ? vvol : vb).push_back(b);
     }
-    for (const Job &j : jobs) {
+    const bool lines = whole_lines(h, vb, vh);
+    size_t nv = 0;
+    for (Job &j : jobs) {
         if (pass >= j.L.npass) continue;
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
         const int ng = (dc + 31) / 32;
         const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk;
-        const bool init = pass == 0 && !j.vol && !(j.L.npass == 1 && ng == 1);
+        const bool by_line = lines || j.vol;
+        const bool init = pass == 0 && !by_line && !(j.L.npass == 1 && ng == 1);
+        if (!j.vol) {   // k_vcol knows the costs with the last pass's keys
+            j.costs_done = lines && pass == j.L.npass - 1;
+            if (j.costs_done) {
+                vb[nv].a.cost[0] = j.cost_l;
+                vb[nv].a.cost[1] = j.cost_r;
+            }
+            nv++;
+        }
         Item<HArgs> a{};
         for (int v = 0; v < 2; v++) {
             a.a.cen[v] = jptr<uint2>(h, j, j.L.cen[v]);
@@ -2816,10 +2856,10 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, const std::vector<Job> 
                            h->yield ? INT_MAX : 2 * h->nsm)) != DCO_OK)
         return st;
     if (vh) {
-        if ((st = launch_second<false, true>(h, "k_hwta", vb, false, dv.L1, s)) != DCO_OK) return st;
+        if ((st = launch_second<false, true>(h, "k_hwta", vb, lines, dv.L1, s)) != DCO_OK) return st;
         return launch_second<false, true>(h, "k_hwta", vvol, true, dv.L1, s);
     }
-    if ((st = launch_second<false, false>(h, "k_vagg", vb, false, dv.L1, s)) != DCO_OK) return st;
+    if ((st = launch_second<false, false>(h, "k_vagg", vb, lines, dv.L1, s)) != DCO_OK) return st;
     return launch_second<false, false>(h, "k_vagg", vvol, true, dv.L1, s);
 }
 
@@ -2853,13 +2893,14 @@ dco_status launch_vote_pass(dco_stereo *h, const Derived &dv, const std::vector<
         b.gz = ng;   // the left view only
         vb.push_back(b);
     }
+    const bool lines = whole_lines(h, vb, false);
     for (const Job &j : jobs) {
         if (!j.vbest || pass >= j.L.npass) continue;
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
         const int ng = (dc + 31) / 32;
         const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk;
         const HGeom hg = hvote_geom(j.W, j.H, dc, dv.L1, hw);
-        const bool init = pass == 0 && !(j.L.npass == 1 && ng == 1);
+        const bool init = pass == 0 && !lines && !(j.L.npass == 1 && ng == 1);
         hsm[hg.nw] = std::max(hsm[hg.nw], hg.smem);
         Item<HVArgs> a{};
         a.a.disp = j.out;
@@ -2878,7 +2919,7 @@ dco_status launch_vote_pass(dco_stereo *h, const Derived &dv, const std::vector<
                                      hsm[kv.first]);
         if (st != DCO_OK) return st;
     }
-    return launch_second<true, false>(h, "k_vvote", vb, false, dv.L1, s);
+    return launch_second<true, false>(h, "k_vvote", vb, lines, dv.L1, s);
 }
 
 // p.vote_iters rounds of Eq. 4 on every job's final map (j.out, in place).
@@ -2925,16 +2966,19 @@ dco_status launch_jobs(dco_stereo *h, const dco_params &p, const Derived &dv, st
         if ((st = launch_pass(h, dv, jobs, pass, s)) != DCO_OK) return st;
     std::vector<Item<EndArgs>> end, end_costs;
     for (const Job &j : jobs) {
-        if (!j.out && !j.disp_l && !j.disp_r && !j.cost_l && !j.cost_r) continue;
+        if (!j.out && !j.disp_l && !j.disp_r && (j.costs_done || (!j.cost_l && !j.cost_r))) continue;
         Item<EndArgs> it{};
         for (int v = 0; v < 2; v++) {
             it.a.best[v] = jptr<unsigned long long>(h, j, j.L.best[v]);
             it.a.arms[v] = jptr<uchar4>(h, j, j.L.arms[v]);
         }
         it.a.disp[0] = j.disp_l; it.a.disp[1] = j.disp_r; it.a.out = j.out;
-        it.a.cost[0] = j.cost_l; it.a.cost[1] = j.cost_r;
+        if (!j.costs_done) {
+            it.a.cost[0] = j.cost_l;
+            it.a.cost[1] = j.cost_r;
+        }
         it.a.W = j.W; it.a.H = j.H; it.a.tol = p.lr_tol; it.a.L1 = dv.L1; it.a.S = dv.S;
-        if (j.cost_l || j.cost_r) {
+        if (it.a.cost[0] || it.a.cost[1]) {
             it.gx = (j.W + kEX - 1) / kEX; it.gy = (j.H + kEY - 1) / kEY; it.gz = 2;
             end_costs.push_back(it);
         } else {

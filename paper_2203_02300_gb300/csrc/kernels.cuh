@@ -126,6 +126,7 @@ struct VArgs {
     int single;            // k_vagg: the only pass and group: keys are stored, not minimised
     int first;             // k_vcol: the first pass: keys are stored, else minimised
     int chunk;             // k_vcol: output rows per block
+    float *cost[2];        // k_vcol: minimum costs (null: none), from this pass's keys
     int L1;
     int strips;            // strips of four columns per layer (group and view)
     int nblk, rounds;      // blocks; whole strips per block

@@ -92,3 +92,29 @@ def test_a_cost_volume_takes_region_sizes_once(env):
     _, _, L, R = _pair(torch, 640, 480, 64)
     vol = _us(torch, st, "k_vagg", lambda: st.cost_volume(L, R, 64, 0))
     assert vol < 5 * _us(torch, st, "k_vagg", lambda: st.match(L, R, 64))
+
+
+# sizes whose second pass runs by whole lines; h_chunk has no part in it
+@pytest.mark.parametrize("W,H,D", [(96, 64, 16), (7, 65, 3), (33, 32, 32), (65, 33, 33), (131, 97, 70), (40, 511, 40),
+                                   (41, 512, 31), (512, 20, 65)])
+@pytest.mark.parametrize("order", [0, 1])
+def test_whole_lines_equal_the_strips(env, W, H, D, order):
+    torch, binding, st = env
+    _, _, L, R = _pair(torch, W, H, D, H)
+    for d_chunk, vote in ((0, 0), (24, 0), (0, 2)):
+        over = dict(agg_order=order, d_chunk=d_chunk, vote_iters=vote, smooth_arms=vote // 2)
+        lines = st.match_views(L, R, D, binding.Params.default(**over))
+        strips = st.match_views(L, R, D, binding.Params.default(v_chunk=16384, **over))
+        for a, b in zip(lines, strips):
+            assert torch.equal(a, b), (over, W, H, D)
+
+
+@pytest.mark.parametrize("W,H,D", [(333, 211, 50), (320, 240, 64)])
+def test_small_launches_are_not_bound_by_one_strip(env, W, H, D):
+    # strips (one block each, as v_chunk asks) against the automatic choice, which also
+    # writes the costs: the same time when that was strips too
+    torch, binding, st = env
+    _, _, L, R = _pair(torch, W, H, D)
+    p = binding.Params.default(v_chunk=16384)
+    lines, strips = (_us(torch, st, "k_vagg k_end", lambda q=q: st.match_views(L, R, D, q), 25) for q in (None, p))
+    assert lines < 0.95 * strips, (lines, strips)
