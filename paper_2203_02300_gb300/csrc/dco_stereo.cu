@@ -659,17 +659,18 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t n,
 
 // ------------------------------------------------------------------ k_hagg
 // Eq. 1 costs and their horizontal segment sums (the first 1-D sum of Eq. 2).
-// Block = (row, view, 32 disparities, a range of columns), sixteen warps: warp
-// = (four disparities, half of the range).  The records of both images, the
-// arms and the tables arrive in shared memory by bulk copies on one mbarrier
+// Block = (row, view, 32 disparities, a range of columns): a warp per four
+// disparities and up to 320 columns, so eight warps for ranges of at most 320 reference
+// columns (four blocks per SM), sixteen up to 640 (two).  The records of both
+// images, the arms and the tables arrive in shared memory by bulk copies on one mbarrier
 // (bounded wait).  Then:
-//   A. a warp walks its half in segments of 160 columns (a short end in one of
-//      32), lane = five (one)
+//   A. a warp walks its part in segments of 160 columns (ends in one of 96 or
+//      32), lane = five (three, one)
 //      consecutive columns x four disparities: the reference records stay in
 //      registers and each candidate loaded serves up to four costs; costs
 //      rounded to fixed point, prefixes within the lane, a scan of the lanes'
 //      totals, and the prefixes stored as one 16-byte word per column
-//      (G[quad][x], lanes five words apart: no bank conflicts);
+//      (G[quad][x], lanes an odd number of words apart: no bank conflicts);
 //   B. every output column: S_H = G(end) - G(start), eight lanes (quads) per
 //      column, a 128-byte line of the slice per column; the planes' stride
 //      puts the eight quads of a column on distinct banks whatever the arms.
@@ -678,31 +679,34 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t n,
 // one block per task with a disparity pair per lane and sixteen-column
 // segments: 45 M instead of 52 M instructions; 640x480, D = 64, one pass 70 -> 66
 // us (the default was two passes: 82), 1280x720, D = 128 481 -> 423 us,
-// 1920x1080, D = 256 1960 -> 1875 us; rows that fill their segments badly lose
-// (333x211, D = 50 22.3 -> 23.8 us).  Both views in one block from one
+// 1920x1080, D = 256 1960 -> 1875 us.  Blocks of sixteen warps alone left half of them
+// idle on rows of up to 160 columns and an SM with two blocks in the same phase on
+// rows of up to 320: 64 pairs of 160x120, D = 32 206 us against 140 with eight warps (one
+// block per row and group before: 121), of 320x240 574 against 465 (502), 256x192,
+// D = 64 22.1 against 17.7 us (17.1).  Both views in one block from one
 // evaluation of every pixel pair (16 disparities, 96 registers, one set of
 // table gathers for two costs) took 72-75 us: 13.5 M wavefronts, but sixteen
 // warps per SM, and right-view windows that move with the disparity.
 constexpr int kHD = 32;        // disparities per block
 constexpr int kHQuads = kHD / 4;
-constexpr int kHWarps = 2 * kHQuads;
 constexpr int kHCols = 5;      // columns per lane (odd: conflict-free stores)
 constexpr int kHSegCols = 32 * kHCols;
 constexpr int kHScan = 40;     // words per value of the scan of the lanes' totals (eight lanes' 16-byte reads hit distinct banks)
-constexpr int kHMaxPairs = 4 * kHSegCols;   // reference columns per block (two blocks per SM)
-constexpr int kHPlane = kHMaxPairs + 1;     // 16-byte words per plane: odd
 constexpr int kTabBytes = kTabFloats * 4;
 
-// Byte offsets of the block's shared memory (the same for every launch): each
+// Byte offsets of the shared memory of a block of kParts warps per quad: each
 // copied range has room for its 16-byte alignment; the arms of two tasks.
-namespace hsm {
-constexpr int e = kHMaxPairs + 4, f = kHMaxPairs + kHD + 4;   // reference and candidate columns
-// (a second copy of the AD table for every other lane: 67.7 against 65.8 us at
-// 640x480, D = 64: neighbouring columns often read the same entry)
-constexpr int rcen = kTabBytes, ccen = rcen + 8 * e, rcol = ccen + 8 * f, ccol = rcol + 4 * e;
-constexpr int arm = ccol + 4 * f, arms = 4 * e, g = arm + 2 * arms;
-constexpr int total = g + kHQuads * kHPlane * 16;
-}   // namespace hsm
+template <int kParts>
+struct HSmem {
+    static constexpr int warps = kParts * kHQuads, cols = kParts * 2 * kHSegCols;   // cols: reference columns
+    static constexpr int plane = cols + 1;   // 16-byte words per plane: odd
+    static constexpr int e = cols + 4, f = cols + kHD + 4;   // reference and candidate columns
+    // (a second copy of the AD table for every other lane: 67.7 against 65.8 us at
+    // 640x480, D = 64: neighbouring columns often read the same entry)
+    static constexpr int rcen = kTabBytes, ccen = rcen + 8 * e, rcol = ccen + 8 * f, ccol = rcol + 4 * e;
+    static constexpr int arm = ccol + 4 * f, arms = 4 * e, g = arm + 2 * arms;
+    static constexpr int total = g + kHQuads * plane * 16;
+};
 
 // one unit of a block's work: a range of output columns of a row, view and group
 struct HTask {
@@ -717,12 +721,14 @@ struct HTask {
     unsigned long long *init;  // keys to set (null: none)
 };
 
-// Blocks are resident (two per SM) and take tasks in turn: the next task's
-// copies are in flight during phase B, which does not read the records.
+// Blocks are resident and take tasks in turn: the next task's copies are in
+// flight during phase B, which does not read the records.  Warp 0 prepares them (a
+// thread's chain of about a microsecond) and takes no part in B.
 // find(t, bx, by, bz): the arguments of task t and its place in their grid.
-template <class Find>
+template <int kParts, class Find>
 __device__ __forceinline__ void hagg_tasks(int ntasks, Find find)
 {
+    using hsm = HSmem<kParts>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     __shared__ __align__(8) unsigned long long hbar_s;
     __shared__ HTask task_s[2];
@@ -817,9 +823,8 @@ __device__ __forceinline__ void hagg_tasks(int ntasks, Find find)
 
         // ---- A: prefixes of the warp's quad over its half of the columns
         const int n = k.n, view = k.view;
-        // first column of the second half: whole segments, of which an end of
-        // at most 32 columns does not count
-        const int nseg = max(1, (n + kHSegCols - 33) / kHSegCols), split = min(n, (nseg + 1) / 2 * kHSegCols);
+        // first column of the second half: whole segments (of 160 and 96) before it
+        const int split = kParts == 1 ? n : n <= 352 ? min(n, 160) : n <= 448 ? 256 : 320;
         {
             const int quad = warp & (kHQuads - 1), half = warp / kHQuads, d0 = k.dlo + 4 * quad;
             const int W = k.W, p0 = k.p0, q0 = k.q0, nq = k.nq;
@@ -828,14 +833,14 @@ __device__ __forceinline__ void hagg_tasks(int ntasks, Find find)
             // indexed by candidate column - q0
             const uint2 *ccen = reinterpret_cast<const uint2 *>(smem_raw + hsm::ccen) + (q0 & 1);
             const uint32_t *ccol = reinterpret_cast<const uint32_t *>(smem_raw + hsm::ccol) + (q0 & 3);
-            uint4 *g = reinterpret_cast<uint4 *>(smem_raw + hsm::g) + quad * kHPlane;
+            uint4 *g = reinterpret_cast<uint4 *>(smem_raw + hsm::g) + quad * hsm::plane;
             const float S = k.S;
             const uint32_t one = k.Sint;
             // Cost j of column c meets candidate c + 3 - j of the lane's eight:
             // disparity d0 + j in the left view, d0 + 3 - j in the right one.
             const int cand = view ? p0 + d0 - q0 : p0 - d0 - 3 - q0;   // of relative column 0, relative to q0
             uint32_t carry = 0;   // of cost lane & 3: the prefix before the segment
-            // columns s .. s + 159 (relative); kEdge: some lie past the range, or
+            // columns s .. s + 32 kCols - 1 (relative); kEdge: some lie past the range, or
             // meet candidates outside the image
             auto segment = [&](int s, auto cols_c, auto edge_c) {
                 constexpr int kCols = decltype(cols_c)::value;
@@ -908,12 +913,13 @@ __device__ __forceinline__ void hagg_tasks(int ntasks, Find find)
                 for (int s = half ? split : 0; s < s1; s += kHSegCols) {
                     const bool inside = view ? p0 + s + kHSegCols + d0 + 3 <= W : p0 + s >= d0 + 3;
                     if (s1 - s <= 32) segment(s, std::integral_constant<int, 1>{}, std::true_type{});
+                    else if (s1 - s <= 96) segment(s, std::integral_constant<int, 3>{}, std::true_type{});
                     else if (inside && s + kHSegCols <= n) segment(s, std::integral_constant<int, kHCols>{}, std::false_type{});
                     else segment(s, std::integral_constant<int, kHCols>{}, std::true_type{});
                 }
                 if (half == 0) {
                     if (lane == 0) g[0] = make_uint4(0u, 0u, 0u, 0u);
-                    if (lane < 4) reinterpret_cast<uint32_t *>(&half_s[quad])[view ? 3 - lane : lane] = carry;
+                    if (kParts > 1 && lane < 4) reinterpret_cast<uint32_t *>(&half_s[quad])[view ? 3 - lane : lane] = carry;
                 }
             }
         }
@@ -922,22 +928,22 @@ __device__ __forceinline__ void hagg_tasks(int ntasks, Find find)
         if (threadIdx.x == 0) prepare(next, slot ^ 1);
 
         // ---- B: segment sums; lane = (column, quad)
-        const int quad = lane & (kHQuads - 1), c0 = 32 / kHQuads * warp;
-        if (k.dlo + 4 * quad < k.dend) {
-            constexpr int kStep = kHWarps * 32 / kHQuads;
+        const int quad = lane & (kHQuads - 1), c0 = 32 / kHQuads * (warp - 1);
+        if (warp > 0 && k.dlo + 4 * quad < k.dend) {
+            constexpr int kStep = (hsm::warps - 1) * 32 / kHQuads;
             const int lead = k.lead, cross = split - lead, m = k.m, col = lane / kHQuads;
-            const uint4 *g = reinterpret_cast<const uint4 *>(smem_raw + hsm::g) + quad * kHPlane + lead + col;
+            const uint4 *g = reinterpret_cast<const uint4 *>(smem_raw + hsm::g) + quad * hsm::plane + lead + col;
             const uchar4 *arm = reinterpret_cast<const uchar4 *>(smem_raw + hsm::arm + slot * hsm::arms) + k.arm + col;
             const size_t ds4 = k.ds4, ostep = kStep * ds4;
             uint4 *o = k.out + (c0 + col) * ds4 + quad;
-            const uint4 tot = half_s[quad];
+            const uint4 tot = kParts > 1 ? half_s[quad] : make_uint4(0u, 0u, 0u, 0u);
             // columns i + col
             auto sum = [&](int i) {
                 const uchar4 am = arm[i];
                 const int hi = i + am.y + 1, lo = i - am.x;
                 const uint4 h = g[hi], w = g[lo];
                 uint4 v = make_uint4(h.x - w.x, h.y - w.y, h.z - w.z, h.w - w.w);
-                if (i + kMaxL1 + 4 > cross && i - kMaxL1 <= cross) {   // near the halves' border (the same in the warp)
+                if (kParts > 1 && i + kMaxL1 + 4 > cross && i - kMaxL1 <= cross) {   // near the halves' border (the same in the warp)
                     if (hi + col > cross && lo + col <= cross) v = make_uint4(v.x + tot.x, v.y + tot.y, v.z + tot.z, v.w + tot.w);
                 }
                 return v;
@@ -1867,11 +1873,11 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_dirs(const __grid_constan
     prep_dirs_body<CW, CH>(b.p[i], bx, by, bz);
 }
 
-template <int N>
-__global__ void __launch_bounds__(kHWarps * 32, 2) k_hagg(const __grid_constant__ Batch<HArgs, N> b)
+template <int N, int kParts>
+__global__ void __launch_bounds__(HSmem<kParts>::warps * 32, 4 / kParts) k_hagg(const __grid_constant__ Batch<HArgs, N> b)
 {
     pdl_enter();
-    hagg_tasks(b.off[b.n], [&](int t, int &bx, int &by, int &bz) -> const HArgs & {
+    hagg_tasks<kParts>(b.off[b.n], [&](int t, int &bx, int &by, int &bz) -> const HArgs & {
         return b.p[batch_pair(b, t, bx, by, bz)];
     });
 }
@@ -2127,28 +2133,31 @@ HGeom hvote_geom(int W, int H, int dc, int L1, int want)
 }
 
 // k_hagg: one task per (row, view, 32 disparities, range of output columns): whole
-// rows up to kHMaxPairs columns, else ranges that fill it with their L1 reach
-// on both sides (the first has a reach on one side only)
+// rows up to what a block of sixteen warps holds, else ranges that fill it with
+// their L1 reach on both sides (the first has a reach on one side only)
 struct HaggGeom {
     int first, chunk;
+    int parts;   // warps per quad: two where a task has more than 320 reference columns
     dim3 grid;   // of tasks: rows, ranges, views and groups
 };
 
 HaggGeom hagg_geom(int W, int H, int dc, int L1, int want)
 {
+    constexpr int most = HSmem<2>::cols;
     HaggGeom g{};
-    if (W <= kHMaxPairs && (want <= 0 || want >= W)) {
+    if (W <= most && (want <= 0 || want >= W)) {
         g.first = g.chunk = W;
     } else {
-        g.chunk = kHMaxPairs - 2 * L1;
-        g.first = kHMaxPairs - L1;
+        g.chunk = most - 2 * L1;
+        g.first = most - L1;
         if (want > 0) {   // (ranges of equal length)
-            const int parts = (W + std::min(want, g.chunk) - 1) / std::min(want, g.chunk);
-            g.first = g.chunk = (W + parts - 1) / parts;
+            const int ranges = (W + std::min(want, g.chunk) - 1) / std::min(want, g.chunk);
+            g.first = g.chunk = (W + ranges - 1) / ranges;
         }
     }
-    const int parts = g.first >= W ? 1 : 1 + (W - g.first + g.chunk - 1) / g.chunk;
-    g.grid = dim3(H, parts, 2 * ((dc + kHD - 1) / kHD));
+    const int ranges = g.first >= W ? 1 : 1 + (W - g.first + g.chunk - 1) / g.chunk;
+    g.parts = (ranges == 1 ? W : std::min(W, std::max(g.first + L1, g.chunk + 2 * L1))) <= HSmem<1>::cols ? 1 : 2;
+    g.grid = dim3(H, ranges, 2 * ((dc + kHD - 1) / kHD));
     return g;
 }
 
@@ -2775,7 +2784,7 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, std::vector<Job> &jobs,
 {
     std::map<int, std::vector<Item<HArgs>>> cb;   // k_vcost, by warps per block
     std::map<int, size_t> csm;
-    std::vector<Item<HArgs>> hb;
+    std::vector<Item<HArgs>> hb[2];   // k_hagg, by warps per quad
     std::vector<Item<VArgs>> vb, vvol;
     const bool vh = dv.order == 1;   // vertical segment sums first (k_vcost), then rows (kRow)
     for (const Job &j : jobs) {
@@ -2844,7 +2853,7 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, std::vector<Job> &jobs,
             const HaggGeom hg = hagg_geom(j.W, j.H, dc, dv.L1, hw);
             a.a.chunk = hg.chunk; a.a.first = hg.first;
             a.gx = hg.grid.x; a.gy = hg.grid.y; a.gz = hg.grid.z;
-            hb.push_back(a);
+            hb[hg.parts - 1].push_back(a);
         }
     }
     dco_status st;
@@ -2852,8 +2861,11 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, std::vector<Job> &jobs,
         if ((st = launch_items(h, s, "k_vcost", k_vcost<1>, k_vcost<kBatchMax>, kv.second, kv.first * 32,
                                csm[kv.first])) != DCO_OK)
             return st;
-    if ((st = launch_items(h, s, "k_hagg", k_hagg<1>, k_hagg<kBatchMax>, hb, kHWarps * 32, hsm::total,
-                           h->yield ? INT_MAX : 2 * h->nsm)) != DCO_OK)
+    if ((st = launch_items(h, s, "k_hagg", k_hagg<1, 1>, k_hagg<kBatchMax, 1>, hb[0], HSmem<1>::warps * 32,
+                           HSmem<1>::total, h->yield ? INT_MAX : 4 * h->nsm)) != DCO_OK)
+        return st;
+    if ((st = launch_items(h, s, "k_hagg", k_hagg<1, 2>, k_hagg<kBatchMax, 2>, hb[1], HSmem<2>::warps * 32,
+                           HSmem<2>::total, h->yield ? INT_MAX : 2 * h->nsm)) != DCO_OK)
         return st;
     if (vh) {
         if ((st = launch_second<false, true>(h, "k_hwta", vb, lines, dv.L1, s)) != DCO_OK) return st;

@@ -118,3 +118,39 @@ def test_small_launches_are_not_bound_by_one_strip(env, W, H, D):
     p = binding.Params.default(v_chunk=16384)
     lines, strips = (_us(torch, st, "k_vagg k_end", lambda q=q: st.match_views(L, R, D, q), 25) for q in (None, p))
     assert lines < 0.95 * strips, (lines, strips)
+
+
+# reference columns at the edges of the first pass's blocks (320), parts (96, 160, 352, 448)
+# and segments, rows that leave disparities outside, partial groups
+@pytest.mark.parametrize("W,D,d_min,L1", [(96, 16, 0, 34), (97, 20, 10, 34), (129, 40, 0, 34), (200, 50, 3, 12), (256, 33, 0, 40),
+                                          (257, 64, 0, 34), (319, 36, 100, 34), (320, 70, 0, 34), (321, 40, 0, 34), (352, 50, 0, 1),
+                                          (353, 96, 0, 34), (416, 33, 60, 34), (448, 40, 0, 34), (449, 64, 0, 34), (577, 40, 0, 40),
+                                          (736, 40, 0, 34)])
+def test_first_pass_at_the_edges_of_its_parts(env, W, D, d_min, L1):
+    torch, binding, st = env
+    H = 11
+    left, right, L, R = _pair(torch, W, H, D, W, d_min)
+    over = dict(d_min=d_min, arm_l1=L1, arm_l2=L1 // 2)
+    got = st.match_views(L, R, D, binding.Params.default(**over))
+    for h_chunk in (50, 300):   # ranges in blocks of eight and of sixteen warps
+        for a, b in zip(got, st.match_views(L, R, D, binding.Params.default(h_chunk=h_chunk, **over))):
+            assert torch.equal(a, b), h_chunk
+    ref = O.match(left, right, D, O.Params(**over))
+    got = [t.cpu().numpy() for t in got]
+    parity.check_disparity(got[1], ref.disp_l, ref.best_l, ref.second_l, f"first pass {W} columns left")
+    parity.check_disparity(got[2], ref.disp_r, ref.best_r, ref.second_r, f"first pass {W} columns right")
+    parity.check_cost(got[3], ref.best_l, got[1], ref.disp_l, f"first pass {W} columns left cost")
+    parity.check_cost(got[4], ref.best_r, got[2], ref.disp_r, f"first pass {W} columns right cost")
+
+
+def test_short_rows_keep_the_first_pass_busy(env):
+    # the same evaluations in rows of 160 and of 640 columns: 1.7 times as long in the short ones
+    # while half of a block's warps had none of their columns, 1.2 since
+    torch, binding, st = env
+
+    def batch(n, W, H):
+        _, _, L, R = _pair(torch, W, H, 32)
+        pairs = [(L, R, 32, torch.empty((H, W), dtype=torch.int16, device="cuda")) for _ in range(n)]
+        return _us(torch, st, "k_hagg", lambda: st.match_batch(pairs))
+    short, long = batch(64, 160, 120), batch(4, 640, 480)
+    assert short < 1.45 * long, (short, long)
