@@ -1056,8 +1056,7 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
     const int ys = by * a.chunk, ye = min(H, ys + a.chunk);
     const int ya = max(0, ys - L1), yb = min(H, ye + L1), len = yb - ya;
     const CSmem L(len, a.chunk, nw);
-    const float *sTA = reinterpret_cast<const float *>(smem_raw);
-    const float *sTC = sTA + kTabAD;
+    const float *sTC = reinterpret_cast<const float *>(smem_raw) + kTabAD;   // (the AD table comes first)
     uint4 *sref = reinterpret_cast<uint4 *>(smem_raw + L.ref);
     uchar4 *sarm = reinterpret_cast<uchar4 *>(smem_raw + L.arm);   // (up, down) of the output rows
     uint32_t *P = reinterpret_cast<uint32_t *>(smem_raw + L.p);    // [len][32], P[-1] = 0
@@ -1071,10 +1070,11 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
 
     for (int i = threadIdx.x; i < kTabBytes / 16; i += blockDim.x)
         cp_async16(smem_raw + 16 * i, reinterpret_cast<const uint8_t *>(a.tables) + 16 * i);
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-        const uint2 ce = cref[(size_t)(ya + i) * a.pw];
-        const uint32_t c = kref[(size_t)(ya + i) * a.pw];
-        sref[i] = make_uint4(ce.x, ce.y, c, __float_as_uint(__ldg(a.tables + kTabAD + kTabCen + (c >> 24))));
+    // a warp stages the rows of its own segment
+    const int sa = warp * kHSegCost, sb = min(len, sa + kHSegCost), own = sa + lane;   // rows relative to ya
+    if (own < len) {
+        cp_async8(sref + own, cref + (size_t)(ya + own) * a.pw);
+        cp_async4(&sref[own].z, kref + (size_t)(ya + own) * a.pw);
     }
     for (int i = threadIdx.x; i < ye - ys; i += blockDim.x) {
         const uchar4 am = aref[(size_t)(ys + i) * W + x];
@@ -1083,6 +1083,8 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
     if (threadIdx.x < 32) P[(int)threadIdx.x - 32] = 0u;
     cp_async_wait_all();
     __syncthreads();
+    if (own < len) reinterpret_cast<float *>(&sref[own])[3] = sTC[kTabCen + (sref[own].z >> 24)];   // alpha
+    __syncwarp();
 
     const int dlo = a.d0 + 32 * g;
     const int dhi = min(min(a.d0 + a.dc, a.D), dlo + 32) - 1;
@@ -1090,45 +1092,42 @@ __device__ __forceinline__ void vcost_body(const HArgs &a, int bx, int by, int b
     const int dd = d <= dhi ? d : dlo;                // dead lanes read a real candidate, results unused
     const int xo = view ? x + dd : x - dd;            // candidate column
     const bool outside = xo < 0 || xo >= W;           // match outside the image: cost 1
-    const uint2 *ccand = coth + max(0, min(xo, W - 1));
-    const uint32_t *kcand = koth + max(0, min(xo, W - 1));
+    const uint32_t pw = (uint32_t)a.pw;
+    uint32_t at = (uint32_t)(ya + warp * kHSegCost) * pw + (uint32_t)max(0, min(xo, W - 1));   // the candidate's plane entry
     const float Sf = a.S;
     const uint32_t Sint = a.Sint;
 
     // ---- A: costs down this warp's segment of rows, local prefix
-    const int sa = warp * kHSegCost, sb = min(len, sa + kHSegCost);   // rows relative to ya
     uint32_t run = 0;
-    int u = sa;
-    for (; u + 4 <= sb; u += 4) {
-        uint2 pc[4];
-        uint32_t po[4];
+    auto rows = [&](auto edge_c) {
+        constexpr bool kEdge = decltype(edge_c)::value;   // some lane's match lies outside the image
+        int u = sa;
+        auto cost = [&](int row, uint2 pc, uint32_t po) {
+            const uint4 pr = sref[row];
+            const int hm = __popc(pr.x ^ pc.x) + __popc(pr.y ^ pc.y);
+            const uint32_t k4 = __dp4a(__vabsdiffu4(pr.z, po), 0x00040404u, 0u);   // byte offset
+            const float av = __uint_as_float(pr.w), ta = *reinterpret_cast<const float *>(smem_raw + k4);
+            const uint32_t q = __float2uint_rn(fmaf(av, ta, (Sf - av) * sTC[hm]));
+            run += kEdge && outside ? Sint : q;
+            P[row * 32 + lane] = run;
+        };
+        constexpr int kRows = 16;
+        for (; u + kRows <= sb; u += kRows) {
+            uint2 pc[kRows];
+            uint32_t po[kRows];
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
-            pc[k] = __ldg(ccand + (size_t)(ya + u + k) * a.pw);
-            po[k] = __ldg(kcand + (size_t)(ya + u + k) * a.pw);
-        }
+            for (int k = 0; k < kRows; k++) {
+                pc[k] = __ldg(coth + at);
+                po[k] = __ldg(koth + at);
+                at += pw;
+            }
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const uint4 pr = sref[u + k];
-            const int hm = __popc(pr.x ^ pc[k].x) + __popc(pr.y ^ pc[k].y);
-            const int kk = (int)__dp4a(__vabsdiffu4(pr.z, po[k]), 0x00010101u, 0u);
-            const float av = __uint_as_float(pr.w);
-            const uint32_t q = __float2uint_rn(fmaf(av, sTA[kk], (Sf - av) * sTC[hm]));
-            run += outside ? Sint : q;
-            P[(u + k) * 32 + lane] = run;
+            for (int k = 0; k < kRows; k++) cost(u + k, pc[k], po[k]);
         }
-    }
-    for (; u < sb; u++) {
-        const uint2 pc = __ldg(ccand + (size_t)(ya + u) * a.pw);
-        const uint32_t po = __ldg(kcand + (size_t)(ya + u) * a.pw);
-        const uint4 pr = sref[u];
-        const int hm = __popc(pr.x ^ pc.x) + __popc(pr.y ^ pc.y);
-        const int kk = (int)__dp4a(__vabsdiffu4(pr.z, po), 0x00010101u, 0u);
-        const float av = __uint_as_float(pr.w);
-        const uint32_t q = __float2uint_rn(fmaf(av, sTA[kk], (Sf - av) * sTC[hm]));
-        run += outside ? Sint : q;
-        P[u * 32 + lane] = run;
-    }
+        for (; u < sb; u++, at += pw) cost(u, __ldg(coth + at), __ldg(koth + at));
+    };
+    if (__any_sync(0xffffffffu, outside)) rows(std::true_type{});
+    else rows(std::false_type{});
     T[warp * 32 + lane] = run;
     __syncthreads();
     // consecutive output rows are one slice row (W * dstride words) apart

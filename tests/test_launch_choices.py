@@ -154,3 +154,13 @@ def test_short_rows_keep_the_first_pass_busy(env):
         return _us(torch, st, "k_hagg", lambda: st.match_batch(pairs))
     short, long = batch(64, 160, 120), batch(4, 640, 480)
     assert short < 1.45 * long, (short, long)
+
+
+def test_the_column_pass_of_tall_images_keeps_two_blocks_per_sm(env):
+    # order 1 at 1280x720: 2.3 times the row pass of order 0 while its registers let one
+    # block of 23 warps in, 1.8 since
+    torch, binding, st = env
+    _, _, L, R = _pair(torch, 1280, 720, 128)
+    cols = _us(torch, st, "k_vcost", lambda p=binding.Params.default(agg_order=1): st.match(L, R, 128, p))
+    rows = _us(torch, st, "k_hagg", lambda: st.match(L, R, 128))
+    assert cols < 2.0 * rows, (cols, rows)
