@@ -1692,9 +1692,9 @@ __device__ __forceinline__ void end_body(const EndArgs &a, size_t i)
 {
     if (i >= (size_t)a.W * a.H) return;
     const int d = (int)(a.best[0][i] & 0xffffu);
-    if (a.out) a.out[i] = checked(a, i, int(i % a.W), d);
     if (a.disp[0]) a.disp[0][i] = (int16_t)d;
     if (a.disp[1]) a.disp[1][i] = (int16_t)(a.best[1][i] & 0xffffu);
+    if (a.out) a.out[i] = checked(a, i, int(i % a.W), d);   // last: a caller may pass one buffer as disp_left and disp_out
 }
 
 // The same with costs, for one view: a cost is the key's sum over the region

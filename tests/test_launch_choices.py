@@ -2,6 +2,8 @@
 maps and costs are the same whichever runs, and no size pays for the rule of
 another (ratios of kernel times of the same process).
 """
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -164,3 +166,22 @@ def test_the_column_pass_of_tall_images_keeps_two_blocks_per_sm(env):
     cols = _us(torch, st, "k_vcost", lambda p=binding.Params.default(agg_order=1): st.match(L, R, 128, p))
     rows = _us(torch, st, "k_hagg", lambda: st.match(L, R, 128))
     assert cols < 2.0 * rows, (cols, rows)
+
+
+def test_one_buffer_for_the_left_view_and_the_checked_map(env):
+    # dco_stereo_match_views with disp_out == disp_left: the checked map, as the
+    # consistency check comes after the views, with and without costs
+    torch, binding, st = env
+    W, H, D = 133, 60, 24
+    _, _, L, R = _pair(torch, W, H, D)
+    p = lambda t: ctypes.c_void_p(t.data_ptr() if t is not None else None)   # noqa: E731
+    want = st.match(L, R, D)
+    assert int((want < 0).sum()) > 0
+    for params in (None, binding.Params.default(v_chunk=64)):
+        for cost in (None, torch.empty((H, W), dtype=torch.float32, device="cuda")):
+            both = torch.full((H, W), -9, dtype=torch.int16, device="cuda")
+            torch.cuda.synchronize()
+            rc = binding.lib().dco_stereo_match_views(st._h, p(L), p(R), W, H, D, ctypes.byref(params) if params else None,
+                                                      p(both), p(both), None, p(cost), None, None)
+            st.sync_status()
+            assert rc == 0 and torch.equal(both, want)
