@@ -8,16 +8,16 @@ hierarchy and the SMs (dco_params.d_chunk, h_chunk, v_chunk):
   run fewer, larger launches of the two aggregation kernels (measured on
   GB300: one pass of 64 disparities beats two of 32 at 640x480, one pass of
   256 beats eight of 32 at 1920x1080);
-- the outputs per block of the first 1-D pass and of the second: shorter
-  blocks give more, smaller blocks (a fuller last wave, more blocks per SM)
-  at the price of reading the arm_l1 halo on both sides of every block once
-  more.
+- the outputs per block of the first 1-D pass and per run of the second:
+  shorter ones give more, smaller units (a fuller last wave) at the price of
+  reading the arm_l1 halo on both sides of every unit once more, and, in the
+  second pass, of the automatic deal to the SMs.
 
 The tuner times candidates on a pair of the shape with CUDA events, one
 parameter at a time (the pass width with automatic blocks, then the first
 pass's blocks, then the second's), keeps a change only when it is faster by
 more than 1 %, and caches the winning Tile per (W, H, D, order, arm limit,
-GPU name) in a JSON file, so later processes and the batch and serving paths
+GPU name, generation of the kernels) in a JSON file, so later processes and the batch and serving paths
 reuse it (dco_pair_desc and dco_stream_desc carry a pair's tile).
 Candidates whose slices would exceed `max_slice_bytes` are not tried.  Only
 timing and bookkeeping live here; the work runs in libdco_stereo.so.
@@ -33,8 +33,9 @@ from .binding import Tile
 
 _LOCK = threading.Lock()
 MAX_SLICE_BYTES = 1 << 30   # both views' slices of one pass
-H_MAX_LEN = 1024            # prefix positions one first-pass block holds
-V_MAX_LEN = 512             # prefix positions one second-pass block holds
+H_MAX_LEN = (640, 1024)     # positions a first-pass block holds with its halo: rows (order 0), columns (1)
+V_MAX_LEN = 512             # longest run tried for the second pass (with its halo)
+KERNELS = 2                 # generation of the two passes' kernels: tiles of another one are not read
 GAIN = 0.99                 # a candidate must be faster than this fraction of the best so far
 
 
@@ -66,7 +67,7 @@ def _store(db: dict) -> None:
 
 
 def key(W: int, H: int, D: int, gpu: str, order: int = 0, L1: int = 34) -> str:
-    return f"{gpu}|{W}x{H}|D{D}|o{order}|L{L1}"
+    return f"{gpu}|{W}x{H}|D{D}|o{order}|L{L1}|k{KERNELS}"
 
 
 def candidates(W: int, H: int, D: int, max_slice_bytes: int = MAX_SLICE_BYTES) -> list[int]:
@@ -78,27 +79,40 @@ def candidates(W: int, H: int, D: int, max_slice_bytes: int = MAX_SLICE_BYTES) -
     return ok or [min(D, 32)]
 
 
-def first_pass_candidates(n: int, L1: int = 34) -> list[int]:
+def _ranges(n: int, want: int, L1: int, order: int) -> tuple:
+    """(first, others) outputs per block of the first 1-D pass over a line of n
+    positions, as the library cuts it for h_chunk = want."""
+    most = H_MAX_LEN[order]
+    if n <= most and (want == 0 or want >= n):
+        return n, n
+    if order:   # columns: the length as asked for
+        c = min(want or 512, most - 2 * L1)
+        return c, c
+    if not want:
+        return most - L1, most - 2 * L1
+    k = -(-n // min(want, most - 2 * L1))   # rows: ranges of equal length
+    return -(-n // k), -(-n // k)
+
+
+def first_pass_candidates(n: int, L1: int = 34, order: int = 0) -> list[int]:
     """Block lengths of the first 1-D pass over lines of n positions: 0
-    (automatic: whole lines up to 1024, else 512) and lines cut into k
-    near-equal blocks (multiples of 32, at least 64) whose prefix range with
-    its halo fits one block."""
-    out = [0]
+    (automatic) and lines cut into k near-equal blocks (multiples of 32, at
+    least 64) whose range with its halo fits one block, each cut only once."""
+    out, cuts = [0], {_ranges(n, 0, L1, order)}
     for k in range(1, 9):
         c = -(-n // k)
         c = -(-c // 32) * 32
-        if c < 64 or c >= n or c + 2 * L1 > H_MAX_LEN or c in out:
+        if c < 64 or c >= n or c + 2 * L1 > H_MAX_LEN[order] or _ranges(n, c, L1, order) in cuts:
             continue
-        if n > H_MAX_LEN and c == 512:
-            continue   # the automatic choice
+        cuts.add(_ranges(n, c, L1, order))
         out.append(c)
     return out[:6]
 
 
 def second_pass_candidates(n: int, L1: int = 34) -> list[int]:
-    """Block lengths of the second 1-D pass over lines of n positions: 0
-    (automatic) and lines cut into k balanced blocks of at least 32 whose
-    prefix range with its halo fits one block (one value per block count)."""
+    """Run lengths of the second 1-D pass over lines of n positions: 0 (dealt
+    out to the SMs) and lines cut into k balanced runs of at least 32 (one
+    value per run count)."""
     auto = 1 if n <= V_MAX_LEN else -(-n // (V_MAX_LEN - 2 * 40))
     out, counts = [0], {auto}
     for k in range(1, 9):
@@ -175,7 +189,7 @@ def tune_tiles(stereo, left, right, D: int, params=None, reps: int = 5, use_cach
         ms = run(t)
         if ms < best_ms * GAIN or best_ms == float("inf"):
             best, best_ms = t, ms
-    for hc in first_pass_candidates(n1, L1)[1:]:
+    for hc in first_pass_candidates(n1, L1, order)[1:]:
         t = best._replace(h_chunk=hc)
         ms = run(t)
         if ms < best_ms * GAIN:
