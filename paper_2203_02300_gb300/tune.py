@@ -36,6 +36,7 @@ MAX_SLICE_BYTES = 1 << 30   # both views' slices of one pass
 H_MAX_LEN = (640, 1024)     # positions a first-pass block holds with its halo: rows (order 0), columns (1)
 V_MAX_LEN = 512             # longest run tried for the second pass (with its halo)
 KERNELS = 2                 # generation of the two passes' kernels: tiles of another one are not read
+BATCH_SLICES = 4 << 30      # slices of a batch's passes from which its tiles are timed together
 GAIN = 0.99                 # a candidate must be faster than this fraction of the best so far
 
 
@@ -211,7 +212,6 @@ def tune_shape(stereo, W: int, H: int, D: int, device: int = 0, reps: int = 5, u
     """Fastest tile for pairs of shape (W, H, D), timed on a seeded synthetic
     plane scene of that shape when no cached answer exists."""
     import torch
-    from . import scenes
 
     order = int(params.agg_order) if params is not None else 0
     L1 = int(params.arm_l1) if params is not None else 34
@@ -220,20 +220,55 @@ def tune_shape(stereo, W: int, H: int, D: int, device: int = 0, reps: int = 5, u
         hit = lookup(W, H, D, gpu, order, L1)
         if hit is not None:
             return hit
+    L, R = _scene(W, H, D, device)
+    return tune_tiles(stereo, L, R, D, params=params, reps=reps, use_cache=False, max_slice_bytes=max_slice_bytes)
+
+
+def _scene(W: int, H: int, D: int, device: int):
+    import torch
+    from . import scenes
     s = scenes.plane_scene(W, H, D, 6, seed=scenes.seed_for(7, W * 7 + H * 3 + D),
                            drange=(2, max(2, D - 2)), noise_sigma=2.0, texture="mixed")
     dev = torch.device(f"cuda:{device}")
-    L = torch.from_numpy(s.left).to(dev)
-    R = torch.from_numpy(s.right).to(dev)
-    return tune_tiles(stereo, L, R, D, params=params, reps=reps, use_cache=False, max_slice_bytes=max_slice_bytes)
+    return torch.from_numpy(s.left).to(dev), torch.from_numpy(s.right).to(dev)
+
+
+def _batch_gains(stereo, shapes, tiles, device, reps: int, use_cache: bool, params) -> bool:
+    """Whether a large batch is not slower with its pairs' own tiles than with
+    the automatic ones (cached like a shape's tile)."""
+    import torch
+    order = int(params.agg_order) if params is not None else 0
+    L1 = int(params.arm_l1) if params is not None else 34
+    what = ",".join(f"{W}x{H}x{D}:{'/'.join(str(v) for v in t)}" for (W, H, D), t in zip(shapes, tiles))
+    k = f"batch|{torch.cuda.get_device_name(device)}|{what}|o{order}|L{L1}|k{KERNELS}"
+    with _LOCK:
+        hit = _load().get(k) if use_cache else None
+    if hit is None:
+        made = {s: _scene(*s, device) for s in set(shapes)}
+        outs = [torch.empty((H, W), dtype=torch.int16, device=f"cuda:{device}") for W, H, _ in shapes]
+        ms = [_time_call(lambda ts=ts: stereo.match_batch(
+                  [(*made[s], s[2], o, t) for s, o, t in zip(shapes, outs, ts)], params), reps)
+              for ts in ([Tile()] * len(shapes), tiles)]
+        hit = {"automatic_ms": ms[0], "tuned_ms": ms[1]}
+        with _LOCK:
+            db = _load()
+            db[k] = hit
+            _store(db)
+    return hit["tuned_ms"] <= hit["automatic_ms"]
 
 
 def tune_batch(stereo, shapes: Sequence[tuple[int, int, int]], device: int = 0, **kw) -> list[Tile]:
     """Per-pair tiles for a batch of (W, H, D) shapes (each distinct shape
-    tuned once)."""
-    won = {}
-    for sh in shapes:
-        sh = tuple(int(v) for v in sh)
-        if sh not in won:
-            won[sh] = tune_shape(stereo, *sh, device=device, **kw)
-    return [won[tuple(int(v) for v in sh)] for sh in shapes]
+    tuned once, alone).  A batch whose passes together hold more than
+    BATCH_SLICES bytes is also timed as a whole, and keeps the automatic tiles
+    if they are faster there: 32 pairs of 320x240 to 1280x720 take 11.22 ms in
+    the passes of 128 disparities that are best for one pair, 10.96 in the
+    automatic ones of 64."""
+    shapes = [tuple(int(v) for v in sh) for sh in shapes]
+    won = {sh: tune_shape(stereo, *sh, device=device, **kw) for sh in dict.fromkeys(shapes)}
+    tiles = [won[sh] for sh in shapes]
+    slices = sum(8 * W * H * (t.d_chunk or D) for (W, H, D), t in zip(shapes, tiles))
+    if slices > BATCH_SLICES and "max_slice_bytes" not in kw and not _batch_gains(
+            stereo, shapes, tiles, device, kw.get("reps", 5), kw.get("use_cache", True), kw.get("params")):
+        return [Tile()] * len(shapes)
+    return tiles
