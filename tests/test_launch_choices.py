@@ -185,3 +185,56 @@ def test_one_buffer_for_the_left_view_and_the_checked_map(env):
                                                       p(both), p(both), None, p(cost), None, None)
             st.sync_status()
             assert rc == 0 and torch.equal(both, want)
+
+
+def _strips(E, F, layers, slots):
+    """The deal of the strip walk: (whole rounds, strips left, bands per strip that is
+    left; 0: equal shares that run on from strip to strip)."""
+    units = -(-F // 4) * layers
+    rounds, rest = divmod(units, slots)
+    nb = slots // rest if rest else 1
+    return rounds, rest, min(nb, -(-E // 32)) if nb > 1 else 1 if E <= 256 else 0
+
+
+SCHEDULES = {   # E, D, what the deal has to be; F is searched for
+    "run-on shares after whole rounds": (300, 64, lambda r, rest, b: r > 0 and rest > 0 and b == 0),
+    "run-on shares alone": (500, 32, lambda r, rest, b: r == 0 and b == 0),
+    "whole strips after whole rounds": (150, 64, lambda r, rest, b: r > 0 and rest > 0 and b == 1),
+    "bands after whole rounds": (360, 64, lambda r, rest, b: r > 0 and b > 1),
+    "bands alone": (600, 40, lambda r, rest, b: r == 0 and b > 1),
+}
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("what", SCHEDULES)
+def test_every_deal_of_the_strips(env, what, order):
+    torch, binding, st = env
+    E, D, wanted = SCHEDULES[what]
+    nsm = torch.cuda.get_device_properties(0).multi_processor_count
+    slots, layers = 3 * nsm, 2 * -(-D // 32)   # three blocks per SM hold the ring of arm_l1 = 34
+    F = next(F for F in range(64, 1400, 20) if wanted(*_strips(E, F, layers, slots))
+             and (E > 512 or F * layers * -(-E // 32) > 110 * nsm))   # (else by whole lines)
+    W, H = (F, E) if order == 0 else (E, F)
+    left, right, L, R = _pair(torch, W, H, D, F)
+    got = st.match_views(L, R, D, binding.Params.default(agg_order=order))
+    for a, b in zip(got, st.match_views(L, R, D, binding.Params.default(agg_order=order, v_chunk=32))):
+        assert torch.equal(a, b), (what, W, H)
+    rows = (H // 2, H // 2 + 4)
+    ref = O.match(left, right, D, O.Params(agg_order=order), rows=rows)
+    got = [t.cpu().numpy()[slice(*rows)] for t in got]
+    parity.check_disparity(got[1], ref.disp_l, ref.best_l, ref.second_l, f"{what}, order {order}, left")
+    parity.check_cost(got[4], ref.best_r, got[2], ref.disp_r, f"{what}, order {order}, right cost")
+
+
+@pytest.mark.parametrize("W,H", [(333, 251), (65, 37)])   # a thread per pixel; a thread per arm (at most two tiles per SM)
+def test_both_preparations_for_every_window_and_arm_rule(env, W, H):
+    torch, binding, st = env
+    img, _, L, _ = _pair(torch, W, H, 16)
+    tiles = -(-W // 32) * -(-H // 8)
+    assert (tiles > 2 * torch.cuda.get_device_properties(0).multi_processor_count) == (W == 333)
+    for cw, ch, l1, l2, t1, t2 in ((9, 7, 34, 17, 20, 6), (7, 5, 10, 4, 15, 5), (11, 5, 40, 20, 30, 8), (1, 1, 1, 0, 256, 256),
+                                   (9, 7, 34, 17, 0, 6), (9, 7, 34, 2, 255, 0), (3, 3, 8, 8, 1, 1), (5, 13, 40, 0, 60, 60)):
+        over = dict(census_w=cw, census_h=ch, arm_l1=l1, arm_l2=l2, tau1=t1, tau2=t2)
+        p = binding.Params.default(**over)
+        assert (st.census(L, p).cpu().numpy().view(np.uint64) == O.census(img, cw, ch)).all(), over
+        assert (st.arms(L, p).cpu().numpy() == O.arms(img, O.Params(**over))).all(), over
