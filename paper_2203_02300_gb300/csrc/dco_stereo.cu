@@ -927,9 +927,11 @@ __device__ __forceinline__ void hagg_tasks(int ntasks, Find find)
         next += gridDim.x;
         if (threadIdx.x == 0) prepare(next, slot ^ 1);
 
-        // ---- B: segment sums; lane = (column, quad)
+        // ---- B: segment sums; lane = (column, quad).  Whole 32-byte sectors are
+        // written, a dead quad beside a live one too (half a sector is read back from
+        // memory when the line leaves the L2: 1920x1080, D = 10 243 us against 146)
         const int quad = lane & (kHQuads - 1), c0 = 32 / kHQuads * (warp - 1);
-        if (warp > 0 && k.dlo + 4 * quad < k.dend) {
+        if (warp > 0 && k.dlo + 4 * (quad & ~1) < k.dend) {
             constexpr int kStep = (hsm::warps - 1) * 32 / kHQuads;
             const int lead = k.lead, cross = split - lead, m = k.m, col = lane / kHQuads;
             const uint4 *g = reinterpret_cast<const uint4 *>(smem_raw + hsm::g) + quad * hsm::plane + lead + col;
