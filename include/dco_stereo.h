@@ -65,7 +65,7 @@ typedef enum {
     DCO_EBUDGET = 3,  /* the call needs more workspace than the handle's budget */
     DCO_ECUDA = 4,    /* a CUDA runtime call failed */
     DCO_ETIMEOUT = 5, /* a bounded device-side wait gave up */
-    DCO_EDEVICE = 6   /* a kernel reported an internal bound-check failure */
+    DCO_EDEVICE = 6   /* a kernel reported a failed internal check (none does at present) */
 } dco_status;
 
 /*
@@ -140,8 +140,9 @@ void dco_stereo_destroy(dco_stereo *h);
  * needs under params p (0 if the arguments are invalid).  Per pixel: the
  * census and colour of both images, two arm words, the best cost and
  * disparity of both views so far; per pixel and per disparity of one pass: the
- * two horizontal-aggregate slices (4 bytes each).  Never the full
- * W x H x D cost volume.
+ * two horizontal-aggregate slices (4 bytes each).  Automatic passes
+ * (d_chunk 0) hold at most 512 MiB of slices per pair, which may be all D
+ * disparities; d_chunk limits them.
  */
 size_t dco_stereo_workspace_bytes(int W, int H, int D, const dco_params *p);
 
@@ -158,14 +159,16 @@ dco_status dco_stereo_reserve(dco_stereo *h, int W, int H, int D, const dco_para
  *   p->vote_iters rounds of the Eq. 4 parallax optimisation (left view).
  * left, right: device, W*H*3 bytes.  disp_out: device, W*H int16.
  * The disparity range is processed in passes of p->d_chunk disparities
- * (automatic when 0) so the workspace holds slices, never the volume.
+ * (automatic when 0: as wide as 512 MiB of slices allow), so the workspace is
+ * bounded whatever D is.
  * Tile shapes (they change the speed, never the result): the first 1-D
  * pass (rows for agg_order 0, columns for 1) splits each line into ranges
  * of p->h_chunk outputs (0: whole rows up to 640 positions, whole columns up to
  * 1024, else ranges that fill a block; otherwise 32 <= h_chunk, capped at what
  * a block holds with its arm_l1 positions of halo); the second
  * pass walks each line in balanced runs of at most p->v_chunk outputs
- * (0: dealt out evenly to the device; otherwise 32 <= v_chunk).  Each block
+ * (0: dealt out evenly to the device, or whole lines where the launch is small;
+ * otherwise 32 <= v_chunk).  Each block
  * reads arm_l1 positions of halo on both sides.
  * p = NULL uses the defaults.
  */

@@ -15,13 +15,14 @@
 //             segment sum of every pixel -> sh slices
 //     k_vagg  column prefix of the sh slice, the vertical sum over the
 //             up/down arms (Eq. 2) and the minimum over the disparities
-//             (Eq. 3), merged into one key per pixel
+//             (Eq. 3), merged into one key per pixel; k_vcol, a block per
+//             column, in small launches
 //   k_end    keys -> disparities; left-right consistency -> disparity map
 // Every kernel is launched with programmatic stream serialization and waits
 // for its predecessors before its first global access.
-// A lane of the two aggregation kernels holds four consecutive disparities of
-// one column, so that a warp's prefix rows hit distinct banks and the slices
-// are written and read as full 128-byte lines.
+// A lane of k_hagg and k_vagg holds four consecutive disparities (of five
+// columns, of one), so that a warp's prefix rows hit distinct banks and the
+// slices are written and read as whole sectors of 128-byte lines.
 
 #include "kernels.cuh"
 #include "dco_stereo.h"
@@ -1275,8 +1276,8 @@ __device__ __forceinline__ void hvote_body(const HVArgs &a, int bx, int by, int 
 // with the tile inside the totals, were slower (eight passes 1060 us).
 // Against one block per column that held its whole column's prefix, lane =
 // disparity: 1920x1080, D = 256, eight passes 2117 -> 998 us, one pass 1073
-// -> 882 us; 640x480, D = 64, two passes 66.3 -> 50.5 us; the smallest images
-// pay for the longer chain (320x240, D = 32: 12.4 -> 14.2 us).  Walks of one
+// -> 882 us; 640x480, D = 64, two passes 66.3 -> 50.5 us; small launches, which
+// the longer chain of a strip would bind, take k_vcol.  Walks of one
 // warp per strip with no block barrier (six or four warps per SM, by loads or
 // TMA boxes) were latency bound: 55-65 us and 1090-1390 us.
 //
@@ -2107,9 +2108,8 @@ int first_pass_chunk(int n, int L1, int want)
     return c;
 }
 
-// the other aggregation order: k_vcost walks columns (one chunk of rows per
-// block while it fits 32 warps of 32 rows), k_vagg<.., kRow> rows (the scan
-// range along x at most 512 columns, like k_vagg's rows)
+// the other aggregation order: k_vcost takes columns, one chunk of rows per
+// block while it fits 32 warps of 32 rows (k_vagg<.., kRow> then walks rows)
 HGeom vcost_geom(int W, int H, int dc, int L1, int want)
 {
     HGeom g{};
@@ -2398,9 +2398,6 @@ dco_status ensure_tables(dco_stereo *h, const dco_params &p, const Derived &dv, 
 template <class T>
 T *ws_ptr(dco_stereo *h, size_t off) { return reinterpret_cast<T *>(h->ws + off); }
 
-
-// grey/colour packing and census + arms for nimg images (1 or 2); arms of
-// image 0 go to arms0 (the caller's buffer for the arms entry point)
 // ----------------------------------------------------------- batched launches
 constexpr int kBatchMax = 64;   // pairs per launch (kernel parameter space)
 static_assert(sizeof(Batch<VArgs, kBatchMax>) <= 32764, "kernel parameters of a full V batch");
@@ -2592,7 +2589,6 @@ dco_status plan_ws(dco_stereo *h, const dco_params &p, const std::vector<Job> &j
 template <class T>
 T *jptr(dco_stereo *h, const Job &j, size_t off) { return ws_ptr<T>(h, j.base + off); }
 
-// grey/colour packing and census + arms for nimg images of every job
 // images the kernels read from host memory (pinned or registered; over
 // NVLink-C2C on Grace systems)
 constexpr int kPackHostRows = 4;   // rows per k_pack thread for those
@@ -2606,6 +2602,8 @@ bool in_host_memory(const void *p)
     return at.type == cudaMemoryTypeHost;
 }
 
+// grey/colour packing and census + arms for nimg images (1 or 2) of every job;
+// arms of image 0 go to arms0 where it is set (the arms entry point)
 dco_status launch_prep(dco_stereo *h, const dco_params &p, const Derived &dv, const std::vector<Job> &jobs,
                        int nimg, cudaStream_t s)
 {
