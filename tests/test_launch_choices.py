@@ -247,3 +247,12 @@ def test_ragged_disparities_write_whole_sectors(env):
     _, _, L, R = _pair(torch, 1920, 1080, 16)
     few, more = (_us(torch, st, "k_hagg", lambda D=D: st.match(L, R, D)) for D in (10, 16))
     assert few < 1.15 * more, (few, more)
+
+
+def test_a_vote_round_of_a_large_image(env):
+    # 0.94 of the second pass of the vote with 40 registers, 0.85 since
+    torch, binding, st = env
+    _, _, L, R = _pair(torch, 1280, 720, 128)
+    p = binding.Params.default(vote_iters=1)
+    counts, sums = (_us(torch, st, k, lambda: st.match(L, R, 128, p)) for k in ("k_hvote", "k_vvote"))
+    assert counts < 0.92 * sums, (counts, sums)
