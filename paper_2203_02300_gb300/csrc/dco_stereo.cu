@@ -1519,9 +1519,9 @@ __device__ __forceinline__ void vagg_body(const VArgs &a, int blk)
 }
 
 // ------------------------------------------------------------------ k_vcol
-// The same second sum and winner, a block per line: for launches whose strips
-// of k_vagg do not fill the SMs (a walk is then one long chain of steps on an
-// idle chip), and for cost volumes.  Block = one column x of one view (kRow: one
+// The same second sum and winner, a block per line: for short lines, for
+// launches whose strips of k_vagg do not fill the SMs (whole_lines), and for
+// cost volumes.  Block = one column x of one view (kRow: one
 // row y), a chunk of output rows and their reach; a warp per 32 rows.  Per
 // group of 32 disparities:
 //   0. the warp's 32 slice rows (128 bytes each) into its rows of Q by 16-byte
@@ -2701,21 +2701,38 @@ int vagg_slots(const dco_stereo *h, int L1)
     return h->nsm * std::max(1, std::min(kVResident, (int)(kSmShared / (vagg_smem_bytes(L1) + kBlockShared))));
 }
 
-// The second pass of a launch: strips (k_vagg) or whole lines (k_vcol).  Lines where
-// every one fits a block (a v_chunk asks for strips) and their warps, counted once per
-// group, are at most 110 per SM (k_vcol holds 32 at once): the strips' long walks
-// then leave the chip idle.  Strips against lines, us, by that count: 69 (320x240,
-// D = 64) 18.6, 16.3; 105 (400x300, D = 64) 23.3, 20.7; 126 (480x320, D = 64) 24.8, 24.8;
-// 126 (640x480, D = 32) 25.4, 28.7; 152 (480x360, D = 64) 27.4, 31.0.
-bool whole_lines(const dco_stereo *h, const std::vector<Item<VArgs>> &it, bool row_scan)
+// The pairs of a call whose second pass runs by whole lines (k_vcol), the others by
+// strips (k_vagg).  Lines have to fit a block, and a v_chunk asks for strips.  A
+// strip's fill of arm_l1 rows and its last part step weigh on short lines, and its long
+// walk leaves the chip idle in small launches; with many lines per SM, k_vcol's one
+// line per block and barrier is the slower form.  Strips against lines, us, arm_l1 = 34,
+// by warps per SM (a warp per 32 positions of a line and group; k_vcol holds 32 at once):
+//   320x240, D = 64    69   18.6, 16.3      1920x100, D = 64    202   40.4, 29.1
+//   400x300, D = 64   105   23.3, 20.7      960x256, D = 64     202   43.2, 36.8
+//   640x480, D = 32   126   25.4, 28.7      960x256, D = 256    808   127.8, 118.2
+//   480x360, D = 64   152   27.4, 31.0      960x320, D = 256   1010   168, 183
+//   640x400, D = 64   219   44.7, 45.3      64 x 320x240, D = 32  2156  300, 306
+// The length from which strips win falls with arm_l1: 640x256, D = 64, arm_l1 = 40 29.5, 24.8;
+// 17 24.5, 24.8; 3 23.5, 24.6.
+std::vector<char> whole_lines(const dco_stereo *h, const std::vector<Item<VArgs>> &it, int L1, bool row_scan)
 {
-    size_t warps = 0;
-    for (const auto &b : it) {
+    std::vector<char> lines(it.size());
+    size_t all = 0, few = 0;   // warps of the pairs whose lines fit, of those with short lines
+    for (size_t i = 0; i < it.size(); i++) {
+        const auto &b = it[i];
         const int E = row_scan ? b.a.W : b.a.H, F = row_scan ? b.a.H : b.a.W;
-        if (b.gy > 0 || E > kColMax) return false;
-        warps += (size_t)F * b.gz * ((E + kColSeg - 1) / kColSeg);
+        if (b.gy > 0 || E > kColMax) {
+            all = SIZE_MAX / 2;   // (strips are launched in any case)
+            continue;
+        }
+        const size_t warps = (size_t)F * b.gz * ((E + kColSeg - 1) / kColSeg);
+        lines[i] = E <= 200 + 3 * L1 ? 2 : 1;
+        all += warps;
+        if (lines[i] == 2) few += warps;
     }
-    return warps <= 110 * (size_t)h->nsm;
+    const int least = all <= 110 * (size_t)h->nsm ? 1 : few <= 1000 * (size_t)h->nsm ? 2 : 3;
+    for (char &l : lines) l = l >= least;
+    return lines;
 }
 
 // Deals the resident V blocks of a launch (of at most kBatchMax pairs) out to its
@@ -2764,17 +2781,19 @@ std::map<int, std::vector<Item<VArgs>>> deal_lines(const std::vector<Item<VArgs>
 }
 
 template <bool kMax, bool kRow>
-dco_status launch_second(dco_stereo *h, const char *name, std::vector<Item<VArgs>> &it, bool lines, int L1, cudaStream_t s)
+dco_status launch_second(dco_stereo *h, const char *name, const std::vector<Item<VArgs>> &it, const std::vector<char> &lines,
+                         int L1, cudaStream_t s)
 {
-    if (!lines) {
-        deal_v_blocks(h, it, L1, kRow);
-        return launch_items(h, s, name, k_vagg<1, kMax, kRow>, k_vagg<kBatchMax, kMax, kRow>, it, kVThreads,
-                            vagg_smem_bytes(L1));
-    }
-    for (const auto &kv : deal_lines(it, L1, kRow)) {
-        const dco_status st = launch_items(h, s, name, k_vcol<1, kMax, kRow>, k_vcol<kBatchMax, kMax, kRow>, kv.second,
+    std::vector<Item<VArgs>> part[2];
+    for (size_t i = 0; i < it.size(); i++) part[lines[i]].push_back(it[i]);
+    deal_v_blocks(h, part[0], L1, kRow);
+    const dco_status st = launch_items(h, s, name, k_vagg<1, kMax, kRow>, k_vagg<kBatchMax, kMax, kRow>, part[0], kVThreads,
+                                       vagg_smem_bytes(L1));
+    if (st != DCO_OK) return st;
+    for (const auto &kv : deal_lines(part[1], L1, kRow)) {
+        const dco_status ls = launch_items(h, s, name, k_vcol<1, kMax, kRow>, k_vcol<kBatchMax, kMax, kRow>, kv.second,
                                            32 * kv.first, vcol_smem_bytes(kv.first));
-        if (st != DCO_OK) return st;
+        if (ls != DCO_OK) return ls;
     }
     return DCO_OK;
 }
@@ -2786,7 +2805,7 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, std::vector<Job> &jobs,
     std::map<int, std::vector<Item<HArgs>>> cb;   // k_vcost, by warps per block
     std::map<int, size_t> csm;
     std::vector<Item<HArgs>> hb[2];   // k_hagg, by warps per quad
-    std::vector<Item<VArgs>> vb, vvol;
+    std::vector<Item<VArgs>> vb;
     const bool vh = dv.order == 1;   // vertical segment sums first (k_vcost), then rows (kRow)
     for (const Job &j : jobs) {
         if (pass >= j.L.npass) continue;
@@ -2805,25 +2824,23 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, std::vector<Job> &jobs,
         b.a.L1 = dv.L1; b.a.S = dv.S;
         b.gy = j.vchunk > 0 ? j.vchunk : dv.vchunk;
         b.gz = 2 * ng;
-        (j.vol ? vvol : vb).push_back(b);
+        vb.push_back(b);
     }
-    const bool lines = whole_lines(h, vb, vh);
+    std::vector<char> lines = whole_lines(h, vb, dv.L1, vh);
     size_t nv = 0;
     for (Job &j : jobs) {
         if (pass >= j.L.npass) continue;
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
         const int ng = (dc + 31) / 32;
         const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk;
-        const bool by_line = lines || j.vol;
-        const bool init = pass == 0 && !by_line && !(j.L.npass == 1 && ng == 1);
-        if (!j.vol) {   // k_vcol knows the costs with the last pass's keys
-            j.costs_done = lines && pass == j.L.npass - 1;
-            if (j.costs_done) {
-                vb[nv].a.cost[0] = j.cost_l;
-                vb[nv].a.cost[1] = j.cost_r;
-            }
-            nv++;
+        if (j.vol) lines[nv] = 1;   // (k_vcol writes the volumes)
+        const bool init = pass == 0 && !lines[nv] && !(j.L.npass == 1 && ng == 1);
+        j.costs_done = lines[nv] && pass == j.L.npass - 1;
+        if (j.costs_done) {   // k_vcol knows the costs with the last pass's keys
+            vb[nv].a.cost[0] = j.cost_l;
+            vb[nv].a.cost[1] = j.cost_r;
         }
+        nv++;
         Item<HArgs> a{};
         for (int v = 0; v < 2; v++) {
             a.a.cen[v] = jptr<uint2>(h, j, j.L.cen[v]);
@@ -2868,12 +2885,8 @@ dco_status launch_pass(dco_stereo *h, const Derived &dv, std::vector<Job> &jobs,
     if ((st = launch_items(h, s, "k_hagg", k_hagg<1, 2>, k_hagg<kBatchMax, 2>, hb[1], HSmem<2>::warps * 32,
                            HSmem<2>::total, h->yield ? INT_MAX : 2 * h->nsm)) != DCO_OK)
         return st;
-    if (vh) {
-        if ((st = launch_second<false, true>(h, "k_hwta", vb, lines, dv.L1, s)) != DCO_OK) return st;
-        return launch_second<false, true>(h, "k_hwta", vvol, true, dv.L1, s);
-    }
-    if ((st = launch_second<false, false>(h, "k_vagg", vb, lines, dv.L1, s)) != DCO_OK) return st;
-    return launch_second<false, false>(h, "k_vagg", vvol, true, dv.L1, s);
+    return vh ? launch_second<false, true>(h, "k_hwta", vb, lines, dv.L1, s)
+              : launch_second<false, false>(h, "k_vagg", vb, lines, dv.L1, s);
 }
 
 dco_status launch_lr(dco_stereo *h, const std::vector<Item<LrArgs>> &items, cudaStream_t s)
@@ -2906,14 +2919,15 @@ dco_status launch_vote_pass(dco_stereo *h, const Derived &dv, const std::vector<
         b.gz = ng;   // the left view only
         vb.push_back(b);
     }
-    const bool lines = whole_lines(h, vb, false);
+    const std::vector<char> lines = whole_lines(h, vb, dv.L1, false);
+    size_t nv = 0;
     for (const Job &j : jobs) {
         if (!j.vbest || pass >= j.L.npass) continue;
         const int d0 = dv.dmin + pass * j.L.dc, dc = std::min(j.L.dc, dv.dmin + j.D - d0);
         const int ng = (dc + 31) / 32;
         const int hw = j.hchunk > 0 ? j.hchunk : dv.hchunk;
         const HGeom hg = hvote_geom(j.W, j.H, dc, dv.L1, hw);
-        const bool init = pass == 0 && !lines && !(j.L.npass == 1 && ng == 1);
+        const bool init = pass == 0 && !lines[nv++] && !(j.L.npass == 1 && ng == 1);
         hsm[hg.nw] = std::max(hsm[hg.nw], hg.smem);
         Item<HVArgs> a{};
         a.a.disp = j.out;

@@ -196,12 +196,24 @@ def _strips(E, F, layers, slots):
     return rounds, rest, min(nb, -(-E // 32)) if nb > 1 else 1 if E <= 256 else 0
 
 
-SCHEDULES = {   # E, D, what the deal has to be; F is searched for
-    "run-on shares after whole rounds": (300, 64, lambda r, rest, b: r > 0 and rest > 0 and b == 0),
-    "run-on shares alone": (500, 32, lambda r, rest, b: r == 0 and b == 0),
-    "whole strips after whole rounds": (150, 64, lambda r, rest, b: r > 0 and rest > 0 and b == 1),
-    "bands after whole rounds": (360, 64, lambda r, rest, b: r > 0 and b > 1),
-    "bands alone": (600, 40, lambda r, rest, b: r == 0 and b > 1),
+def _lines(E, F, layers, L1, nsm):
+    """Whether the second pass of one pair takes whole lines."""
+    warps = F * layers * -(-E // 32)
+    return E <= 512 and (warps <= 110 * nsm or E <= 200 + 3 * L1 and warps <= 1000 * nsm)
+
+
+def _slots(L1, nsm):
+    """Resident blocks of the strip walk: by its ring in shared memory, at most four."""
+    ring = (-(-(2 * L1 + 1) // 8) * 8 + 32) * 512
+    return nsm * min(4, (228 << 10) // (ring + 6 * 512 + 4 * (8 * 128 + 128) + 1024))
+
+
+SCHEDULES = {   # E, D, arm_l1, what the deal has to be; F is searched for
+    "run-on shares after whole rounds": (310, 64, 34, lambda r, rest, b: r > 0 and rest > 0 and b == 0),
+    "run-on shares alone": (500, 32, 34, lambda r, rest, b: r == 0 and b == 0),
+    "whole strips after whole rounds": (240, 64, 3, lambda r, rest, b: r > 0 and rest > 0 and b == 1),
+    "bands after whole rounds": (360, 64, 34, lambda r, rest, b: r > 0 and b > 1),
+    "bands alone": (600, 40, 34, lambda r, rest, b: r == 0 and b > 1),
 }
 
 
@@ -209,18 +221,19 @@ SCHEDULES = {   # E, D, what the deal has to be; F is searched for
 @pytest.mark.parametrize("what", SCHEDULES)
 def test_every_deal_of_the_strips(env, what, order):
     torch, binding, st = env
-    E, D, wanted = SCHEDULES[what]
+    E, D, L1, wanted = SCHEDULES[what]
     nsm = torch.cuda.get_device_properties(0).multi_processor_count
-    slots, layers = 3 * nsm, 2 * -(-D // 32)   # three blocks per SM hold the ring of arm_l1 = 34
-    F = next(F for F in range(64, 1400, 20) if wanted(*_strips(E, F, layers, slots))
-             and (E > 512 or F * layers * -(-E // 32) > 110 * nsm))   # (else by whole lines)
+    layers = 2 * -(-D // 32)
+    F = next(F for F in range(64, 1400, 20)
+             if wanted(*_strips(E, F, layers, _slots(L1, nsm))) and not _lines(E, F, layers, L1, nsm))
     W, H = (F, E) if order == 0 else (E, F)
     left, right, L, R = _pair(torch, W, H, D, F)
-    got = st.match_views(L, R, D, binding.Params.default(agg_order=order))
-    for a, b in zip(got, st.match_views(L, R, D, binding.Params.default(agg_order=order, v_chunk=32))):
+    over = dict(agg_order=order, arm_l1=L1, arm_l2=L1 // 2)
+    got = st.match_views(L, R, D, binding.Params.default(**over))
+    for a, b in zip(got, st.match_views(L, R, D, binding.Params.default(v_chunk=32, **over))):
         assert torch.equal(a, b), (what, W, H)
     rows = (H // 2, H // 2 + 4)
-    ref = O.match(left, right, D, O.Params(agg_order=order), rows=rows)
+    ref = O.match(left, right, D, O.Params(**over), rows=rows)
     got = [t.cpu().numpy()[slice(*rows)] for t in got]
     parity.check_disparity(got[1], ref.disp_l, ref.best_l, ref.second_l, f"{what}, order {order}, left")
     parity.check_cost(got[4], ref.best_r, got[2], ref.disp_r, f"{what}, order {order}, right cost")
@@ -247,6 +260,30 @@ def test_ragged_disparities_write_whole_sectors(env):
     _, _, L, R = _pair(torch, 1920, 1080, 16)
     few, more = (_us(torch, st, "k_hagg", lambda D=D: st.match(L, R, D)) for D in (10, 16))
     assert few < 1.15 * more, (few, more)
+
+
+@pytest.mark.parametrize("W,H,order", [(1920, 100, 0), (160, 1080, 1)])
+def test_short_lines_are_not_walked_in_strips(env, W, H, order):
+    # strips (as v_chunk asks) against the automatic choice: the same time when that was
+    # strips too, 0.72 and 0.77 of it since
+    torch, binding, st = env
+    _, _, L, R = _pair(torch, W, H, 64)
+    auto, strips = (_us(torch, st, "k_hwta" if order else "k_vagg", lambda p=binding.Params.default(agg_order=order, v_chunk=v):
+                        st.match(L, R, 64, p), 20) for v in (0, 16384))
+    assert auto < 0.88 * strips, (auto, strips)
+
+
+def test_a_batch_of_short_and_long_pairs(env):
+    # strips and lines in one call, with and without passes and votes: each pair as alone
+    torch, binding, st = env
+    shapes = [(640, 480, 64), (200, 150, 40), (333, 211, 50), (96, 600, 20), (1000, 120, 33), (64, 64, 64)] * 2
+    made = [_pair(torch, *s, seed=k)[2:] for k, s in enumerate(shapes)]
+    outs = [torch.empty((H, W), dtype=torch.int16, device="cuda") for W, H, _ in shapes]
+    for over in ({}, {"vote_iters": 2}, {"d_chunk": 32}, {"agg_order": 1}):
+        p = binding.Params.default(**over)
+        st.match_batch([(*m, s[2], o) for m, s, o in zip(made, shapes, outs)], p)
+        for m, s, o in zip(made, shapes, outs):
+            assert torch.equal(o, st.match(*m, s[2], p)), (over, s)
 
 
 def test_a_vote_round_of_a_large_image(env):
