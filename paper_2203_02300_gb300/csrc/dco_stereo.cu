@@ -675,12 +675,12 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t n,
 //   B. every output column: S_H = G(end) - G(start), eight lanes (quads) per
 //      column, a 128-byte line of the slice per column; the planes' stride
 //      puts the eight quads of a column on distinct banks whatever the arms.
-// Bound by the shared-memory data path (15 M wavefronts at 640x480, D = 64, 87 %
+// Bound by the shared-memory data path (15 M wavefronts at 640x480, D = 64, 88 %
 // of the L1 throughput, a third of them the table gathers of Eq. 1).  Against
 // one block per task with a disparity pair per lane and sixteen-column
-// segments: 45 M instead of 52 M instructions; 640x480, D = 64, one pass 70 -> 66
-// us (the default was two passes: 82), 1280x720, D = 128 481 -> 423 us,
-// 1920x1080, D = 256 1960 -> 1875 us.  Blocks of sixteen warps alone left half of them
+// segments: 46 M instead of 52 M instructions; 640x480, D = 64, one pass 70 -> 66
+// us (in two passes 82), 1280x720, D = 128 481 -> 416 us, 1920x1080, D = 256 in
+// eight passes 1960 -> 1817 us.  Blocks of sixteen warps alone left half of them
 // idle on rows of up to 160 columns and an SM with two blocks in the same phase on
 // rows of up to 320: 64 pairs of 160x120, D = 32 206 us against 140 with eight warps (one
 // block per row and group before: 121), of 320x240 574 against 465 (502), 256x192,
@@ -1037,6 +1037,11 @@ __device__ __forceinline__ void hagg_tail(const uint32_t *P, uint32_t *T, const 
 // phases of a horizontal pass along the column: local prefixes over warp
 // segments of 32 rows, segment offsets, segment sums (hagg_tail, with the
 // up / down arms), written to the same slice layout.
+// Bound by the L1 data path and its latency (76 % of its throughput; fewer
+// instructions per row changed nothing), so by the warps that fit: with the
+// plane entry as one 32-bit index the loop takes 38 registers (44 with two
+// pointers), and two blocks of 720 rows share an SM: 1280x720, D = 128 974 -> 752
+// us, 320x240, D = 32 22.7 -> 20.7, 333x211, D = 50 27.5 -> 29.3.
 struct CSmem {
     int ref, arm, p, t, total;
     __host__ __device__ CSmem(int len, int chunk, int nw)
