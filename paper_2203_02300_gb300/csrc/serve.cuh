@@ -374,8 +374,19 @@ dco_status dco_server_create(dco_server **out, int device, const dco_stream_desc
             cudaStreamCreateWithPriority(&ln.stream_hi, cudaStreamNonBlocking, greatest) != cudaSuccess)
             st = DCO_ECUDA;
     }
-    // warm every lane up with the largest batch admission allows, so its
-    // workspace never grows (a synchronising reallocation) while serving
+    // every lane holds the largest workspace that admission allows, so that it
+    // never grows while serving (a synchronising reallocation).  A lane that cannot
+    // have it grows when it has to.
+    if (st == DCO_OK) {
+        std::vector<size_t> slots;
+        for (int i = 0; i < nstreams; i++) slots.insert(slots.end(), (size_t)slots_per_stream, s->ws[i]);
+        std::sort(slots.rbegin(), slots.rend());
+        size_t most = 0;
+        for (size_t k = 0; k < slots.size() && k < (size_t)max_batch; k++) most += slots[k];
+        for (auto &ln : s->lanes)
+            if (ensure_ws(ln.h, std::min(most, s->lane_budget)) != DCO_OK) break;
+    }
+    // and is warmed up: tables, shared-memory opt-ins, the batch kernels
     if (st == DCO_OK) {
         std::vector<dco_pair_desc> warm;
         size_t used = 0;

@@ -103,13 +103,15 @@ class Server:
         self.slots = [[_Slot(torch, self.dev, W, H) for _ in range(slots_per_stream)]
                       for (W, H, _) in self.shapes]
         self.lanes = [_Lane(torch, self.dev, device, self.lane_budget) for _ in range(lanes)]
-        # warm every lane up with the largest batch admission allows, so its
-        # workspace never grows (a synchronising reallocation) while serving
+        # warm every lane up with a batch as large as admission allows (the largest
+        # frames first, of every stream in turn), so that its workspace does not
+        # grow (a synchronising reallocation) while serving
         warm, used = [], 0
-        for s, (W, H, D) in enumerate(self.shapes):
-            for sl in self.slots[s]:
+        for k in range(slots_per_stream):
+            for s in sorted(range(len(self.shapes)), key=lambda s: -ws[s]):
+                sl = self.slots[s][k]
                 if used + ws[s] <= self.lane_budget and len(warm) < max_batch:
-                    warm.append((sl.left, sl.right, D, sl.out, self.tiles[s]))
+                    warm.append((sl.left, sl.right, self.shapes[s][2], sl.out, self.tiles[s]))
                     used += ws[s]
         for sl_list in self.slots:
             for sl in sl_list:
