@@ -2060,10 +2060,10 @@ bool dims_valid(int W, int H, int D, int dmin = 0)
 // (about the L2) is what the serving lanes admit frames by, and the fallback
 // where the device cannot allocate the wide one.
 constexpr size_t kSlicesWide = 512u << 20, kSlicesNarrow = 96u << 20;
-// all pairs of a call together: from 33 pairs on, the wide cap of each is its
-// part of this (at least the narrow one), so that a batch's workspace stays
-// bounded by what narrow passes or 16 GiB of slices take
-constexpr size_t kSlicesCall = size_t(16) << 30;
+// all pairs of a call together: from 65 pairs on (more than one launch), the wide cap
+// of each is its part of this (at least the narrow one), so that a batch's
+// workspace stays bounded by what narrow passes or 32 GiB of slices take
+constexpr size_t kSlicesCall = size_t(32) << 30;
 size_t wide_cap(size_t pairs) { return std::max(kSlicesNarrow, std::min(kSlicesWide, kSlicesCall / std::max<size_t>(1, pairs))); }
 int auto_width(int W, int H, int D, size_t cap)
 {

@@ -82,16 +82,16 @@ def test_reserve_and_batches_take_the_narrow_plan(env):
 
 
 def test_a_large_batch_bounds_its_slices(env):
-    # from 33 pairs on the pairs share 16 GiB of slices
+    # from 65 pairs on the pairs share 32 GiB of slices
     torch, binding, left, right, want = env
-    w, h, n = 640, 360, 200   # alone: one pass of 256 (472 MB); among 200: narrow passes of 32
+    w, h, n = 640, 360, 200   # alone: one pass of 256 (472 MB); among 200: passes of 64
     s = scenes.plane_scene(w, h, 256, 6, seed=scenes.seed_for(8, 78), drange=(2, 250), noise_sigma=2.0, texture="mixed")
     a, b = torch.from_numpy(s.left).cuda(), torch.from_numpy(s.right).cuda()
     outs = [torch.empty((h, w), dtype=torch.int16, device="cuda") for _ in range(n)]
     with binding.Stereo(0) as st:
         st.match_batch([(a, b, 256, o) for o in outs])
         torch.cuda.synchronize()
-        assert st.workspace_allocated() < (20 << 30)
+        assert st.workspace_allocated() < (36 << 30)
         alone = st.match(a, b, 256)
         for o in outs:
             assert torch.equal(o, alone)
