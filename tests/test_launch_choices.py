@@ -265,7 +265,7 @@ def test_ragged_disparities_write_whole_sectors(env):
 @pytest.mark.parametrize("W,H,order", [(1920, 100, 0), (160, 1080, 1)])
 def test_short_lines_are_not_walked_in_strips(env, W, H, order):
     # strips (as v_chunk asks) against the automatic choice: the same time when that was
-    # strips too, 0.72 and 0.77 of it since
+    # strips too, 0.68 and 0.75 of it since
     torch, binding, st = env
     _, _, L, R = _pair(torch, W, H, 64)
     auto, strips = (_us(torch, st, "k_hwta" if order else "k_vagg", lambda p=binding.Params.default(agg_order=order, v_chunk=v):
@@ -287,7 +287,7 @@ def test_a_batch_of_short_and_long_pairs(env):
 
 
 def test_a_vote_round_of_a_large_image(env):
-    # 0.94 of the second pass of the vote with 40 registers, 0.85 since
+    # 0.93 of the second pass of the vote with 40 registers, 0.82 since
     torch, binding, st = env
     _, _, L, R = _pair(torch, 1280, 720, 128)
     p = binding.Params.default(vote_iters=1)
